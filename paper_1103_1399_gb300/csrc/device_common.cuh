@@ -58,6 +58,75 @@ __device__ __forceinline__ void reg_rot(float2 (&v)[32], const float2 (&tab)[6])
   reg_wht<0, B>(v);
 }
 
+// ---- one-qubit rotations in the gauge i^popcount ------------------------------
+// exp(-i theta H_B) = prod_i e^(-ih) (cos h + i sin h sigma^x_i), h = theta / 2
+// (Sec. 2.1).  With phi_x = i^popcount(x) psi_x (an exact swap and negation of
+// components) every factor is real: (u, w) <- (a u + b w, a w - b u) on the pair
+// of amplitudes whose index differs in the bit (u: bit clear), so it acts on
+// (re, im) as a packed pair.  Rows of the tangent form (a = 1, b = tan h, kept for
+// |tan h| <= 1) need one packed FMA per amplitude and qubit, against the two
+// additions and a fifth of a complex multiply of the Walsh-Hadamard sandwich,
+// and round once; the factor (a^2 + b^2)^(-n/2) e^(-inh) of the rounded a, b is
+// part of the phase row that ends the step (p_entry), so rounding a and b
+// changes the angle by less than 1e-7 of itself and the norm not at all.
+// Other angles use a = cos h, b = sin h.
+struct RotCoef {
+  unsigned long long a, b, nb;
+  bool tangent;
+};
+__device__ __forceinline__ RotCoef rot_coef(float2 ab) {
+  RotCoef c;
+  c.a = f2_bits(make_float2(ab.x, ab.x));
+  c.b = f2_bits(make_float2(ab.y, ab.y));
+  c.nb = f2_bits(make_float2(-ab.y, -ab.y));
+  c.tangent = ab.x == 1.0f;
+  return c;
+}
+__device__ __forceinline__ float2 fma2(unsigned long long k, float2 x, float2 y) {
+  unsigned long long d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(k), "l"(f2_bits(x)), "l"(f2_bits(y)));
+  return bits_f2(d);
+}
+__device__ __forceinline__ float2 mul2(unsigned long long k, float2 x) {
+  unsigned long long d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(k), "l"(f2_bits(x)));
+  return bits_f2(d);
+}
+// Register-index bits [B0, B1) of an N-entry register tile.
+template <int B0, int B1, int N>
+__device__ __forceinline__ void reg_turn(float2 (&v)[N], const RotCoef& c) {
+  if (c.tangent) {
+#pragma unroll
+    for (int b = B0; b < B1; ++b) {
+#pragma unroll
+      for (int r = 0; r < N; ++r) {
+        if (!(r & (1 << b))) {
+          const float2 u = v[r], w = v[r | (1 << b)];
+          v[r] = fma2(c.b, w, u);
+          v[r | (1 << b)] = fma2(c.nb, u, w);
+        }
+      }
+    }
+  } else {
+#pragma unroll
+    for (int b = B0; b < B1; ++b) {
+#pragma unroll
+      for (int r = 0; r < N; ++r) {
+        if (!(r & (1 << b))) {
+          const float2 u = v[r], w = v[r | (1 << b)];
+          v[r] = fma2(c.b, w, mul2(c.a, u));
+          v[r | (1 << b)] = fma2(c.nb, u, mul2(c.a, w));
+        }
+      }
+    }
+  }
+}
+// v <- i^k v (exact).
+__device__ __forceinline__ float2 times_i(float2 v, int k) {
+  const float2 s = (k & 1) ? make_float2(-v.y, v.x) : v;
+  return (k & 2) ? make_float2(-s.x, -s.y) : s;
+}
+
 // Runtime-bounded variant (bits [b0, b1) with b0, b1 in [0, 5]).
 __device__ __forceinline__ void reg_wht_rt(float2 (&v)[32], int b0, int b1) {
 #pragma unroll
@@ -117,24 +186,20 @@ __device__ __forceinline__ void csa(unsigned& h, unsigned& l, unsigned b, unsign
   h = (a & b) | (a & c) | (b & c);
 }
 
-// For every register index r (0..31) count the active entries whose lane_pat
-// has `lanebit` set and whose reg_pat has bit r set.  Result: pl[b] holds bit b
-// of each of the 32 counts (bit r of pl[b] belongs to register r).  Harley-Seal
-// carry-save tree over 16 entries at a time, then a ripple add of the weight-16
-// carries.  Counts up to 1023 are exact.
-__device__ __forceinline__ void count_active(const uint2* __restrict__ act, int npad, unsigned lanebit,
-                                             unsigned (&pl)[kPlanes]) {
+// Sum of `count` (a multiple of 16) 32-bit words get(0), get(1), ... bit by bit:
+// pl[b] holds bit b of each of the 32 sums.  Harley-Seal carry-save tree over
+// 16 words at a time, then a ripple add of the weight-16 carries.  Sums up to
+// 1023 are exact.
+template <class Get>
+__device__ __forceinline__ void count_words(int count, Get&& get, unsigned (&pl)[kPlanes]) {
   unsigned ones = 0, twos = 0, fours = 0, eights = 0;
   unsigned hi[kPlanes - 4];
 #pragma unroll
   for (int k = 0; k < kPlanes - 4; ++k) hi[k] = 0;
-  for (int i = 0; i < npad; i += 16) {
+  for (int i = 0; i < count; i += 16) {
     unsigned d[16];
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const uint2 e = act[i + j];
-      d[j] = (e.y & lanebit) ? e.x : 0u;
-    }
+    for (int j = 0; j < 16; ++j) d[j] = get(i + j);
     unsigned twosA, twosB, foursA, foursB, eightsA, eightsB, sixteens;
     csa(twosA, ones, d[0], d[1]);
     csa(twosB, ones, d[2], d[3]);
@@ -165,6 +230,20 @@ __device__ __forceinline__ void count_active(const uint2* __restrict__ act, int 
   pl[3] = eights;
 #pragma unroll
   for (int k = 0; k < kPlanes - 4; ++k) pl[4 + k] = hi[k];
+}
+
+// For every register index r (0..31) count the active entries whose lane_pat
+// has `lanebit` set and whose reg_pat has bit r set.  Result: pl[b] holds bit b
+// of each of the 32 counts (bit r of pl[b] belongs to register r).
+__device__ __forceinline__ void count_active(const uint2* __restrict__ act, int npad, unsigned lanebit,
+                                             unsigned (&pl)[kPlanes]) {
+  count_words(
+      npad,
+      [&](int i) {
+        const uint2 e = act[i];
+        return (e.y & lanebit) ? e.x : 0u;
+      },
+      pl);
 }
 
 // Stored per-tile counts (layout Y: registers hold bits 0..4).  E(x) never

@@ -307,7 +307,7 @@ qaa_status evolve_impl(qaa_ctx* h, void* psi, double dt, long long K, long long 
     const long long c1 = std::min(k1, c0 + chunk);
     QAA_CK(timed(h, QAA_K_TABLES, [&] {
       return qaa::launch_tables(lc, ptab, btab, h->n, h->m, dt, s_dev, K, k0, k1, c0, c1,
-                                h->n > qaa::kOnchipMaxBits && h->plan.wht_kind == qaa::kRotationForm, dt_dev);
+                                qaa::row_form(h->plan), dt_dev);
     }));
     if (h->n <= qaa::kOnchipMaxBits) {
       QAA_CK(timed(h, QAA_K_ONCHIP, [&] {

@@ -73,6 +73,11 @@ void clear_tuned_plans();
 void build_passes(const PassPlan& plan, long long k0, long long k1, long long c0, long long c1,
                   std::vector<Pass>& out);
 
+// The phase rows (RowForm) this plan's kernels read.
+inline int row_form(const PassPlan& plan) {
+  return plan.onchip ? kRowsTurn : (plan.wht_kind == kRotationForm ? kRowsBlock : kRowsWbw);
+}
+
 std::string describe_plan(const PassPlan& plan);
 
 // Launch one pass with the kernel family the plan selects.  fold: kFoldBytes

@@ -1,242 +1,468 @@
-// Small-instance evolver (n <= 14): the whole complex64 state (<= 128 KiB) and
-// its energies E(x) stay in one CTA's shared memory for every step of a run, so
-// HBM is touched once on entry and once on exit.
+// Small-instance evolver (n <= 14): the whole complex64 state stays on chip for
+// every step of a run, so HBM is touched once on entry and once on exit.
 //
-// Same Strang step as the streaming path (Eq. (1) frozen at s_k; H_B applied as
-// a popcount phase between two Walsh-Hadamard transforms, Sec. 2.1; H_P the
-// violated-clause count, Sec. 4.3), with half phases of adjacent steps merged.
-// The transform runs in "rounds" over groups of up to 5 index bits: each thread
-// pulls a column of 2^w amplitudes into registers, applies the butterflies (and
-// any phase due in that round) and writes it back.
-//   step: [group 0: W] [groups 1..G-2: W] [group G-1: W B W] [groups G-2..1: W]
-//         [group 0: W P(next) W(next step)]
-// E(x) is evaluated once per launch from the clause bit masks (bit exact) and
-// kept as uint16 in shared memory.
+// Same Strang step as the streaming path (Eq. (1) frozen at s_k; H_P the
+// violated-clause count, Sec. 4.3), with half phases of adjacent steps merged;
+// exp(-i theta H_B) is applied as its n one-qubit factors in the gauge
+// i^popcount (RotCoef): one packed FMA per amplitude and qubit.
+//
+// * n <= 8: one warp, the state in its registers (x = lane + 32 r): lane bits by
+//   shuffles, no barrier and no shared-memory transpose in a step.
+// * 9 <= n <= 14: one CTA of 2^(n-R) threads with 2^R amplitudes each.  A
+//   thread's registers hold a window of R index bits: TOP [n-R, n), BOT [0, R) or
+//   MID [R, 2R).  A step turns one window, moves the state through shared memory
+//   to the next and ends with P: TOP BOT MID P, the next step MID BOT TOP P, so
+//   two transposes per step.  E(x) of both P layouts stays in registers (16 bits
+//   per amplitude, times 8: the byte offset in the phase row).
+// Bound by shared memory (two transposes and the P row lookups) and, below
+// n = 12, by the latency of a step's two barriers.  The earlier form (W B W in
+// columns of 32 amplitudes, 24 butterfly levels, four shared-memory rounds and
+// P rows from global memory) had 2^(n-5) threads busy.  Measured, us per step of
+// a 400-step run, before and after: n = 6 1.76 / 0.44, n = 9 1.83 / 0.61, n = 12
+// 3.23 / 1.39, n = 14 8.60 / 4.79.
+// Phase rows come through a ring of cp.async copies issued kRing - 1 steps ahead.
 #include "device_common.cuh"
 
 namespace qaa {
 
-constexpr int kOnchipThreads = 512;
+namespace {
 
-// Shared slot of amplitude x: rows of 32 padded to 33 (bank-conflict-free for
-// columns along any 5-bit group, base + immediate addressing within a column).
-__device__ __forceinline__ int oswz(int x) { return x + (x >> 5); }
+constexpr int kBatchThreads = 512;
 
-enum : unsigned { kPreP = 1u, kW1 = 2u, kMidB = 4u, kW2 = 8u, kPostP = 16u, kW3 = 32u, kNorm = 64u };
-
-template <int W>
-__device__ __forceinline__ void col_wht(float2 (&v)[1 << W]) {
-#pragma unroll
-  for (int b = 0; b < W; ++b) {
-#pragma unroll
-    for (int r = 0; r < (1 << W); ++r) {
-      if (!(r & (1 << b))) butterfly(v[r], v[r | (1 << b)]);
-    }
-  }
+__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
+               "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// kNorm: add |psi|^2 of the round's outputs to *nacc (FP32: at most one column
-// per thread at n <= 14); cs = c - 1 scales the popcount phase (the norm fold of the
-// previous step).
-template <int W>
-__device__ void onchip_round(float2* __restrict__ s_psi, const uint16_t* __restrict__ s_e, int n, int b0,
-                             unsigned flags, const float2* __restrict__ prow_a, const float2* __restrict__ brow,
-                             const float2* __restrict__ prow_b, float cs, float* nacc) {
-  const int ncols = (1 << n) >> W;
-  const int lo_mask = (1 << b0) - 1;
-  for (int col = threadIdx.x; col < ncols; col += blockDim.x) {
-    const int xb = (col & lo_mask) | ((col >> b0) << (b0 + W));
-    // slot(xb + (r << b0)) = slot(xb) + r * rstep: xb has no bits in [b0, b0+W)
-    // and, for b0 = 0, is a multiple of 32 (W = 5) or the whole index is < 32.
-    const int sx = oswz(xb);
-    const int rstep = (1 << b0) + (b0 >= 5 ? (1 << (b0 - 5)) : 0);
-    float2 v[1 << W];
-#pragma unroll
-    for (int r = 0; r < (1 << W); ++r) v[r] = s_psi[sx + r * rstep];
-    if (flags & kPreP) {
-#pragma unroll
-      for (int r = 0; r < (1 << W); ++r) v[r] = cmul(v[r], prow_a[s_e[sx + r * rstep]]);
-    }
-    if (flags & kW1) col_wht<W>(v);
-    if (flags & kMidB) {
-      const int pc = __popc(xb);
-#pragma unroll
-      for (int r = 0; r < (1 << W); ++r) v[r] = cmul(v[r], brow[pc + __popc(r)]);
-      if (cs != 0.0f) {
-#pragma unroll
-        for (int r = 0; r < (1 << W); ++r) v[r] = fold_apply(v[r], cs);
-      }
-    }
-    if (flags & kW2) col_wht<W>(v);
-    if (flags & kPostP) {
-#pragma unroll
-      for (int r = 0; r < (1 << W); ++r) v[r] = cmul(v[r], prow_b[s_e[sx + r * rstep]]);
-    }
-    if (flags & kW3) col_wht<W>(v);
-#pragma unroll
-    for (int r = 0; r < (1 << W); ++r) s_psi[sx + r * rstep] = v[r];
-    if (flags & kNorm) {
-      // pairwise tree over the column (at most 5 levels of FP32 rounding)
-      float p[1 << W];
-#pragma unroll
-      for (int r = 0; r < (1 << W); ++r) p[r] = fmaf(v[r].x, v[r].x, v[r].y * v[r].y);
-#pragma unroll
-      for (int h = (1 << W) >> 1; h > 0; h >>= 1) {
-#pragma unroll
-        for (int r = 0; r < h; ++r) p[r] += p[r + h];
-      }
-      *nacc += p[0];
-    }
-  }
+// Barrier over the NT threads that run an instance (the others of a batch
+// CTA have left).
+template <int NT>
+__device__ __forceinline__ void team_sync() {
+  if constexpr (NT <= 32)
+    __syncwarp();
+  else
+    asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");
 }
 
-__device__ __forceinline__ void round_dispatch(float2* s_psi, const uint16_t* s_e, int n, int g, unsigned flags,
-                                               const float2* pa, const float2* br, const float2* pb, float cs,
-                                               float* nacc) {
-  const int b0 = 5 * g;
-  const int w = (n - b0) < 5 ? (n - b0) : 5;
-  switch (w) {
-    case 1: onchip_round<1>(s_psi, s_e, n, b0, flags, pa, br, pb, cs, nacc); break;
-    case 2: onchip_round<2>(s_psi, s_e, n, b0, flags, pa, br, pb, cs, nacc); break;
-    case 3: onchip_round<3>(s_psi, s_e, n, b0, flags, pa, br, pb, cs, nacc); break;
-    case 4: onchip_round<4>(s_psi, s_e, n, b0, flags, pa, br, pb, cs, nacc); break;
-    default: onchip_round<5>(s_psi, s_e, n, b0, flags, pa, br, pb, cs, nacc); break;
-  }
-  __syncthreads();
-}
-
-// The norm fold of a step (as in the streaming low passes): the block's sum of
-// one FP32 value per thread -- a fixed FP32 shuffle tree per warp, the warps'
-// sums added as double-floats by thread 0 -- returned as a double-float pair
-// when ref is null, else the correction c - 1 = fold_scale(ref, sum) in .hi.  Every
-// thread gets the result.  Contains __syncthreads: every thread calls it.
-__device__ DFloat onchip_fold(float v, const DFloat* ref) {
-  __shared__ float s_w[kOnchipThreads / 32];
-  __shared__ DFloat s_out;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0) s_w[warp] = v;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    DFloat t{0.f, 0.f};
-    for (int w = 0; w < static_cast<int>(blockDim.x >> 5); ++w) t = df_add1(t, s_w[w]);
-    s_out = ref ? DFloat{fold_scale(*ref, t), 0.f} : t;
-  }
-  __syncthreads();
-  const DFloat out = s_out;
-  __syncthreads();  // s_out is written again by the next call
-  return out;
-}
-
-// Shared layout: [psi slots | E slots (uint16) | clauses], every region starting
-// on a 16-byte boundary (the clause records are read with 128-bit loads).
-struct OnchipLayout {
-  size_t slots, off_e, off_cl, total;
-  __host__ __device__ explicit OnchipLayout(int n, int m) {
-    const size_t N = static_cast<size_t>(1) << n;
-    slots = N + (N >> 5) + 1;
-    off_e = (slots * 8u + 15u) & ~static_cast<size_t>(15);
-    off_cl = off_e + ((slots * 2u + 15u) & ~static_cast<size_t>(15));
-    total = off_cl + 16u * static_cast<size_t>(m);
-  }
+struct RunArgs {
+  float2* psi;
+  const ClauseMV* cl;
+  const float2* ptab;
+  const float2* btab;
+  int n, m, nsteps;
+  bool first_p, init;
+  float init_val;
 };
 
-size_t onchip_smem_bytes(int n, int m) { return OnchipLayout(n, m).total; }
-
-// One whole run (or chunk of a run) of one instance, by one CTA.
-__device__ void onchip_run(float2* __restrict__ psi, int n, int m, const ClauseMV* __restrict__ cl,
-                           const float2* __restrict__ ptab, const float2* __restrict__ btab, int nsteps, int first_p,
-                           unsigned char* smem, bool init_uniform = false, float init_val = 0.0f) {
-  const int N = 1 << n;
-  const OnchipLayout L(n, m);
-  float2* s_psi = reinterpret_cast<float2*>(smem);
-  uint16_t* s_e = reinterpret_cast<uint16_t*>(smem + L.off_e);
-  ClauseMV* s_cl = reinterpret_cast<ClauseMV*>(smem + L.off_cl);
-  for (int i = threadIdx.x; i < m; i += blockDim.x) s_cl[i] = cl[i];
-  // the uniform start state 2^(-n/2) (Sec. 2.1, value rounded on the host as
-  // for qaa_init_uniform), or the caller's state
-  const float2 u = make_float2(init_val, 0.0f);
-  float racc = 0.0f;  // |psi|^2 of the input: the norm every step is folded back to
-  for (int x = threadIdx.x; x < N; x += blockDim.x) {
-    const float2 a = init_uniform ? u : psi[x];
-    s_psi[oswz(x)] = a;
-    racc += fmaf(a.x, a.x, a.y * a.y);  // at most 32 terms per thread (N <= 2^14)
+// Phase rows of step j (the P row that ends it, its rotation) into ring slot j.
+// One commit group per call, empty beyond the last step.
+template <int NT, int RING>
+__device__ __forceinline__ void fetch_rows(const RunArgs& A, float2* s_p, float2* s_ab, int j, int tid) {
+  if (j < A.nsteps) {
+    const int mp1 = A.m + 1;
+    float2* dst = s_p + (j % RING) * mp1;
+    const float2* src = A.ptab + static_cast<size_t>(j + 1) * mp1;
+    for (int i = tid; i < mp1; i += NT) cp_async8(dst + i, src + i);
+    if (tid == 0) cp_async8(s_ab + j % RING, A.btab + static_cast<size_t>(j) * (A.n + 1));
   }
-  const DFloat nref = onchip_fold(racc, nullptr);
-  for (int x = threadIdx.x; x < N; x += blockDim.x) {
-    int e = 0;
-    for (int c = 0; c < m; ++c) {
-      const unsigned mk = static_cast<unsigned>(s_cl[c].mask), vl = static_cast<unsigned>(s_cl[c].viol);
-      e += (static_cast<unsigned>(x) & mk) == vl;
+  cp_async_commit();
+}
+
+// v <- prow[E] v; E of register pairs packed as two byte offsets.
+template <int N>
+__device__ __forceinline__ void apply_rows(float2 (&v)[N], const unsigned (&e)[(N + 1) / 2], const float2* prow) {
+  const char* p = reinterpret_cast<const char*>(prow);
+#pragma unroll
+  for (int r = 0; r < N; ++r) {
+    const unsigned off = (r & 1) ? e[r / 2] >> 16 : e[r / 2] & 0xffffu;
+    v[r] = cmul(v[r], *reinterpret_cast<const float2*>(p + off));
+  }
+}
+
+template <int N>
+__device__ __forceinline__ float norm_of(const float2 (&v)[N]) {
+  float a = 0.f, b = 0.f;
+#pragma unroll
+  for (int r = 0; r < N; ++r) {
+    a = fmaf(v[r].x, v[r].x, a);
+    b = fmaf(v[r].y, v[r].y, b);
+  }
+  return a + b;
+}
+
+// ------------------------------------------------------------ one warp ------
+constexpr int kWarpRing = 8;
+
+template <int N>
+__device__ void warp_run(const RunArgs& A, unsigned char* smem) {
+  const int lane = threadIdx.x & 31;
+  const int n = A.n, mp1 = A.m + 1;
+  float2* s_ab = reinterpret_cast<float2*>(smem);
+  float2* s_p = s_ab + kWarpRing;
+  ClauseMV* s_cl = reinterpret_cast<ClauseMV*>(smem + ((8u * (kWarpRing + kWarpRing * mp1) + 15u) & ~15u));
+  for (int j = 0; j < kWarpRing - 1; ++j) fetch_rows<32, kWarpRing>(A, s_p, s_ab, j, lane);
+  for (int c = lane; c < A.m; c += 32) s_cl[c] = A.cl[c];
+  const bool mine = lane < (1 << n);  // n < 5: the other lanes hold zeros
+  float2 v[N];
+#pragma unroll
+  for (int r = 0; r < N; ++r)
+    v[r] = !mine ? make_float2(0.f, 0.f) : (A.init ? make_float2(A.init_val, 0.f) : A.psi[lane + 32 * r]);
+  __syncwarp();
+  int ev[N];
+#pragma unroll
+  for (int r = 0; r < N; ++r) ev[r] = 0;
+  for (int c = 0; c < A.m; ++c) {
+    const unsigned mk = static_cast<unsigned>(s_cl[c].mask), vl = static_cast<unsigned>(s_cl[c].viol);
+#pragma unroll
+    for (int r = 0; r < N; ++r) ev[r] += (static_cast<unsigned>(lane + 32 * r) & mk) == vl;
+  }
+  unsigned e[(N + 1) / 2];
+#pragma unroll
+  for (int r = 0; r < N; r += 2) e[r / 2] = static_cast<unsigned>(8 * ev[r]) | (r + 1 < N ? static_cast<unsigned>(8 * ev[r + 1 < N ? r + 1 : r]) << 16 : 0u);
+  auto warp_norm = [&]() {
+    float s = norm_of<N>(v);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return DFloat{s, 0.f};
+  };
+  const DFloat nref = warp_norm();
+  const int pc = __popc(lane);
+#pragma unroll
+  for (int r = 0; r < N; ++r) v[r] = times_i(v[r], pc + __popc(r));
+  if (A.first_p) {
+#pragma unroll
+    for (int r = 0; r < N; ++r) v[r] = cmul(v[r], A.ptab[ev[r]]);
+  }
+  float fd = 0.f;
+  for (int j = 0; j < A.nsteps; ++j) {
+    fetch_rows<32, kWarpRing>(A, s_p, s_ab, j + kWarpRing - 1, lane);
+    cp_async_wait<kWarpRing - 1>();
+    __syncwarp();
+    const RotCoef c = rot_coef(s_ab[j % kWarpRing]);
+    if constexpr (N >= 2) reg_turn<0, (N >= 8 ? 3 : (N >= 4 ? 2 : 1))>(v, c);
+#pragma unroll
+    for (int b = 0; b < 5; ++b) {
+      if (b < n) {
+        const unsigned long long k = ((lane >> b) & 1) ? c.nb : c.b;
+#pragma unroll
+        for (int r = 0; r < N; ++r) {
+          const float2 p = make_float2(__shfl_xor_sync(0xffffffffu, v[r].x, 1 << b), __shfl_xor_sync(0xffffffffu, v[r].y, 1 << b));
+          v[r] = fma2(k, p, c.tangent ? v[r] : mul2(c.a, v[r]));
+        }
+      }
     }
-    s_e[oswz(x)] = static_cast<uint16_t>(e);
+    apply_rows<N>(v, e, s_p + (j % kWarpRing) * mp1);
+    if (fd != 0.f) {
+#pragma unroll
+      for (int r = 0; r < N; ++r) v[r] = fold_apply(v[r], fd);
+    }
+    fd = 0.f;
+    if ((j + 1) % fold_period(n) == 0 && j + 1 < A.nsteps)
+      fd = __shfl_sync(0xffffffffu, fold_scale(nref, warp_norm()), 0);
+    __syncwarp();
   }
-  __syncthreads();
+  if (mine) {
+#pragma unroll
+    for (int r = 0; r < N; ++r) A.psi[lane + 32 * r] = times_i(v[r], -(pc + __popc(r)));
+  }
+}
 
-  const int G = (n + 4) / 5;
-  const int mp1 = m + 1;
-  bool w0_done = false;
-  float cs = 0.0f;  // norm fold c - 1 of the previous step, applied with the popcount phase
-  for (int j = 0; j < nsteps; ++j) {
-    const float2* p_first = ptab;  // row 0, only when first_p and j == 0
-    const float2* p_next = ptab + static_cast<size_t>(j + 1) * mp1;
-    const float2* brow = btab + static_cast<size_t>(j) * (n + 1);
-    const bool last = j == nsteps - 1;
-    const unsigned pre = (j == 0 && first_p) ? kPreP : 0u;
-    // measure every fold_period(n)-th step; the factor corrects the step after it only
-    const bool measure = !last && (j + 1) % fold_period(n) == 0;
-    const unsigned nrm = measure ? kNorm : 0u;
-    float nacc = 0.0f;
-    if (G == 1) {
-      const unsigned f = pre | (w0_done ? 0u : kW1) | kMidB | kW2 | kPostP | (last ? 0u : kW3) | nrm;
-      round_dispatch(s_psi, s_e, n, 0, f, p_first, brow, p_next, cs, &nacc);
+size_t warp_smem(int m) {
+  return ((8u * (kWarpRing + static_cast<size_t>(kWarpRing) * (m + 1)) + 15u) & ~static_cast<size_t>(15)) + 16u * m;
+}
+
+// ------------------------------------------------------------- one CTA ------
+constexpr int kCtaRing = 4;
+
+template <int T, int R>
+struct CtaGeom {
+  static_assert(2 * R < T && T <= 3 * R, "three windows");
+  static constexpr int NT = 1 << (T - R);
+  static constexpr int N = 1 << R;
+  // Padded slot of index l, linear in disjoint bits.  Conflict-free for 8-byte
+  // accesses along consecutive l and along strides of 2^R (R = 3: a two-way
+  // conflict on a few lanes of the MID window).
+  __host__ __device__ static constexpr int slot(int l) { return R >= 4 ? l + (l >> R) : l + 2 * (l >> 4) + (l >> 6); }
+  static constexpr int SLOTS = slot((1 << T) - 1) + 1;
+  static constexpr bool kTwoBuffers = T <= 13;  // one barrier per transpose instead of two
+};
+
+enum Window { kTop, kBot, kMid };
+
+template <int T, int R, int W>
+__device__ __forceinline__ int win_base(int tid) {
+  if (W == kTop) return tid;
+  if (W == kBot) return tid << R;
+  return (tid & ((1 << R) - 1)) | ((tid >> R) << (2 * R));
+}
+template <int T, int R, int W>
+__device__ __forceinline__ constexpr int win_step() {
+  return W == kTop ? 1 << (T - R) : (W == kBot ? 1 : 1 << R);
+}
+
+template <int T, int R, int W>
+__device__ __forceinline__ void put(const float2 (&v)[1 << R], float2* buf, int tid) {
+  using G = CtaGeom<T, R>;
+  float2* p = buf + G::slot(win_base<T, R, W>(tid));
+#pragma unroll
+  for (int r = 0; r < (1 << R); ++r) p[G::slot(r * win_step<T, R, W>())] = v[r];
+}
+template <int T, int R, int W>
+__device__ __forceinline__ void get(float2 (&v)[1 << R], const float2* buf, int tid) {
+  using G = CtaGeom<T, R>;
+  const float2* p = buf + G::slot(win_base<T, R, W>(tid));
+#pragma unroll
+  for (int r = 0; r < (1 << R); ++r) v[r] = p[G::slot(r * win_step<T, R, W>())];
+}
+
+// Violated-clause counts of a thread's amplitudes (base xb, window bits
+// [p, p+R)), packed as byte offsets: every clause becomes (fixed mask, fixed
+// value, truth table over the window) in shared memory once, then each thread
+// adds the tables of the clauses whose fixed literals are all false, bit-sliced.
+template <int R, int NT>
+__device__ void window_energies(const ClauseMV* __restrict__ cl, int m, uint4* s_ent, int p, unsigned xb, int tid,
+                                unsigned (&e)[1 << (R - 1)]) {
+  const unsigned win = ((1u << R) - 1u) << p;
+  const int padded = (m + 15) & ~15;
+  team_sync<NT>();
+  for (int c = tid; c < padded; c += NT) {
+    uint4 t = make_uint4(0u, 0u, 0u, 0u);
+    if (c < m) {
+      const unsigned mk = static_cast<unsigned>(cl[c].mask), vl = static_cast<unsigned>(cl[c].viol);
+      unsigned pat = 0xffffffffu;
+      const unsigned half[5] = {0xaaaaaaaau, 0xccccccccu, 0xf0f0f0f0u, 0xff00ff00u, 0xffff0000u};
+#pragma unroll
+      for (int b = 0; b < R; ++b)
+        if ((mk >> (p + b)) & 1u) pat &= ((vl >> (p + b)) & 1u) ? half[b] : ~half[b];
+      t = make_uint4(mk & ~win, vl & ~win, pat, 0u);
+    }
+    s_ent[c] = t;
+  }
+  team_sync<NT>();
+  unsigned pl[kPlanes];
+  count_words(
+      padded,
+      [&](int i) {
+        const uint4 t = s_ent[i];
+        return ((xb ^ t.y) & t.x) == 0u ? t.z : 0u;
+      },
+      pl);
+#pragma unroll
+  for (int r = 0; r < (1 << R); r += 2) {
+    unsigned w = 0;
+#pragma unroll
+    for (int b = 0; b < kPlanes; ++b) w |= ((pl[b] >> r) & 1u) << (b + 3) | ((pl[b] >> (r + 1)) & 1u) << (b + 19);
+    e[r / 2] = w;
+  }
+}
+
+template <int T, int R>
+__host__ __device__ inline size_t cta_smem(int m) {
+  using G = CtaGeom<T, R>;
+  const size_t buf = (8u * static_cast<size_t>(G::SLOTS) * (G::kTwoBuffers ? 2 : 1) + 15u) & ~static_cast<size_t>(15);
+  const size_t ent = 16u * static_cast<size_t>((m + 15) & ~15);  // the buffers hold the clause tables first
+  return (buf > ent ? buf : ent) + 8u * kCtaRing * static_cast<size_t>(m + 2);
+}
+
+// The sum of one FP32 value per thread as a double-float pair (fixed order);
+// every thread gets it.
+template <int NT>
+__device__ DFloat cta_norm(float v, float* s_w, int tid) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  team_sync<NT>();
+  if ((tid & 31) == 0) s_w[tid >> 5] = v;
+  team_sync<NT>();
+  DFloat t{0.f, 0.f};
+#pragma unroll
+  for (int w = 0; w < NT / 32; ++w) t = df_add1(t, s_w[w]);
+  return t;
+}
+
+template <int T, int R>
+__device__ void cta_run(const RunArgs& A, unsigned char* smem) {
+  using G = CtaGeom<T, R>;
+  constexpr int NT = G::NT, N = G::N;
+  __shared__ float s_w[kBatchThreads / 32];
+  const int tid = threadIdx.x;
+  const int mp1 = A.m + 1;
+  float2* s_buf = reinterpret_cast<float2*>(smem);
+  float2* s_ab = reinterpret_cast<float2*>(smem + cta_smem<T, R>(A.m) - 8u * kCtaRing * static_cast<size_t>(A.m + 2));
+  float2* s_p = s_ab + kCtaRing;
+  for (int j = 0; j < kCtaRing - 1; ++j) fetch_rows<NT, kCtaRing>(A, s_p, s_ab, j, tid);
+  const int xt = win_base<T, R, kTop>(tid), xm = win_base<T, R, kMid>(tid);
+  float2 v[N];
+#pragma unroll
+  for (int r = 0; r < N; ++r) v[r] = A.init ? make_float2(A.init_val, 0.f) : A.psi[xt + (r << (T - R))];
+  unsigned et[N / 2], em[N / 2];
+  window_energies<R, NT>(A.cl, A.m, reinterpret_cast<uint4*>(smem), T - R, xt, tid, et);
+  window_energies<R, NT>(A.cl, A.m, reinterpret_cast<uint4*>(smem), R, xm, tid, em);
+  const DFloat nref = cta_norm<NT>(norm_of<N>(v), s_w, tid);  // also ends the use of s_buf as the clause tables
+#pragma unroll
+  for (int r = 0; r < N; ++r) v[r] = times_i(v[r], __popc(xt) + __popc(r));
+  if (A.first_p) apply_rows<N>(v, et, A.ptab);
+  float2* b0 = s_buf;
+  float2* b1 = s_buf + (G::kTwoBuffers ? G::SLOTS : 0);
+  float fd = 0.f;
+  cp_async_wait<1>();
+  team_sync<NT>();  // the first rotation is in
+  for (int j = 0; j < A.nsteps; ++j) {
+    if (!G::kTwoBuffers && j > 0) team_sync<NT>();  // the buffer is free
+    const RotCoef c = rot_coef(s_ab[j % kCtaRing]);
+    const float2* prow = s_p + (j % kCtaRing) * mp1;
+    const bool down = !(j & 1);
+    if (down) {
+      reg_turn<0, R>(v, c);
+      put<T, R, kTop>(v, b0, tid);
     } else {
-      if (!w0_done) round_dispatch(s_psi, s_e, n, 0, pre | kW1, p_first, brow, p_next, cs, &nacc);
-      for (int g = 1; g <= G - 2; ++g) round_dispatch(s_psi, s_e, n, g, kW1, p_first, brow, p_next, cs, &nacc);
-      round_dispatch(s_psi, s_e, n, G - 1, kW1 | kMidB | kW2, p_first, brow, p_next, cs, &nacc);
-      for (int g = G - 2; g >= 1; --g) round_dispatch(s_psi, s_e, n, g, kW1, p_first, brow, p_next, cs, &nacc);
-      round_dispatch(s_psi, s_e, n, 0, kW1 | kPostP | (last ? 0u : kW3) | nrm, p_first, brow, p_next, cs, &nacc);
+      reg_turn<0, T - 2 * R>(v, c);
+      put<T, R, kMid>(v, b0, tid);
     }
-    cs = measure ? onchip_fold(nacc, &nref).hi : 0.0f;
-    w0_done = !last;
+    cp_async_wait<1>();  // rows up to step j + 1, visible to all beyond the barrier
+    team_sync<NT>();
+    fetch_rows<NT, kCtaRing>(A, s_p, s_ab, j + kCtaRing - 1, tid);  // into the slot of step j - 1, which all have left
+    get<T, R, kBot>(v, b0, tid);
+    if (!G::kTwoBuffers) team_sync<NT>();
+    reg_turn<0, R>(v, c);
+    put<T, R, kBot>(v, b1, tid);
+    team_sync<NT>();
+    if (down) {
+      get<T, R, kMid>(v, b1, tid);
+      reg_turn<0, T - 2 * R>(v, c);
+      apply_rows<N>(v, em, prow);
+    } else {
+      get<T, R, kTop>(v, b1, tid);
+      reg_turn<0, R>(v, c);
+      apply_rows<N>(v, et, prow);
+    }
+    if (fd != 0.f) {
+#pragma unroll
+      for (int r = 0; r < N; ++r) v[r] = fold_apply(v[r], fd);
+    }
+    // measure every fold_period(n)-th step; the factor corrects the step after it only
+    fd = 0.f;
+    if ((j + 1) % fold_period(T) == 0 && j + 1 < A.nsteps) fd = fold_scale(nref, cta_norm<NT>(norm_of<N>(v), s_w, tid));
   }
-  for (int x = threadIdx.x; x < N; x += blockDim.x) psi[x] = s_psi[oswz(x)];
+  if (A.nsteps & 1) {
+#pragma unroll
+    for (int r = 0; r < N; ++r) A.psi[xm + (r << R)] = times_i(v[r], -(__popc(xm) + __popc(r)));
+  } else {
+#pragma unroll
+    for (int r = 0; r < N; ++r) A.psi[xt + (r << (T - R))] = times_i(v[r], -(__popc(xt) + __popc(r)));
+  }
 }
 
-__global__ void __launch_bounds__(kOnchipThreads)
-    onchip_kernel(float2* __restrict__ psi, int n, int m, const ClauseMV* __restrict__ cl,
-                  const float2* __restrict__ ptab, const float2* __restrict__ btab, int nsteps, int first_p) {
+// Register bits per thread of the CTA form: 32 amplitudes from n = 13, 16 at n =
+// 10..12, 8 at n = 9 (at least two warps).
+#define QAA_ONCHIP_SIZES(X) X(9, 3) X(10, 4) X(11, 4) X(12, 4) X(13, 5) X(14, 5)
+
+template <int T, int R>
+__global__ void __launch_bounds__(CtaGeom<T, R>::NT) cta_kernel(const RunArgs A) {
   extern __shared__ __align__(16) unsigned char smem[];
-  onchip_run(psi, n, m, cl, ptab, btab, nsteps, first_p, smem);
+  cta_run<T, R>(A, smem);
 }
 
-// A batch of independent instances of uneven size and length: one CTA each.
-__global__ void __launch_bounds__(kOnchipThreads) onchip_batch_kernel(const OnchipJob* __restrict__ jobs, int njobs) {
+__device__ void warp_dispatch(const RunArgs& A, unsigned char* smem) {
+  if (A.n <= 5)
+    warp_run<1>(A, smem);
+  else if (A.n == 6)
+    warp_run<2>(A, smem);
+  else if (A.n == 7)
+    warp_run<4>(A, smem);
+  else
+    warp_run<8>(A, smem);
+}
+
+__global__ void __launch_bounds__(32) warp_kernel(const RunArgs A) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  warp_dispatch(A, smem);
+}
+
+// A batch of independent instances of uneven size and length: one CTA each;
+// the threads an instance does not use leave at once.
+__global__ void __launch_bounds__(kBatchThreads) onchip_batch_kernel(const OnchipJob* __restrict__ jobs, int njobs) {
   extern __shared__ __align__(16) unsigned char smem[];
   if (static_cast<int>(blockIdx.x) >= njobs) return;
   const OnchipJob jb = jobs[blockIdx.x];
   if (jb.stamp && threadIdx.x == 0) *jb.stamp = global_ns();
-  onchip_run(jb.psi, jb.n, jb.m, jb.cl, jb.ptab, jb.btab, jb.nsteps, jb.first_p, smem, jb.init != 0, jb.init_val);
+  const RunArgs A{jb.psi, jb.cl, jb.ptab, jb.btab, jb.n, jb.m, jb.nsteps, jb.first_p != 0, jb.init != 0, jb.init_val};
+  switch (jb.n) {
+#define QAA_CASE(T, R)                                                        \
+  case T:                                                                     \
+    if (threadIdx.x < static_cast<unsigned>(CtaGeom<T, R>::NT)) cta_run<T, R>(A, smem); \
+    break;
+    QAA_ONCHIP_SIZES(QAA_CASE)
+#undef QAA_CASE
+    default:
+      if (threadIdx.x < 32) warp_dispatch(A, smem);
+  }
+}
+
+template <int T, int R>
+cudaError_t launch_cta(const LaunchCtx& lc, const RunArgs& A) {
+  const cudaError_t e =
+      allow_smem(reinterpret_cast<const void*>(cta_kernel<T, R>), cta_smem<T, R>(QAA_MAX_CLAUSES_DEV));
+  if (e != cudaSuccess) return e;
+  cta_kernel<T, R><<<1, CtaGeom<T, R>::NT, cta_smem<T, R>(A.m), lc.stream>>>(A);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+size_t onchip_smem_bytes(int n, int m) {
+  switch (n) {
+#define QAA_CASE(T, R) \
+  case T:              \
+    return cta_smem<T, R>(m);
+    QAA_ONCHIP_SIZES(QAA_CASE)
+#undef QAA_CASE
+    default:
+      return warp_smem(m);
+  }
+}
+
+// The largest dynamic shared memory any on-chip instance needs.
+static size_t onchip_smem_max() {
+  size_t b = 0;
+  for (int n = 1; n <= kOnchipMaxBits; ++n) {
+    const size_t s = onchip_smem_bytes(n, QAA_MAX_CLAUSES_DEV);
+    if (s > b) b = s;
+  }
+  return b;
 }
 
 cudaError_t launch_onchip_batch(const LaunchCtx& lc, const OnchipJob* jobs_dev, int njobs, size_t smem_bytes) {
   if (njobs <= 0) return cudaSuccess;
-  cudaError_t err =
-      allow_smem(reinterpret_cast<const void*>(onchip_batch_kernel), onchip_smem_bytes(kOnchipMaxBits, QAA_MAX_CLAUSES_DEV));
+  cudaError_t err = allow_smem(reinterpret_cast<const void*>(onchip_batch_kernel), onchip_smem_max());
   if (err != cudaSuccess) return err;
-  onchip_batch_kernel<<<njobs, kOnchipThreads, smem_bytes, lc.stream>>>(jobs_dev, njobs);
+  onchip_batch_kernel<<<njobs, kBatchThreads, smem_bytes, lc.stream>>>(jobs_dev, njobs);
   return cudaGetLastError();
 }
 
 cudaError_t launch_onchip(const LaunchCtx& lc, float2* psi, int n, int m, const ClauseMV* cl, const float2* ptab,
                           const float2* btab, int nsteps, bool first_p) {
-  if (n > kOnchipMaxBits) return cudaErrorInvalidValue;
-  const size_t smem = onchip_smem_bytes(n, m);
-  cudaError_t err = allow_smem(reinterpret_cast<const void*>(onchip_kernel), onchip_smem_bytes(kOnchipMaxBits, QAA_MAX_CLAUSES_DEV));
-  if (err != cudaSuccess) return err;
-  onchip_kernel<<<1, kOnchipThreads, smem, lc.stream>>>(psi, n, m, cl, ptab, btab, nsteps, first_p ? 1 : 0);
-  return cudaGetLastError();
+  if (n < 1 || n > kOnchipMaxBits) return cudaErrorInvalidValue;
+  const RunArgs A{psi, cl, ptab, btab, n, m, nsteps, first_p, false, 0.f};
+  switch (n) {
+#define QAA_CASE(T, R) \
+  case T:              \
+    return launch_cta<T, R>(lc, A);
+    QAA_ONCHIP_SIZES(QAA_CASE)
+#undef QAA_CASE
+    default: {
+      const cudaError_t e =
+          allow_smem(reinterpret_cast<const void*>(warp_kernel), onchip_smem_bytes(8, QAA_MAX_CLAUSES_DEV));
+      if (e != cudaSuccess) return e;
+      warp_kernel<<<1, 32, onchip_smem_bytes(n, m), lc.stream>>>(A);
+      return cudaGetLastError();
+    }
+  }
 }
 
 }  // namespace qaa

@@ -238,11 +238,43 @@ __device__ __forceinline__ double sched_s(const double* s_dev, long long K, long
   return s_dev ? s_dev[k] : (static_cast<double>(k) + 0.5) / static_cast<double>(K);
 }
 
+// The rotation of step k in the kRowsTurn form (RotCoef): h = dt (1 - s)/2,
+// (a, b) = (1, tan h) where |tan h| <= 1, with flip when cos h < 0 (then the
+// factor per qubit is -1/sqrt(1 + b^2)), else (cos h, sin h); a, b as rounded to FP32.
+struct Turn {
+  double h, a, b;
+  bool flip;
+};
+__device__ __forceinline__ Turn turn_of(double dt, double s) {
+  Turn t;
+  t.h = 0.5 * (dt * (1.0 - s));
+  double sn, cs;
+  sincos(t.h, &sn, &cs);
+  const bool tangent = fabs(sn) <= fabs(cs);
+  t.a = tangent ? 1.0 : static_cast<double>(static_cast<float>(cs));
+  t.b = static_cast<double>(static_cast<float>(tangent ? sn / cs : sn));
+  t.flip = tangent && cs < 0.0;
+  return t;
+}
+
+// The factor of P row p in the kRowsTurn form: (a^2 + b^2)^(-n/2) e^(-inh) of the
+// step the row ends (1 for p = 0), FP64.
+__device__ __noinline__ double2 row_factor(double dt, const double* dt_dev, const double* s_dev, long long K,
+                                           long long k0, long long p, int n) {
+  if (p < 1) return make_double2(1.0, 0.0);
+  const long long k = k0 + p - 1;
+  const Turn t = turn_of(dt_dev ? dt_dev[k] : dt, sched_s(s_dev, K, k));
+  const double amp = exp(-0.5 * n * log(t.a * t.a + t.b * t.b)) * (t.flip && (n & 1) ? -1.0 : 1.0);
+  double sn, cs;
+  sincos(n * t.h, &sn, &cs);
+  return make_double2(amp * cs, -amp * sn);
+}
+
 // With dt_dev (sub-steps of individual length, e.g. the fourth-order triple
 // jump) the two half phases are weighted by their own lengths:
 //   theta_p = 1/2 ( dt_(k0+p-1) s_(k0+p-1) [p >= 1] + dt_(k0+p) s_(k0+p) [p < k1-k0] ).
 __device__ __noinline__ float2 p_entry(double dt, const double* dt_dev, const double* s_dev, long long K, long long k0,
-                                       long long k1, long long p, int e) {
+                                       long long k1, long long p, int e, int form, double2 f) {
   double th = 0.0;
   if (dt_dev) {
     if (p >= 1) th += dt_dev[k0 + p - 1] * sched_s(s_dev, K, k0 + p - 1);
@@ -255,17 +287,28 @@ __device__ __noinline__ float2 p_entry(double dt, const double* dt_dev, const do
   }
   double sn, cs;
   sincos(th * static_cast<double>(e), &sn, &cs);
+  if (form == kRowsTurn) {
+    const double re = cs * f.x + sn * f.y;
+    sn = sn * f.x - cs * f.y;
+    cs = re;
+  }
   return make_float2(static_cast<float>(cs), static_cast<float>(-sn));
 }
 
-// With rot set (rotation form) the row instead holds exp(-i dt (1 - s_k) q)
+// Form kRowsBlock (rotation form): the row instead holds exp(-i dt (1 - s_k) q)
 // unscaled for q = 0..6, the rest zero: the per-block popcount phases of the
-// rotation form's 5- and 6-qubit Walsh-Hadamard sandwiches.
+// rotation form's 5- and 6-qubit Walsh-Hadamard sandwiches.  Form kRowsTurn:
+// entry 0 is (a, b) of turn_of, the rest zero.
 __device__ __noinline__ float2 b_entry(double dt, const double* dt_dev, const double* s_dev, long long K, long long k,
-                                       int q, double scale, int rot) {
+                                       int q, double scale, int form) {
   const double s = sched_s(s_dev, K, k);
   if (dt_dev) dt = dt_dev[k];
-  if (rot) {
+  if (form == kRowsTurn) {
+    if (q > 0) return make_float2(0.f, 0.f);
+    const Turn t = turn_of(dt, s);
+    return make_float2(static_cast<float>(t.a), static_cast<float>(t.b));
+  }
+  if (form == kRowsBlock) {
     if (q > 6) return make_float2(0.f, 0.f);
     scale = 1.0;
   }
@@ -276,23 +319,39 @@ __device__ __noinline__ float2 b_entry(double dt, const double* dt_dev, const do
 }
 
 // Phase tables for the steps c0 <= k < c1 of a range [k0, k1): P row rho is
-// position p = c0 - k0 + rho, B row rho is step k = c0 + rho.
-__global__ void tables_kernel(float2* __restrict__ ptab, float2* __restrict__ btab, int n, int m, double dt,
-                              const double* __restrict__ dt_dev, const double* __restrict__ s_dev, long long K,
-                              long long k0, long long k1, long long c0, long long c1, double scale, int rot) {
+// position p = c0 - k0 + rho, B row rho is step k = c0 + rho.  One thread per
+// entry, bound by the FP64 sine and cosine (GB300 does two FP64 operations per
+// clock and SM); a block's row factors (kRowsTurn) are computed once per row by
+// its first threads, not once per entry.
+constexpr int kTableThreads = 256;
+__global__ void __launch_bounds__(kTableThreads)
+    tables_kernel(float2* __restrict__ ptab, float2* __restrict__ btab, int n, int m, double dt,
+                  const double* __restrict__ dt_dev, const double* __restrict__ s_dev, long long K, long long k0,
+                  long long k1, long long c0, long long c1, double scale, int form) {
+  __shared__ double2 s_f[kTableThreads + 1];
   const long long prow_n = c1 - c0 + 1, brow_n = c1 - c0;
   const long long np = prow_n * (m + 1), nb = brow_n * (n + 1);
-  for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < np + nb;
-       i += static_cast<long long>(gridDim.x) * blockDim.x) {
+  for (long long b = blockIdx.x * static_cast<long long>(kTableThreads); b < np + nb;
+       b += static_cast<long long>(gridDim.x) * kTableThreads) {
+    const long long i = b + threadIdx.x;
+    const long long first = b / (m + 1);
+    if (form == kRowsTurn) {
+      __syncthreads();
+      const long long last = (b + kTableThreads - 1 < np ? b + kTableThreads - 1 : np - 1) / (m + 1);
+      if (b < np && first + threadIdx.x <= last)
+        s_f[threadIdx.x] = row_factor(dt, dt_dev, s_dev, K, k0, c0 - k0 + first + threadIdx.x, n);
+      __syncthreads();
+    }
     if (i < np) {
       const long long rho = i / (m + 1);
       const int e = static_cast<int>(i - rho * (m + 1));
-      ptab[i] = p_entry(dt, dt_dev, s_dev, K, k0, k1, c0 - k0 + rho, e);
-    } else {
+      ptab[i] = p_entry(dt, dt_dev, s_dev, K, k0, k1, c0 - k0 + rho, e, form,
+                        form == kRowsTurn ? s_f[rho - first] : make_double2(1.0, 0.0));
+    } else if (i < np + nb) {
       const long long j = i - np;
       const long long rho = j / (n + 1);
       const int q = static_cast<int>(j - rho * (n + 1));
-      btab[j] = b_entry(dt, dt_dev, s_dev, K, c0 + rho, q, scale, rot);
+      btab[j] = b_entry(dt, dt_dev, s_dev, K, c0 + rho, q, scale, form);
     }
   }
 }
@@ -305,7 +364,7 @@ __global__ void graph_rows_kernel(float2* __restrict__ prow, int dst_p0, long lo
                                   float2* __restrict__ brow, long long k_first, int nbrow,
                                   const long long* __restrict__ ctr, int n, int m, double dt,
                                   const double* __restrict__ dt_dev, const double* __restrict__ s_dev, long long K,
-                                  long long k0, long long k1, double scale, int rot) {
+                                  long long k0, long long k1, double scale, int form) {
   const long long off = ctr ? *ctr : 0;
   const long long np = static_cast<long long>(nprow) * (m + 1), nb = static_cast<long long>(nbrow) * (n + 1);
   for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < np + nb;
@@ -313,12 +372,14 @@ __global__ void graph_rows_kernel(float2* __restrict__ prow, int dst_p0, long lo
     if (i < np) {
       const long long j = i / (m + 1);
       const int e = static_cast<int>(i - j * (m + 1));
-      prow[(dst_p0 + j) * (m + 1) + e] = p_entry(dt, dt_dev, s_dev, K, k0, k1, p_first + off + j, e);
+      prow[(dst_p0 + j) * (m + 1) + e] = p_entry(dt, dt_dev, s_dev, K, k0, k1, p_first + off + j, e, form,
+                                           form == kRowsTurn ? row_factor(dt, dt_dev, s_dev, K, k0, p_first + off + j, n)
+                                                             : make_double2(1.0, 0.0));
     } else {
       const long long t = i - np;
       const long long j = t / (n + 1);
       const int q = static_cast<int>(t - j * (n + 1));
-      brow[t] = b_entry(dt, dt_dev, s_dev, K, k_first + off + j, q, scale, rot);
+      brow[t] = b_entry(dt, dt_dev, s_dev, K, k_first + off + j, q, scale, form);
     }
   }
 }
@@ -415,7 +476,7 @@ cudaError_t launch_init_uniform(const LaunchCtx& lc, float2* psi, int n) {
 
 cudaError_t launch_graph_rows(const LaunchCtx& lc, float2* prow, int dst_p0, long long p_first, int nprow, float2* brow,
                               long long k_first, int nbrow, const long long* ctr, int n, int m, double dt,
-                              const double* s_dev, long long K, long long k0, long long k1, bool rot,
+                              const double* s_dev, long long K, long long k0, long long k1, int form,
                               const double* dt_dev) {
   const long long total = static_cast<long long>(nprow) * (m + 1) + static_cast<long long>(nbrow) * (n + 1);
   long long grid = (total + 127) / 128;
@@ -423,7 +484,7 @@ cudaError_t launch_graph_rows(const LaunchCtx& lc, float2* prow, int dst_p0, lon
   if (grid < 1) grid = 1;
   graph_rows_kernel<<<static_cast<unsigned>(grid), 128, 0, lc.stream>>>(
       prow, dst_p0, p_first, nprow, brow, k_first, nbrow, ctr, n, m, dt, dt_dev, s_dev, K, k0, k1,
-      exp2(-static_cast<double>(n)), rot ? 1 : 0);
+      exp2(-static_cast<double>(n)), form);
   return cudaGetLastError();
 }
 
@@ -435,13 +496,13 @@ cudaError_t launch_graph_advance(const LaunchCtx& lc, long long* ctr, long long 
 
 cudaError_t launch_tables(const LaunchCtx& lc, float2* ptab, float2* btab, int n, int m, double dt,
                           const double* s_dev, long long K, long long k0, long long k1, long long c0, long long c1,
-                          bool rot, const double* dt_dev) {
+                          int form, const double* dt_dev) {
   const long long total = (c1 - c0 + 1) * (m + 1) + (c1 - c0) * (n + 1);
-  long long grid = (total + 255) / 256;
+  long long grid = (total + kTableThreads - 1) / kTableThreads;
   if (grid > 4ll * lc.num_sms) grid = 4ll * lc.num_sms;
   if (grid < 1) grid = 1;
-  tables_kernel<<<static_cast<unsigned>(grid), 256, 0, lc.stream>>>(ptab, btab, n, m, dt, dt_dev, s_dev, K, k0, k1,
-                                                                    c0, c1, exp2(-static_cast<double>(n)), rot ? 1 : 0);
+  tables_kernel<<<static_cast<unsigned>(grid), kTableThreads, 0, lc.stream>>>(ptab, btab, n, m, dt, dt_dev, s_dev, K, k0, k1,
+                                                                    c0, c1, exp2(-static_cast<double>(n)), form);
   return cudaGetLastError();
 }
 

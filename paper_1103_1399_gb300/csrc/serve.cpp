@@ -361,7 +361,7 @@ cudaError_t issue_streaming(qaa_server* s, Req* r, cudaStream_t st) {
   for (long long c0 = 0; e == cudaSuccess && c0 < r->K; c0 += r->chunk) {
     const long long c1 = std::min(r->K, c0 + r->chunk);
     e = qaa::launch_tables(lc, ptab, btab, r->n, r->m, dt, nullptr, r->K, 0, r->K, c0, c1,
-                           r->plan.wht_kind == qaa::kRotationForm);
+                           qaa::row_form(r->plan));
     qaa::build_passes(r->plan, 0, r->K, c0, c1, passes);
     for (const qaa::Pass& ps : passes) {
       if (e != cudaSuccess) break;
@@ -449,7 +449,8 @@ bool launch_batch(qaa_server* s, std::vector<Req*>& small) {
     const double dt = r->T / static_cast<double>(r->K);
     float2* ptab = r->d_tab;
     float2* btab = r->d_tab + static_cast<size_t>(r->K + 1) * (r->m + 1);
-    if (e == cudaSuccess) e = qaa::launch_tables(lc, ptab, btab, r->n, r->m, dt, nullptr, r->K, 0, r->K, 0, r->K);
+    if (e == cudaSuccess) 
+      e = qaa::launch_tables(lc, ptab, btab, r->n, r->m, dt, nullptr, r->K, 0, r->K, 0, r->K, qaa::row_form(r->plan));
     if (e != cudaSuccess) break;
     qaa::OnchipJob& j = s->h_jobs[t][nj++];
     j.psi = r->psi;
