@@ -66,16 +66,24 @@ __device__ __forceinline__ void reg_rot(float2 (&v)[32], const float2 (&tab)[6])
 // (re, im) as a packed pair.  Rows of the tangent form (a = 1, b = tan h, kept for
 // |tan h| <= 1) need one packed FMA per amplitude and qubit, against the two
 // additions and a fifth of a complex multiply of the Walsh-Hadamard sandwich,
-// and round once; the factor (a^2 + b^2)^(-n/2) e^(-inh) of the rounded a, b is
-// part of the phase row that ends the step (p_entry), so rounding a and b
-// changes the angle by less than 1e-7 of itself and the norm not at all.
-// Other angles use a = cos h, b = sin h.
+// and round once.  Other angles use a = cos h, b = sin h.  The norm of the rounded
+// (a, b) is taken out by the scale (a^2 + b^2)^(-n/2) = (1 + r) 2^-e: 2^-e in every step, the
+// product of the (1 + r) with the norm fold (TurnScale), so rounding a and b changes
+// the angle by less than 1e-7 of itself and the norm not at all; the phase e^(-inh), the same for
+// every amplitude, is left out until the last P row of a launch.  (As a factor of
+// every P row it would round the entry of E = 0, else exactly 1, in every step, and
+// with it the weight of the ground state: 2.6e-6 instead of 5e-7 after 400 steps.)
 struct RotCoef {
   unsigned long long a, b, nb;
+  float r, pow2;
   bool tangent;
 };
-__device__ __forceinline__ RotCoef rot_coef(float2 ab) {
+// row: the B row's entries 0 and 1.
+__device__ __forceinline__ RotCoef rot_coef(const float2* row) {
+  const float2 ab = row[0], sc = row[1];
   RotCoef c;
+  c.r = sc.x;
+  c.pow2 = sc.y;
   c.a = f2_bits(make_float2(ab.x, ab.x));
   c.b = f2_bits(make_float2(ab.y, ab.y));
   c.nb = f2_bits(make_float2(-ab.y, -ab.y));
@@ -92,35 +100,116 @@ __device__ __forceinline__ float2 mul2(unsigned long long k, float2 x) {
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(k), "l"(f2_bits(x)));
   return bits_f2(d);
 }
-// Register-index bits [B0, B1) of an N-entry register tile.
+__device__ __forceinline__ float2 add2(float2 x, float2 y) {
+  unsigned long long d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(f2_bits(x)), "l"(f2_bits(y)));
+  return bits_f2(d);
+}
+__device__ __forceinline__ float2 sub2(float2 x, float2 y) {
+  unsigned long long d;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(f2_bits(x)), "l"(f2_bits(y)));
+  return bits_f2(d);
+}
+// Turns of the register-index bits [B0, B1) of an N-entry tile by any angle.
 template <int B0, int B1, int N>
-__device__ __forceinline__ void reg_turn(float2 (&v)[N], const RotCoef& c) {
-  if (c.tangent) {
+__device__ __forceinline__ void reg_turn_any(float2 (&v)[N], const RotCoef& c) {
 #pragma unroll
-    for (int b = B0; b < B1; ++b) {
+  for (int b = B0; b < B1; ++b) {
 #pragma unroll
-      for (int r = 0; r < N; ++r) {
-        if (!(r & (1 << b))) {
-          const float2 u = v[r], w = v[r | (1 << b)];
-          v[r] = fma2(c.b, w, u);
-          v[r | (1 << b)] = fma2(c.nb, u, w);
-        }
-      }
-    }
-  } else {
-#pragma unroll
-    for (int b = B0; b < B1; ++b) {
-#pragma unroll
-      for (int r = 0; r < N; ++r) {
-        if (!(r & (1 << b))) {
-          const float2 u = v[r], w = v[r | (1 << b)];
-          v[r] = fma2(c.b, w, mul2(c.a, u));
-          v[r | (1 << b)] = fma2(c.nb, u, mul2(c.a, w));
-        }
+    for (int r = 0; r < N; ++r) {
+      if (!(r & (1 << b))) {
+        const float2 u = v[r], w = v[r | (1 << b)];
+        v[r] = fma2(c.b, w, mul2(c.a, u));
+        v[r | (1 << b)] = fma2(c.nb, u, mul2(c.a, w));
       }
     }
   }
 }
+// The same for either form of row; tangents two bits at a time:
+// on the four amplitudes of two bits
+//   (1 + tJ)(1 + tJ') v = v + t (Jv + J'v + t JJ'v),
+// so an amplitude rounds once per two qubits (the inner sum's errors come times
+// t) for 2.5 packed operations instead of 2.
+template <int B0, int B1, int N>
+__device__ __forceinline__ void reg_turn(float2 (&v)[N], const RotCoef& c) {
+  if (c.tangent) {
+#pragma unroll
+    for (int b = B0; b + 1 < B1; b += 2) {
+      const int p = 1 << b, q = 2 << b;
+#pragma unroll
+      for (int r = 0; r < N; ++r) {
+        if (!(r & (p | q))) {
+          const float2 v0 = v[r], v1 = v[r | p], v2 = v[r | q], v3 = v[r | p | q];
+          const float2 s = add2(v1, v2), e = sub2(v3, v0);
+          v[r] = fma2(c.b, fma2(c.b, v3, s), v0);
+          v[r | p] = fma2(c.b, fma2(c.nb, v2, e), v1);
+          v[r | q] = fma2(c.b, fma2(c.nb, v1, e), v2);
+          v[r | p | q] = fma2(c.nb, fma2(c.nb, v0, s), v3);
+        }
+      }
+    }
+    if constexpr ((B1 - B0) % 2 == 1) {
+#pragma unroll
+      for (int r = 0; r < N; ++r) {
+        constexpr int p = 1 << (B1 - 1);
+        if (!(r & p)) {
+          const float2 u = v[r], w = v[r | p];
+          v[r] = fma2(c.b, w, u);
+          v[r | p] = fma2(c.nb, u, w);
+        }
+      }
+    }
+  } else {
+    reg_turn_any<B0, B1>(v, c);
+  }
+}
+
+// A register tile with the increments since its last rounding kept apart: the
+// value is v + d.  A step's turns and phases are small changes, so d is computed to
+// 2^-24 of itself and an amplitude rounds once per settle() instead of once or
+// twice per turn and phase.  Where most of the weight sits in a few amplitudes
+// their rounding is the error of the ground-state probability and of <H_P>.
+template <int N>
+struct Inc {
+  float2 v[N], d[N];
+  __device__ __forceinline__ float2 at(int r) const { return add2(v[r], d[r]); }
+  __device__ __forceinline__ void zero() {
+#pragma unroll
+    for (int r = 0; r < N; ++r) d[r] = make_float2(0.f, 0.f);
+  }
+  __device__ __forceinline__ void settle() {
+#pragma unroll
+    for (int r = 0; r < N; ++r) v[r] = at(r);
+    zero();
+  }
+  // Turns of the register-index bits [B0, B1); `fresh`: d is zero.
+  template <int B0, int B1>
+  __device__ __forceinline__ void turn(const RotCoef& c, bool fresh = false) {
+    if (!c.tangent) {
+      settle();
+      reg_turn_any<B0, B1>(v, c);
+      return;
+    }
+#pragma unroll
+    for (int b = B0; b < B1; ++b) {
+#pragma unroll
+      for (int r = 0; r < N; ++r) {
+        if (!(r & (1 << b))) {
+          const int w = r | (1 << b);
+          const bool first = fresh && b == B0;
+          const float2 su = first ? v[r] : at(r), sw = first ? v[w] : at(w);
+          d[r] = first ? mul2(c.b, sw) : fma2(c.b, sw, d[r]);
+          d[w] = first ? mul2(c.nb, su) : fma2(c.nb, su, d[w]);
+        }
+      }
+    }
+  }
+  // a - 1 of both halves (exact: 0.5 <= a <= 1 or the result's own rounding).
+  __device__ __forceinline__ static unsigned long long add2_bits(unsigned long long a) {
+    return f2_bits(add2(bits_f2(a), make_float2(-1.0f, -1.0f)));
+  }
+};
+
 // v <- i^k v (exact).
 __device__ __forceinline__ float2 times_i(float2 v, int k) {
   const float2 s = (k & 1) ? make_float2(-v.y, v.x) : v;
@@ -443,6 +532,37 @@ __device__ __forceinline__ float fold_factor_block(const NormFold& f) {
   }
   __syncthreads();
   return s_c;
+}
+
+// The scale the turns of the steps so far still owe, as R = prod (1 + r) - 1, and
+// the norm fold.  Both are applied together, every fold_period steps and after the
+// last of a launch (so that the result carries no drift of the steps since the
+// last fold: up to 8e-7 with most of the weight in one amplitude): multiplying by 1 + r in every step (r ~ -1e-7 towards the end of a
+// sweep) would round an amplitude that hardly changes the same way every time.
+struct TurnScale {
+  float R = 0.f;
+  __device__ __forceinline__ void step(float r) { R = fmaf(R, r, R + r); }
+  // The factor minus 1 that brings the measured sum s to ref, R included; R restarts.
+  __device__ __forceinline__ float fold(DFloat ref, DFloat s) {
+    const float q = fmaf(R, R, 2.0f * R), p = s.hi * q;  // s (1 + R)^2
+    const float d = fold_scale(ref, df_add(s, DFloat{p, fmaf(s.hi, q, -p) + s.lo * q}));
+    const float k = fmaf(R, d, R + d);
+    R = 0.f;
+    return k;
+  }
+};
+template <int N>
+__device__ __forceinline__ void scale_by(float2 (&v)[N], float k) {
+  const unsigned long long kk = f2_bits(make_float2(k, k));
+#pragma unroll
+  for (int r = 0; r < N; ++r) v[r] = fma2(kk, v[r], v[r]);
+}
+template <int N>
+__device__ __forceinline__ void scale_pow2(float2 (&v)[N], float p) {
+  if (p == 1.0f) return;
+  const unsigned long long pp = f2_bits(make_float2(p, p));
+#pragma unroll
+  for (int r = 0; r < N; ++r) v[r] = mul2(pp, v[r]);
 }
 
 // Write the block's partial: the double-float sum of one pair per thread in a

@@ -77,6 +77,11 @@ struct qaa_ctx {
   // QAA_LP_COUNTS=0)
   unsigned* d_counts = nullptr;
   int counts_state = 0;
+  // team evolver (team.cu): E(x) and exchange scratch in one allocation made on
+  // first use; 0 = not yet, 1 = ready, 2 = scratch to be reset, -1 = not used
+  // (the device cannot hold the team, or no memory)
+  char* d_team = nullptr;
+  int team_state = 0;
   // Lanczos workspace (qaa_lowest_eigenvalues), allocated on first use
   void* d_lz = nullptr;
   size_t lz_bytes = 0;
@@ -110,10 +115,10 @@ cudaEvent_t take_event(qaa_ctx* h) {
   return e;
 }
 
-// Run `launch` (returns cudaError_t), bracketed by events when profiling.
+// Run `launch` (returns cudaError_t), bracketed by events when profiling (kind < 0: not).
 template <class F>
 cudaError_t timed(qaa_ctx* h, int kind, F&& launch) {
-  if (!h->prof) return launch();
+  if (!h->prof || kind < 0) return launch();
   cudaEvent_t a = take_event(h), b = take_event(h);
   if (a) cudaEventRecord(a, h->stream);
   const cudaError_t err = launch();
@@ -126,6 +131,26 @@ cudaError_t timed(qaa_ctx* h, int kind, F&& launch) {
   }
   return err;
 }
+
+// One profiler entry around everything enqueued during its life (h null: none).
+struct ProfSpan {
+  qaa_ctx* h;
+  int kind;
+  cudaEvent_t a = nullptr;
+  ProfSpan(qaa_ctx* h_, int k) : h(h_ && h_->prof ? h_ : nullptr), kind(k) {
+    if (h && (a = take_event(h))) cudaEventRecord(a, h->stream);
+  }
+  ~ProfSpan() {
+    if (!a) return;
+    cudaEvent_t b = take_event(h);
+    if (b) {
+      cudaEventRecord(b, h->stream);
+      h->pending.push_back({kind, a, b});
+    } else {
+      h->ev_free.push_back(a);
+    }
+  }
+};
 
 qaa_status fold_profile(qaa_ctx* h) {
   if (h->pending.empty()) return QAA_OK;
@@ -173,7 +198,9 @@ qaa_status check_device_error(qaa_ctx* h) {
   QAA_CK(cudaMemcpy(&e, h->d_err, sizeof(int), cudaMemcpyDeviceToHost));
   if (e != 0) {
     QAA_CK(cudaMemset(h->d_err, 0, sizeof(int)));
-    return fail(QAA_E_TIMEOUT, "a bounded wait on a TMA copy expired in a streaming pass");
+    if (h->team_state == 1) h->team_state = 2;
+    return fail(QAA_E_TIMEOUT, e == 2 ? "a bounded wait on another CTA of the evolving team expired"
+                                      : "a bounded wait on a TMA copy expired in a streaming pass");
   }
   return QAA_OK;
 }
@@ -212,6 +239,25 @@ const unsigned* stored_counts(qaa_ctx* h) {
     }
   }
   return h->counts_state == 1 ? h->d_counts : nullptr;
+}
+
+size_t energy_bytes(int n) { return ((size_t{2} << n) + 255) & ~size_t{255}; }
+
+// The team evolver's E(x) and scratch, made on the handle's stream the first
+// time; false when the passes run instead.
+bool team_ready(qaa_ctx* h) {
+  if (h->team_state == 0) {
+    h->team_state = -1;
+    if (qaa::team_fits(h->n, h->m, h->num_sms) &&
+        cudaMalloc(&h->d_team, energy_bytes(h->n) + qaa::team_bytes(h->n)) == cudaSuccess) {
+      if (qaa::launch_hp_diag(lctx(h), reinterpret_cast<uint16_t*>(h->d_team), h->n, h->m, h->d_lp) == cudaSuccess)
+        h->team_state = 2;
+    }
+    cudaGetLastError();
+    stored_counts(h);  // for the observables
+  }
+  if (h->team_state == 2 && qaa::team_reset(lctx(h), h->n, h->d_team + energy_bytes(h->n)) == cudaSuccess) h->team_state = 1;
+  return h->team_state == 1;
 }
 
 // Streaming plan, launch-graph mode: build (or reuse) the graph of the whole
@@ -292,8 +338,11 @@ qaa_status evolve_impl(qaa_ctx* h, void* psi, double dt, long long K, long long 
       dt_dev = h->d_s + K;
     }
   }
-  if (h->launch_mode == QAA_LAUNCH_GRAPH && h->n > qaa::kOnchipMaxBits)
-    return evolve_graph(h, static_cast<float2*>(psi), dt, K, k0, k1, s_dev, dt_dev);
+  const bool team = qaa::team_plan(h->plan) && team_ready(h);
+  // launch-graph mode: a team needs no graph (one launch per 1024 steps); the
+  // whole call counts as the graph it stands for
+  const bool graph = h->launch_mode == QAA_LAUNCH_GRAPH && h->n > qaa::kOnchipMaxBits;
+  if (graph && !team) return evolve_graph(h, static_cast<float2*>(psi), dt, K, k0, k1, s_dev, dt_dev);
   const long long chunk = std::min(kChunkSteps, k1 - k0);
   const size_t prow = static_cast<size_t>(h->m + 1), brow = static_cast<size_t>(h->n + 1);
   st = ensure_tab(h, static_cast<size_t>(chunk + 1) * prow + static_cast<size_t>(chunk) * brow);
@@ -303,12 +352,20 @@ qaa_status evolve_impl(qaa_ctx* h, void* psi, double dt, long long K, long long 
   const qaa::LaunchCtx lc = lctx(h);
   float2* p = static_cast<float2*>(psi);
   std::vector<qaa::Pass> passes;
+  ProfSpan span(graph ? h : nullptr, QAA_K_GRAPH);
   for (long long c0 = k0; c0 < k1; c0 += chunk) {
     const long long c1 = std::min(k1, c0 + chunk);
-    QAA_CK(timed(h, QAA_K_TABLES, [&] {
+    QAA_CK(timed(h, graph ? -1 : QAA_K_TABLES, [&] {
       return qaa::launch_tables(lc, ptab, btab, h->n, h->m, dt, s_dev, K, k0, k1, c0, c1,
-                                qaa::row_form(h->plan), dt_dev);
+                                qaa::row_form(h->plan, team), dt_dev);
     }));
+    if (team) {
+      QAA_CK(timed(h, graph ? -1 : QAA_K_ONCHIP, [&] {
+        return qaa::launch_team(lc, p, h->n, h->m, reinterpret_cast<const uint16_t*>(h->d_team), ptab, btab,
+                                static_cast<int>(c1 - c0), c0 == k0, h->d_team + energy_bytes(h->n), h->d_fold, h->d_err);
+      }));
+      continue;
+    }
     if (h->n <= qaa::kOnchipMaxBits) {
       QAA_CK(timed(h, QAA_K_ONCHIP, [&] {
         return qaa::launch_onchip(lc, p, h->n, h->m, h->d_mv, ptab, btab, static_cast<int>(c1 - c0), c0 == k0);
@@ -422,6 +479,7 @@ qaa_status qaa_destroy(qaa_handle h) {
   if (h->gexec) cudaGraphExecDestroy(h->gexec);
   cudaFree(h->d_gscratch);
   cudaFree(h->d_lz);
+  cudaFree(h->d_team);
   cudaFree(h->d_counts);
   cudaFree(h->d_tab);
   cudaFree(h->d_s);
@@ -592,7 +650,7 @@ qaa_status qaa_autotune(qaa_handle h, void* psi, int steps, double budget_ms, ch
     return finish(fail(QAA_E_CUDA, "autotune: no candidate plan ran"));
   }
   // stage 2: run length of each group that has a choice (Q >= 7 on TMA passes)
-  if (best.use_tma)
+  if (best.use_tma && !(best.team && !tc_kind))
     for (size_t i = 0; i < best.strided.size() && spent() <= budget_ms; ++i) {
       if (best.strided[i].q < 7) continue;
       qaa::PassPlan c = best;
@@ -600,7 +658,7 @@ qaa_status qaa_autotune(qaa_handle h, void* psi, int steps, double budget_ms, ch
       consider(c);
     }
   // stage 3: two equal q-bit groups (q >= 10) recombined as {10..14, 15+q..} and {15..14+q}, or back
-  if (best.use_tma && best.strided.size() == 2 && best.strided[0].q == best.strided[1].q && best.strided[0].q >= 10 &&
+  if (best.use_tma && !(best.team && !tc_kind) && best.strided.size() == 2 && best.strided[0].q == best.strided[1].q && best.strided[0].q >= 10 &&
       spent() <= budget_ms) {
     qaa::PassPlan c = best;
     const int q = c.strided[0].q, L = c.low_bits;
@@ -617,7 +675,7 @@ qaa_status qaa_autotune(qaa_handle h, void* psi, int steps, double budget_ms, ch
   // stage 4: plain loads instead of TMA (groups of at most 10 bits, contiguous)
   bool narrow = true;
   for (const auto& g : best.strided) narrow = narrow && g.q <= 10;
-  if (best.use_tma && narrow && best.low_bits == qaa::kLowBits && spent() <= budget_ms) {
+  if (best.use_tma && !(best.team && !tc_kind) && narrow && best.low_bits == qaa::kLowBits && spent() <= budget_ms) {
     qaa::PassPlan c = best;
     c.use_tma = false;
     c.wht_kind = 0;  // plain loads: the W.B.W form only
@@ -630,7 +688,7 @@ qaa_status qaa_autotune(qaa_handle h, void* psi, int steps, double budget_ms, ch
   }
   // stage 5: the rotation form of the H_B factor on the best plan (same step,
   // g instead of 2g - 2 round trips; FP32 CUDA-core passes only)
-  if (!tc_kind && best.use_tma && spent() <= budget_ms) {
+  if (!tc_kind && best.use_tma && !(best.team && !tc_kind) && spent() <= budget_ms) {
     qaa::PassPlan c = best;
     c.wht_kind = qaa::kRotationForm;
     consider(c);

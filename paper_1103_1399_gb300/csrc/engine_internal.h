@@ -38,6 +38,9 @@ struct PassPlan {
   int phase_group = 0;         // strided group whose pass fuses W B W
   std::vector<int> run_c;      // per strided group: 4 = 128-byte runs, 0 = default
   int low_bits = kLowBits;     // bits of the low pass: 10, or 12 (rotation form, kLpRot12)
+  // 15 <= n <= 21, rotation form with its default groups: runs on a team of CTAs
+  // (team.cu) instead of the passes
+  bool team = false;
 };
 
 // Plan for n: the one qaa_autotune chose for n on the current device, if any
@@ -73,9 +76,14 @@ void clear_tuned_plans();
 void build_passes(const PassPlan& plan, long long k0, long long k1, long long c0, long long c1,
                   std::vector<Pass>& out);
 
+// Whether the plan's evolutions run on a team of CTAs where the device can hold it.
+inline bool team_plan(const PassPlan& plan) {
+  return plan.onchip ? plan.n >= kTeamMinBits : plan.team && plan.wht_kind == kRotationForm;
+}
+
 // The phase rows (RowForm) this plan's kernels read.
-inline int row_form(const PassPlan& plan) {
-  return plan.onchip ? kRowsTurn : (plan.wht_kind == kRotationForm ? kRowsBlock : kRowsWbw);
+inline int row_form(const PassPlan& plan, bool team = false) {
+  return plan.onchip || team ? kRowsTurn : (plan.wht_kind == kRotationForm ? kRowsBlock : kRowsWbw);
 }
 
 std::string describe_plan(const PassPlan& plan);

@@ -1,4 +1,4 @@
-// Small-instance evolver (n <= 14): the whole complex64 state stays on chip for
+// Small-instance evolver (n <= 14): the whole complex64 state stays in one CTA for
 // every step of a run, so HBM is touched once on entry and once on exit.
 //
 // Same Strang step as the streaming path (Eq. (1) frozen at s_k; H_P the
@@ -18,37 +18,17 @@
 // n = 12, by the latency of a step's two barriers.  The earlier form (W B W in
 // columns of 32 amplitudes, 24 butterfly levels, four shared-memory rounds and
 // P rows from global memory) had 2^(n-5) threads busy.  Measured, us per step of
-// a 400-step run, before and after: n = 6 1.76 / 0.44, n = 9 1.83 / 0.61, n = 12
-// 3.23 / 1.39, n = 14 8.60 / 4.79.
+// a 400-step run, before and after: n = 6 1.76 / 0.48, n = 9 1.83 / 0.77, n = 11
+// 3.09 / 1.19 (from n = 12 on a single run takes a cluster, team.cu; batches keep one
+// CTA per instance).
 // Phase rows come through a ring of cp.async copies issued kRing - 1 steps ahead.
-#include "device_common.cuh"
+#include "tile.cuh"
 
 namespace qaa {
 
 namespace {
 
 constexpr int kBatchThreads = 512;
-
-__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
-               "l"(src)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
-// Barrier over the NT threads that run an instance (the others of a batch
-// CTA have left).
-template <int NT>
-__device__ __forceinline__ void team_sync() {
-  if constexpr (NT <= 32)
-    __syncwarp();
-  else
-    asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");
-}
 
 struct RunArgs {
   float2* psi;
@@ -69,31 +49,9 @@ __device__ __forceinline__ void fetch_rows(const RunArgs& A, float2* s_p, float2
     float2* dst = s_p + (j % RING) * mp1;
     const float2* src = A.ptab + static_cast<size_t>(j + 1) * mp1;
     for (int i = tid; i < mp1; i += NT) cp_async8(dst + i, src + i);
-    if (tid == 0) cp_async8(s_ab + j % RING, A.btab + static_cast<size_t>(j) * (A.n + 1));
+    if (tid < 2) cp_async8(s_ab + 2 * (j % RING) + tid, A.btab + static_cast<size_t>(j) * (A.n + 1) + tid);
   }
   cp_async_commit();
-}
-
-// v <- prow[E] v; E of register pairs packed as two byte offsets.
-template <int N>
-__device__ __forceinline__ void apply_rows(float2 (&v)[N], const unsigned (&e)[(N + 1) / 2], const float2* prow) {
-  const char* p = reinterpret_cast<const char*>(prow);
-#pragma unroll
-  for (int r = 0; r < N; ++r) {
-    const unsigned off = (r & 1) ? e[r / 2] >> 16 : e[r / 2] & 0xffffu;
-    v[r] = cmul(v[r], *reinterpret_cast<const float2*>(p + off));
-  }
-}
-
-template <int N>
-__device__ __forceinline__ float norm_of(const float2 (&v)[N]) {
-  float a = 0.f, b = 0.f;
-#pragma unroll
-  for (int r = 0; r < N; ++r) {
-    a = fmaf(v[r].x, v[r].x, a);
-    b = fmaf(v[r].y, v[r].y, b);
-  }
-  return a + b;
 }
 
 // ------------------------------------------------------------ one warp ------
@@ -104,12 +62,13 @@ __device__ void warp_run(const RunArgs& A, unsigned char* smem) {
   const int lane = threadIdx.x & 31;
   const int n = A.n, mp1 = A.m + 1;
   float2* s_ab = reinterpret_cast<float2*>(smem);
-  float2* s_p = s_ab + kWarpRing;
-  ClauseMV* s_cl = reinterpret_cast<ClauseMV*>(smem + ((8u * (kWarpRing + kWarpRing * mp1) + 15u) & ~15u));
+  float2* s_p = s_ab + 2 * kWarpRing;
+  ClauseMV* s_cl = reinterpret_cast<ClauseMV*>(smem + ((8u * (2 * kWarpRing + kWarpRing * mp1) + 15u) & ~15u));
   for (int j = 0; j < kWarpRing - 1; ++j) fetch_rows<32, kWarpRing>(A, s_p, s_ab, j, lane);
   for (int c = lane; c < A.m; c += 32) s_cl[c] = A.cl[c];
   const bool mine = lane < (1 << n);  // n < 5: the other lanes hold zeros
-  float2 v[N];
+  Inc<N> x;
+  auto& v = x.v;
 #pragma unroll
   for (int r = 0; r < N; ++r)
     v[r] = !mine ? make_float2(0.f, 0.f) : (A.init ? make_float2(A.init_val, 0.f) : A.psi[lane + 32 * r]);
@@ -125,46 +84,42 @@ __device__ void warp_run(const RunArgs& A, unsigned char* smem) {
   unsigned e[(N + 1) / 2];
 #pragma unroll
   for (int r = 0; r < N; r += 2) e[r / 2] = static_cast<unsigned>(8 * ev[r]) | (r + 1 < N ? static_cast<unsigned>(8 * ev[r + 1 < N ? r + 1 : r]) << 16 : 0u);
-  auto warp_norm = [&]() {
-    float s = norm_of<N>(v);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    return DFloat{s, 0.f};
-  };
+  auto warp_norm = [&]() { return warp_sum(norm_of<N>(v)); };
   const DFloat nref = warp_norm();
   const int pc = __popc(lane);
 #pragma unroll
   for (int r = 0; r < N; ++r) v[r] = times_i(v[r], pc + __popc(r));
   if (A.first_p) {
 #pragma unroll
-    for (int r = 0; r < N; ++r) v[r] = cmul(v[r], A.ptab[ev[r]]);
+    for (int r = 0; r < N; ++r) v[r] = add2(v[r], cmac(make_float2(0.f, 0.f), v[r], A.ptab[ev[r]]));
   }
-  float fd = 0.f;
+  x.zero();
+  TurnScale ts;
   for (int j = 0; j < A.nsteps; ++j) {
     fetch_rows<32, kWarpRing>(A, s_p, s_ab, j + kWarpRing - 1, lane);
     cp_async_wait<kWarpRing - 1>();
     __syncwarp();
-    const RotCoef c = rot_coef(s_ab[j % kWarpRing]);
-    if constexpr (N >= 2) reg_turn<0, (N >= 8 ? 3 : (N >= 4 ? 2 : 1))>(v, c);
+    const RotCoef c = rot_coef(s_ab + 2 * (j % kWarpRing));
+    const unsigned long long am1 = Inc<N>::add2_bits(c.a);
+    if constexpr (N >= 2) x.template turn<0, (N >= 8 ? 3 : (N >= 4 ? 2 : 1))>(c, true);
 #pragma unroll
     for (int b = 0; b < 5; ++b) {
       if (b < n) {
         const unsigned long long k = ((lane >> b) & 1) ? c.nb : c.b;
 #pragma unroll
         for (int r = 0; r < N; ++r) {
-          const float2 p = make_float2(__shfl_xor_sync(0xffffffffu, v[r].x, 1 << b), __shfl_xor_sync(0xffffffffu, v[r].y, 1 << b));
-          v[r] = fma2(k, p, c.tangent ? v[r] : mul2(c.a, v[r]));
+          const float2 s = x.at(r);
+          const float2 p = make_float2(__shfl_xor_sync(0xffffffffu, s.x, 1 << b), __shfl_xor_sync(0xffffffffu, s.y, 1 << b));
+          x.d[r] = fma2(k, p, c.tangent ? x.d[r] : fma2(am1, s, x.d[r]));
         }
       }
     }
-    apply_rows<N>(v, e, s_p + (j % kWarpRing) * mp1);
-    if (fd != 0.f) {
-#pragma unroll
-      for (int r = 0; r < N; ++r) v[r] = fold_apply(v[r], fd);
-    }
-    fd = 0.f;
-    if ((j + 1) % fold_period(n) == 0 && j + 1 < A.nsteps)
-      fd = __shfl_sync(0xffffffffu, fold_scale(nref, warp_norm()), 0);
+    apply_rows<N>(x, e, s_p + (j % kWarpRing) * mp1);
+    x.settle();
+    scale_pow2<N>(v, c.pow2);
+    // every fold_period(n)-th step and the last
+    ts.step(c.r);
+    if ((j + 1) % fold_period(n) == 0 || j + 1 == A.nsteps) scale_by<N>(v, __shfl_sync(0xffffffffu, ts.fold(nref, warp_norm()), 0));
     __syncwarp();
   }
   if (mine) {
@@ -174,52 +129,11 @@ __device__ void warp_run(const RunArgs& A, unsigned char* smem) {
 }
 
 size_t warp_smem(int m) {
-  return ((8u * (kWarpRing + static_cast<size_t>(kWarpRing) * (m + 1)) + 15u) & ~static_cast<size_t>(15)) + 16u * m;
+  return ((8u * (2 * kWarpRing + static_cast<size_t>(kWarpRing) * (m + 1)) + 15u) & ~static_cast<size_t>(15)) + 16u * m;
 }
 
 // ------------------------------------------------------------- one CTA ------
 constexpr int kCtaRing = 4;
-
-template <int T, int R>
-struct CtaGeom {
-  static_assert(2 * R < T && T <= 3 * R, "three windows");
-  static constexpr int NT = 1 << (T - R);
-  static constexpr int N = 1 << R;
-  // Padded slot of index l, linear in disjoint bits.  Conflict-free for 8-byte
-  // accesses along consecutive l and along strides of 2^R (R = 3: a two-way
-  // conflict on a few lanes of the MID window).
-  __host__ __device__ static constexpr int slot(int l) { return R >= 4 ? l + (l >> R) : l + 2 * (l >> 4) + (l >> 6); }
-  static constexpr int SLOTS = slot((1 << T) - 1) + 1;
-  static constexpr bool kTwoBuffers = T <= 13;  // one barrier per transpose instead of two
-};
-
-enum Window { kTop, kBot, kMid };
-
-template <int T, int R, int W>
-__device__ __forceinline__ int win_base(int tid) {
-  if (W == kTop) return tid;
-  if (W == kBot) return tid << R;
-  return (tid & ((1 << R) - 1)) | ((tid >> R) << (2 * R));
-}
-template <int T, int R, int W>
-__device__ __forceinline__ constexpr int win_step() {
-  return W == kTop ? 1 << (T - R) : (W == kBot ? 1 : 1 << R);
-}
-
-template <int T, int R, int W>
-__device__ __forceinline__ void put(const float2 (&v)[1 << R], float2* buf, int tid) {
-  using G = CtaGeom<T, R>;
-  float2* p = buf + G::slot(win_base<T, R, W>(tid));
-#pragma unroll
-  for (int r = 0; r < (1 << R); ++r) p[G::slot(r * win_step<T, R, W>())] = v[r];
-}
-template <int T, int R, int W>
-__device__ __forceinline__ void get(float2 (&v)[1 << R], const float2* buf, int tid) {
-  using G = CtaGeom<T, R>;
-  const float2* p = buf + G::slot(win_base<T, R, W>(tid));
-#pragma unroll
-  for (int r = 0; r < (1 << R); ++r) v[r] = p[G::slot(r * win_step<T, R, W>())];
-}
 
 // Violated-clause counts of a thread's amplitudes (base xb, window bits
 // [p, p+R)), packed as byte offsets: every clause becomes (fixed mask, fixed
@@ -267,21 +181,19 @@ __host__ __device__ inline size_t cta_smem(int m) {
   using G = CtaGeom<T, R>;
   const size_t buf = (8u * static_cast<size_t>(G::SLOTS) * (G::kTwoBuffers ? 2 : 1) + 15u) & ~static_cast<size_t>(15);
   const size_t ent = 16u * static_cast<size_t>((m + 15) & ~15);  // the buffers hold the clause tables first
-  return (buf > ent ? buf : ent) + 8u * kCtaRing * static_cast<size_t>(m + 2);
+  return (buf > ent ? buf : ent) + 8u * kCtaRing * static_cast<size_t>(m + 3);
 }
 
-// The sum of one FP32 value per thread as a double-float pair (fixed order);
-// every thread gets it.
+// The sum over the threads of a double-float (fixed order); every thread gets it.
 template <int NT>
-__device__ DFloat cta_norm(float v, float* s_w, int tid) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+__device__ DFloat cta_norm(DFloat v, DFloat* s_w, int tid) {
+  v = warp_sum(v);
   team_sync<NT>();
   if ((tid & 31) == 0) s_w[tid >> 5] = v;
   team_sync<NT>();
   DFloat t{0.f, 0.f};
 #pragma unroll
-  for (int w = 0; w < NT / 32; ++w) t = df_add1(t, s_w[w]);
+  for (int w = 0; w < NT / 32; ++w) t = df_add(t, s_w[w]);
   return t;
 }
 
@@ -289,15 +201,16 @@ template <int T, int R>
 __device__ void cta_run(const RunArgs& A, unsigned char* smem) {
   using G = CtaGeom<T, R>;
   constexpr int NT = G::NT, N = G::N;
-  __shared__ float s_w[kBatchThreads / 32];
+  __shared__ DFloat s_w[kBatchThreads / 32];
   const int tid = threadIdx.x;
   const int mp1 = A.m + 1;
   float2* s_buf = reinterpret_cast<float2*>(smem);
-  float2* s_ab = reinterpret_cast<float2*>(smem + cta_smem<T, R>(A.m) - 8u * kCtaRing * static_cast<size_t>(A.m + 2));
-  float2* s_p = s_ab + kCtaRing;
+  float2* s_ab = reinterpret_cast<float2*>(smem + cta_smem<T, R>(A.m) - 8u * kCtaRing * static_cast<size_t>(A.m + 3));
+  float2* s_p = s_ab + 2 * kCtaRing;
   for (int j = 0; j < kCtaRing - 1; ++j) fetch_rows<NT, kCtaRing>(A, s_p, s_ab, j, tid);
   const int xt = win_base<T, R, kTop>(tid), xm = win_base<T, R, kMid>(tid);
-  float2 v[N];
+  Tile<N, (R < 5)> x;
+  auto& v = x.v;
 #pragma unroll
   for (int r = 0; r < N; ++r) v[r] = A.init ? make_float2(A.init_val, 0.f) : A.psi[xt + (r << (T - R))];
   unsigned et[N / 2], em[N / 2];
@@ -307,21 +220,24 @@ __device__ void cta_run(const RunArgs& A, unsigned char* smem) {
 #pragma unroll
   for (int r = 0; r < N; ++r) v[r] = times_i(v[r], __popc(xt) + __popc(r));
   if (A.first_p) apply_rows<N>(v, et, A.ptab);
+  x.zero();
   float2* b0 = s_buf;
   float2* b1 = s_buf + (G::kTwoBuffers ? G::SLOTS : 0);
-  float fd = 0.f;
+  TurnScale ts;
   cp_async_wait<1>();
   team_sync<NT>();  // the first rotation is in
   for (int j = 0; j < A.nsteps; ++j) {
     if (!G::kTwoBuffers && j > 0) team_sync<NT>();  // the buffer is free
-    const RotCoef c = rot_coef(s_ab[j % kCtaRing]);
+    const RotCoef c = rot_coef(s_ab + 2 * (j % kCtaRing));
     const float2* prow = s_p + (j % kCtaRing) * mp1;
     const bool down = !(j & 1);
     if (down) {
-      reg_turn<0, R>(v, c);
+      x.template turn<0, R>(c);
+      x.settle();
       put<T, R, kTop>(v, b0, tid);
     } else {
-      reg_turn<0, T - 2 * R>(v, c);
+      x.template turn<0, T - 2 * R>(c);
+      x.settle();
       put<T, R, kMid>(v, b0, tid);
     }
     cp_async_wait<1>();  // rows up to step j + 1, visible to all beyond the barrier
@@ -329,25 +245,28 @@ __device__ void cta_run(const RunArgs& A, unsigned char* smem) {
     fetch_rows<NT, kCtaRing>(A, s_p, s_ab, j + kCtaRing - 1, tid);  // into the slot of step j - 1, which all have left
     get<T, R, kBot>(v, b0, tid);
     if (!G::kTwoBuffers) team_sync<NT>();
-    reg_turn<0, R>(v, c);
+    x.template turn<0, R>(c, true);
+    x.settle();
     put<T, R, kBot>(v, b1, tid);
     team_sync<NT>();
     if (down) {
       get<T, R, kMid>(v, b1, tid);
-      reg_turn<0, T - 2 * R>(v, c);
-      apply_rows<N>(v, em, prow);
+      x.template turn<0, T - 2 * R>(c, true);
+      x.phase(em, prow);
     } else {
       get<T, R, kTop>(v, b1, tid);
-      reg_turn<0, R>(v, c);
-      apply_rows<N>(v, et, prow);
+      x.template turn<0, R>(c, true);
+      x.phase(et, prow);
     }
-    if (fd != 0.f) {
-#pragma unroll
-      for (int r = 0; r < N; ++r) v[r] = fold_apply(v[r], fd);
+    if (c.pow2 != 1.0f) {
+      x.settle();
+      scale_pow2<N>(v, c.pow2);
     }
-    // measure every fold_period(n)-th step; the factor corrects the step after it only
-    fd = 0.f;
-    if ((j + 1) % fold_period(T) == 0 && j + 1 < A.nsteps) fd = fold_scale(nref, cta_norm<NT>(norm_of<N>(v), s_w, tid));
+    ts.step(c.r);
+    if ((j + 1) % fold_period(T) == 0 || j + 1 == A.nsteps) {
+      x.settle();
+      scale_by<N>(v, ts.fold(nref, cta_norm<NT>(norm_of<N>(v), s_w, tid)));
+    }
   }
   if (A.nsteps & 1) {
 #pragma unroll

@@ -238,6 +238,8 @@ __device__ __forceinline__ double sched_s(const double* s_dev, long long K, long
   return s_dev ? s_dev[k] : (static_cast<double>(k) + 0.5) / static_cast<double>(K);
 }
 
+constexpr int kTableThreads = 256;
+
 // The rotation of step k in the kRowsTurn form (RotCoef): h = dt (1 - s)/2,
 // (a, b) = (1, tan h) where |tan h| <= 1, with flip when cos h < 0 (then the
 // factor per qubit is -1/sqrt(1 + b^2)), else (cos h, sin h); a, b as rounded to FP32.
@@ -257,24 +259,31 @@ __device__ __forceinline__ Turn turn_of(double dt, double s) {
   return t;
 }
 
-// The factor of P row p in the kRowsTurn form: (a^2 + b^2)^(-n/2) e^(-inh) of the
-// step the row ends (1 for p = 0), FP64.
-__device__ __noinline__ double2 row_factor(double dt, const double* dt_dev, const double* s_dev, long long K,
-                                           long long k0, long long p, int n) {
-  if (p < 1) return make_double2(1.0, 0.0);
-  const long long k = k0 + p - 1;
-  const Turn t = turn_of(dt_dev ? dt_dev[k] : dt, sched_s(s_dev, K, k));
-  const double amp = exp(-0.5 * n * log(t.a * t.a + t.b * t.b)) * (t.flip && (n & 1) ? -1.0 : 1.0);
-  double sn, cs;
-  sincos(n * t.h, &sn, &cs);
-  return make_double2(amp * cs, -amp * sn);
+// kRowsTurn: the sum over the steps [c0, c1) of the phase n (h + pi [flip]) that the
+// rotations leave out, by every thread of the block (FP64, fixed order).
+__device__ double turn_phase(double dt, const double* dt_dev, const double* s_dev, long long K, long long c0,
+                             long long c1, int n) {
+  if (!dt_dev && !s_dev && fabs(dt) <= 1.5)  // linear sweep, no flips: the closed form
+    return 0.5 * n * dt * (static_cast<double>(c1 - c0) * (1.0 - 0.5 * static_cast<double>(c0 + c1) / static_cast<double>(K)));
+  __shared__ double s_sum[kTableThreads];
+  double t = 0.0;
+  for (long long k = c0 + threadIdx.x; k < c1; k += kTableThreads) {
+    const Turn u = turn_of(dt_dev ? dt_dev[k] : dt, sched_s(s_dev, K, k));
+    t += n * (u.h + (u.flip ? 3.141592653589793 : 0.0));
+  }
+  s_sum[threadIdx.x] = t;
+  __syncthreads();
+  t = 0.0;
+  for (int i = 0; i < kTableThreads; ++i) t += s_sum[i];
+  __syncthreads();
+  return t;
 }
 
 // With dt_dev (sub-steps of individual length, e.g. the fourth-order triple
 // jump) the two half phases are weighted by their own lengths:
 //   theta_p = 1/2 ( dt_(k0+p-1) s_(k0+p-1) [p >= 1] + dt_(k0+p) s_(k0+p) [p < k1-k0] ).
 __device__ __noinline__ float2 p_entry(double dt, const double* dt_dev, const double* s_dev, long long K, long long k0,
-                                       long long k1, long long p, int e, int form, double2 f) {
+                                       long long k1, long long p, int e, int form, double phase = 0.0) {
   double th = 0.0;
   if (dt_dev) {
     if (p >= 1) th += dt_dev[k0 + p - 1] * sched_s(s_dev, K, k0 + p - 1);
@@ -286,27 +295,26 @@ __device__ __noinline__ float2 p_entry(double dt, const double* dt_dev, const do
     th *= 0.5 * dt;
   }
   double sn, cs;
-  sincos(th * static_cast<double>(e), &sn, &cs);
-  if (form == kRowsTurn) {
-    const double re = cs * f.x + sn * f.y;
-    sn = sn * f.x - cs * f.y;
-    cs = re;
-  }
+  sincos(th * static_cast<double>(e) + phase, &sn, &cs);
+  if (form == kRowsTurn) cs -= 1.0;  // e^(-i theta E) - 1
   return make_float2(static_cast<float>(cs), static_cast<float>(-sn));
 }
 
 // Form kRowsBlock (rotation form): the row instead holds exp(-i dt (1 - s_k) q)
 // unscaled for q = 0..6, the rest zero: the per-block popcount phases of the
 // rotation form's 5- and 6-qubit Walsh-Hadamard sandwiches.  Form kRowsTurn:
-// entry 0 is (a, b) of turn_of, the rest zero.
+// entry 0 is (a, b) of turn_of, entry 1 the scale (a^2 + b^2)^(-n/2) = (1 + r) 2^-e
+// as (r, 2^-e), the rest zero; the phase e^(-inh) is part of the last P row.
 __device__ __noinline__ float2 b_entry(double dt, const double* dt_dev, const double* s_dev, long long K, long long k,
-                                       int q, double scale, int form) {
+                                       int q, double scale, int form, int n) {
   const double s = sched_s(s_dev, K, k);
   if (dt_dev) dt = dt_dev[k];
   if (form == kRowsTurn) {
-    if (q > 0) return make_float2(0.f, 0.f);
+    if (q > 1) return make_float2(0.f, 0.f);
     const Turn t = turn_of(dt, s);
-    return make_float2(static_cast<float>(t.a), static_cast<float>(t.b));
+    if (q == 0) return make_float2(static_cast<float>(t.a), static_cast<float>(t.b));
+    const double lg = -0.5 * n * log2(t.a * t.a + t.b * t.b), e = rint(lg);
+    return make_float2(static_cast<float>(exp2(lg - e) - 1.0), static_cast<float>(exp2(e)));
   }
   if (form == kRowsBlock) {
     if (q > 6) return make_float2(0.f, 0.f);
@@ -321,37 +329,28 @@ __device__ __noinline__ float2 b_entry(double dt, const double* dt_dev, const do
 // Phase tables for the steps c0 <= k < c1 of a range [k0, k1): P row rho is
 // position p = c0 - k0 + rho, B row rho is step k = c0 + rho.  One thread per
 // entry, bound by the FP64 sine and cosine (GB300 does two FP64 operations per
-// clock and SM); a block's row factors (kRowsTurn) are computed once per row by
-// its first threads, not once per entry.
-constexpr int kTableThreads = 256;
+// clock and SM).
 __global__ void __launch_bounds__(kTableThreads)
     tables_kernel(float2* __restrict__ ptab, float2* __restrict__ btab, int n, int m, double dt,
                   const double* __restrict__ dt_dev, const double* __restrict__ s_dev, long long K, long long k0,
                   long long k1, long long c0, long long c1, double scale, int form) {
-  __shared__ double2 s_f[kTableThreads + 1];
   const long long prow_n = c1 - c0 + 1, brow_n = c1 - c0;
   const long long np = prow_n * (m + 1), nb = brow_n * (n + 1);
+  const long long last = np - (m + 1);  // the last P row
   for (long long b = blockIdx.x * static_cast<long long>(kTableThreads); b < np + nb;
        b += static_cast<long long>(gridDim.x) * kTableThreads) {
     const long long i = b + threadIdx.x;
-    const long long first = b / (m + 1);
-    if (form == kRowsTurn) {
-      __syncthreads();
-      const long long last = (b + kTableThreads - 1 < np ? b + kTableThreads - 1 : np - 1) / (m + 1);
-      if (b < np && first + threadIdx.x <= last)
-        s_f[threadIdx.x] = row_factor(dt, dt_dev, s_dev, K, k0, c0 - k0 + first + threadIdx.x, n);
-      __syncthreads();
-    }
+    double phase = 0.0;
+    if (form == kRowsTurn && b < np && b + kTableThreads > last) phase = turn_phase(dt, dt_dev, s_dev, K, c0, c1, n);
     if (i < np) {
       const long long rho = i / (m + 1);
       const int e = static_cast<int>(i - rho * (m + 1));
-      ptab[i] = p_entry(dt, dt_dev, s_dev, K, k0, k1, c0 - k0 + rho, e, form,
-                        form == kRowsTurn ? s_f[rho - first] : make_double2(1.0, 0.0));
+      ptab[i] = p_entry(dt, dt_dev, s_dev, K, k0, k1, c0 - k0 + rho, e, form, i >= last ? phase : 0.0);
     } else if (i < np + nb) {
       const long long j = i - np;
       const long long rho = j / (n + 1);
       const int q = static_cast<int>(j - rho * (n + 1));
-      btab[j] = b_entry(dt, dt_dev, s_dev, K, c0 + rho, q, scale, form);
+      btab[j] = b_entry(dt, dt_dev, s_dev, K, c0 + rho, q, scale, form, n);
     }
   }
 }
@@ -372,14 +371,12 @@ __global__ void graph_rows_kernel(float2* __restrict__ prow, int dst_p0, long lo
     if (i < np) {
       const long long j = i / (m + 1);
       const int e = static_cast<int>(i - j * (m + 1));
-      prow[(dst_p0 + j) * (m + 1) + e] = p_entry(dt, dt_dev, s_dev, K, k0, k1, p_first + off + j, e, form,
-                                           form == kRowsTurn ? row_factor(dt, dt_dev, s_dev, K, k0, p_first + off + j, n)
-                                                             : make_double2(1.0, 0.0));
+      prow[(dst_p0 + j) * (m + 1) + e] = p_entry(dt, dt_dev, s_dev, K, k0, k1, p_first + off + j, e, form);
     } else {
       const long long t = i - np;
       const long long j = t / (n + 1);
       const int q = static_cast<int>(t - j * (n + 1));
-      brow[t] = b_entry(dt, dt_dev, s_dev, K, k_first + off + j, q, scale, form);
+      brow[t] = b_entry(dt, dt_dev, s_dev, K, k_first + off + j, q, scale, form, n);
     }
   }
 }

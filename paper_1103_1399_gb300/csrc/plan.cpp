@@ -155,6 +155,12 @@ void plan_with_groups(int n, const std::vector<int>& sizes, int phase_group, boo
   set_default_run_c(plan);
 }
 
+// Whether a default plan is run by a team of CTAs (not when its passes were asked
+// for through the environment).
+static bool default_team(const PassPlan& plan) {
+  return !plan.onchip && plan.n <= kTeamMaxBits && plan.wht_kind == kRotationForm && !env_overrides();
+}
+
 void plan_candidates(int n, std::vector<PassPlan>& out) {
   out.clear();
   if (n <= kOnchipMaxBits) return;
@@ -167,6 +173,7 @@ void plan_candidates(int n, std::vector<PassPlan>& out) {
   compositions(rest, g, max_q, cur, comps);
   PassPlan def;
   make_default_plan(n, def);
+  def.team = default_team(def);
   out.push_back(def);
   for (const auto& c : comps)
     for (int pg = 0; pg < g; ++pg) {
@@ -195,6 +202,7 @@ static bool fits(const PassPlan& plan, int max_q) {
 void make_plan(int n, PassPlan& plan, int max_q) {
   if (n > kOnchipMaxBits && !env_overrides() && tuned_plan(n, plan) && fits(plan, max_q)) return;
   make_default_plan(n, plan, max_q);
+  plan.team = default_team(plan);
 }
 
 void make_default_plan(int n, PassPlan& plan, int max_q, int low) {
@@ -367,7 +375,9 @@ void build_passes(const PassPlan& plan, long long k0, long long k1, long long c0
 }
 
 std::string describe_plan(const PassPlan& plan) {
-  if (plan.onchip) return "on-chip: whole run in one CTA's shared memory (n=" + std::to_string(plan.n) + ")";
+  if (plan.onchip)
+    return std::string("on-chip: whole run in the registers of ") +
+           (team_plan(plan) ? "a cluster of 8 CTAs" : (plan.n <= 8 ? "one warp" : "one CTA")) + " (n=" + std::to_string(plan.n) + ")";
   const int ng = static_cast<int>(plan.strided.size());
   if (plan.wht_kind == kRotationForm) {
     std::string d = "streaming, TMA loads, rotation form (H_B per 5-qubit block: W.diag.W); low pass bits [0," +
@@ -378,7 +388,8 @@ std::string describe_plan(const PassPlan& plan) {
       if (g.q > 5) d += "+[" + std::to_string(g.a2) + "," + std::to_string(g.a2 + g.q - 5) + ")";
       d += " R " + std::to_string(tma_run_bytes(g.q, plan.run_c[i])) + "B runs";
     }
-    return d + "; " + std::to_string(ng + 1) + " HBM round trips per step";
+    d += "; " + std::to_string(ng + 1) + " HBM round trips per step";
+    return team_plan(plan) ? d + "; none by default: the state in the registers of a team of CTAs" : d;
   }
   const char* wk = plan.wht_kind == 1 ? "tensor-core BF16x3" : (plan.wht_kind == 2 ? "tensor-core BF16x2" : "FP32");
   std::string d = "streaming, " + std::string(plan.wht_kind ? "plain" : (plan.use_tma ? "TMA" : "classic")) +

@@ -147,8 +147,8 @@ struct LaunchCtx {
 
 // Phase rows for: the W.B.W form (B rows 2^-n exp(-i dt (1 - s_k) q), q = 0..n),
 // the 5- and 6-qubit sandwiches of the rotation form (exp(-i dt (1 - s_k) q), q =
-// 0..6, unscaled), one-qubit rotations (B entry 0 = (a, b) of RotCoef, the step's
-// factor in the P row that ends it).
+// 0..6, unscaled), one-qubit rotations (B entries 0 and 1: RotCoef; the phase that
+// the rotations leave out is part of the last P row; P entries e^(-i theta E) - 1).
 enum RowForm : int { kRowsWbw = 0, kRowsBlock = 1, kRowsTurn = 2 };
 cudaError_t launch_init_uniform(const LaunchCtx& lc, float2* psi, int n);
 // Phase tables for steps c0 <= k < c1 of the range [k0, k1) of a K-step run:
@@ -190,6 +190,17 @@ struct OnchipJob {
   unsigned long long* stamp;  // if not null: the device time at the job's start (global_ns)
 };
 cudaError_t launch_onchip_batch(const LaunchCtx& lc, const OnchipJob* jobs_dev, int njobs, size_t smem_bytes);
+// The state in the registers of a team of CTAs for `nsteps` >= 1 steps (team.cu),
+// 12 <= n <= 21.  energy: E(x) as launch_hp_diag writes it; rows of the kRowsTurn
+// form; work: team_bytes(n) of device scratch, team_reset before its first launch
+// and after one that ran out of time (every complete launch leaves it reset);
+// fold: the range's norm-fold slots (first = the launch starts the range).
+constexpr int kTeamMinBits = 12, kTeamMaxBits = 21;
+bool team_fits(int n, int m, int num_sms);
+size_t team_bytes(int n);
+cudaError_t team_reset(const LaunchCtx& lc, int n, void* work);
+cudaError_t launch_team(const LaunchCtx& lc, float2* psi, int n, int m, const uint16_t* energy, const float2* ptab,
+                        const float2* btab, int nsteps, bool first, void* work, double* fold, int* err);
 cudaError_t launch_hp_diag(const LaunchCtx& lc, uint16_t* out, int n, int m, const ClauseLP* cl);
 // Observables: partials has room for obs_partials_len(n) doubles; result is 5 doubles
 // {norm, <H_P>, ground_prob, ground_count, sum of pair correlations} on the device.

@@ -132,6 +132,8 @@ struct Req {
   unsigned* d_bar = nullptr;
   unsigned* d_counts = nullptr;  // stored per-tile clause counts (streamed requests), else null
   size_t counts_bytes = 0;
+  char* d_team = nullptr;  // team evolver: E(x), then its exchange scratch (team requests), else null
+  size_t team_bytes = 0;
   double* d_fold = nullptr;  // norm-fold slots of the low passes (streamed and persistent requests)
   cudaEvent_t done_ev = nullptr;
   cudaGraphExec_t gexec = nullptr;  // launch graph of a streamed request, kept until it completes
@@ -140,6 +142,9 @@ struct Req {
   bool small() const { return plan.onchip; }
   bool persistent() const { return persist; }
 };
+
+// E(x) at the head of a team request's scratch.
+size_t energy_bytes(int n) { return align_up(static_cast<size_t>(2) << n); }
 
 // Phase-table bytes of a request: the whole run for on-chip and persistent
 // requests, the graph scratch (8 steps of rows) for launch-graph requests, a
@@ -152,9 +157,9 @@ size_t table_bytes(int n, int m, long long K, bool whole_run, bool graph) {
 // Device bytes of one request: state, clause tables, phase tables, reduction
 // partials, results, an error word, a grid-barrier word pair and, beyond the
 // on-chip sizes, the low passes' norm-fold slots.
-size_t request_bytes(int n, int m, size_t tab_bytes, size_t counts_bytes, int num_sms) {
+size_t request_bytes(int n, int m, size_t tab_bytes, size_t counts_bytes, size_t team_bytes, int num_sms) {
   size_t b = align_up((static_cast<size_t>(8) << n));
-  b += align_up(counts_bytes);
+  b += align_up(counts_bytes) + align_up(team_bytes);
   if (n > qaa::kOnchipMaxBits) b += align_up(qaa::kFoldBytes);
   b += align_up(16u * static_cast<size_t>(std::max(m, 1))) * 2;
   b += align_up(tab_bytes);
@@ -256,7 +261,7 @@ void release(qaa_server* s, Req* r) {
 bool place(qaa_server* s, Req* r) {
   r->chunk = (r->small() || r->persistent()) ? r->K : std::min(qaa::kChunkSteps, r->K);
   const size_t tb = table_bytes(r->n, r->m, r->K, r->small() || r->persistent(), r->graph);
-  const size_t need = request_bytes(r->n, r->m, tb, r->counts_bytes, s->num_sms);
+  const size_t need = request_bytes(r->n, r->m, tb, r->counts_bytes, r->team_bytes, s->num_sms);
   if (s->free_slots.empty()) return false;
   size_t off = 0;
   if (!s->arena.alloc(need, &off)) return false;
@@ -279,6 +284,7 @@ bool place(qaa_server* s, Req* r) {
   r->d_err = reinterpret_cast<int*>(take(16));
   r->d_bar = reinterpret_cast<unsigned*>(take(16));
   r->d_counts = r->counts_bytes ? reinterpret_cast<unsigned*>(take(r->counts_bytes)) : nullptr;
+  r->d_team = r->team_bytes ? take(r->team_bytes) : nullptr;
   r->d_fold = r->n > qaa::kOnchipMaxBits ? reinterpret_cast<double*>(take(qaa::kFoldBytes)) : nullptr;
   return true;
 }
@@ -326,8 +332,8 @@ cudaError_t mark_start(qaa_server* s, Req* r, cudaStream_t st) {
 }
 
 // The streaming evolution of one request (issuer thread, its own stream):
-// one launch graph for the whole run, or one launch per pass.
-
+// a team of CTAs (one launch per 1024 steps), one launch graph for the whole run,
+// or one launch per pass.
 cudaError_t issue_streaming(qaa_server* s, Req* r, cudaStream_t st) {
   const qaa::LaunchCtx lc{st, s->num_sms};
   cudaError_t e = mark_start(s, r, st);
@@ -335,7 +341,11 @@ cudaError_t issue_streaming(qaa_server* s, Req* r, cudaStream_t st) {
   if (e == cudaSuccess) e = qaa::launch_init_uniform(lc, r->psi, r->n);
   if (e == cudaSuccess && r->d_counts) e = qaa::launch_lp_counts(lc, r->d_counts, r->n, r->m, r->d_lp);
   const double dt = r->T / static_cast<double>(r->K);
-  if (r->graph) {
+  char* team_work = r->d_team ? r->d_team + energy_bytes(r->n) : nullptr;
+  if (r->d_team) {
+    if (e == cudaSuccess) e = qaa::launch_hp_diag(lc, reinterpret_cast<uint16_t*>(r->d_team), r->n, r->m, r->d_lp);
+    if (e == cudaSuccess) e = qaa::team_reset(lc, r->n, team_work);
+  } else if (r->graph) {
     qaa::GraphSpec gs;
     gs.plan = &r->plan;
     gs.psi = r->psi;
@@ -361,7 +371,13 @@ cudaError_t issue_streaming(qaa_server* s, Req* r, cudaStream_t st) {
   for (long long c0 = 0; e == cudaSuccess && c0 < r->K; c0 += r->chunk) {
     const long long c1 = std::min(r->K, c0 + r->chunk);
     e = qaa::launch_tables(lc, ptab, btab, r->n, r->m, dt, nullptr, r->K, 0, r->K, c0, c1,
-                           qaa::row_form(r->plan));
+                           qaa::row_form(r->plan, r->d_team != nullptr));
+    if (r->d_team) {
+      if (e == cudaSuccess)
+        e = qaa::launch_team(lc, r->psi, r->n, r->m, reinterpret_cast<const uint16_t*>(r->d_team), ptab, btab,
+                             static_cast<int>(c1 - c0), c0 == 0, team_work, r->d_fold, r->d_err);
+      continue;
+    }
     qaa::build_passes(r->plan, 0, r->K, c0, c1, passes);
     for (const qaa::Pass& ps : passes) {
       if (e != cudaSuccess) break;
@@ -739,13 +755,23 @@ qaa_status qaa_submit(qaa_server* s, int n, const int32_t* clauses, int m, doubl
     if (!r->plan.onchip && !r->persist && r->plan.use_tma && n > qaa::kOnchipMaxBits && !(env && std::atoi(env) == 0))
       r->counts_bytes = qaa::lp_counts_bytes(n);
   }
+  // A team's scratch is three times the state: only where it is a small part of
+  // the arena, so that it never decides whether a request fits.
+  if (!r->plan.onchip && !r->persist && qaa::team_plan(r->plan) && qaa::team_fits(n, m, s->num_sms)) {
+    const size_t tb = energy_bytes(n) + qaa::team_bytes(n);
+    if (tb <= s->arena.size() / 16) {
+      r->team_bytes = tb;
+      r->counts_bytes = 0;
+      r->graph = false;
+    }
+  }
   if (r->plan.onchip && qaa::onchip_smem_bytes(n, m) > 227u * 1024u) {
     delete r;
     return sfail(QAA_E_ARG, "instance too large for the on-chip evolver");
   }
   const size_t need =
       request_bytes(n, m, table_bytes(n, m, steps, r->plan.onchip || r->persist, r->graph), r->counts_bytes,
-                    s->num_sms);
+                    r->team_bytes, s->num_sms);
   if (need > s->arena.size()) {
     delete r;
     return sfail(QAA_E_NOMEM, "request needs " + std::to_string(need) + " device bytes, more than the server's " +

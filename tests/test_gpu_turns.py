@@ -1,5 +1,6 @@
-"""One-qubit rotations in the gauge i^popcount (on-chip sizes): every register
-window and lane layout, at angles of both row forms.
+"""One-qubit rotations in the gauge i^popcount (the sizes whose state stays on
+chip, n <= 21): every register window, lane layout and CTA team, at angles of
+both row forms, and runs longer than one launch.
 
 Steps of dt = 4.1 take theta = dt (1 - s) over (0, 4.1): tan(theta/2) below and
 above 1 in magnitude and cos(theta/2) of both signs, from a random state and
@@ -17,8 +18,7 @@ import satgen
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("K", [7, 18])
-@pytest.mark.parametrize("n", list(range(1, 15)))
+@pytest.mark.parametrize("n,K", [(n, K) for n in range(1, 22) for K in (7, 18)] + [(8, 1030), (13, 1030), (15, 1030)])
 def test_large_angles_match_oracle(n, K):
     import torch
     import paper_1103_1399_gb300 as q
