@@ -752,26 +752,35 @@ int sturm_count(const std::vector<double>& a, const std::vector<double>& b, int 
   return cnt;
 }
 
-// All eigenvalues (ascending) of the tridiagonal matrix rows [first, m) by bisection.
-std::vector<double> tridiag_eigs(const std::vector<double>& a, const std::vector<double>& b, int first, int m) {
-  double lo = 0.0, hi = 0.0;
-  for (int i = first; i < m; ++i) {
-    const double r = (i > first ? std::fabs(b[i]) : 0.0) + (i + 1 < m ? std::fabs(b[i + 1]) : 0.0);
-    lo = i == first ? a[i] - r : std::min(lo, a[i] - r);
-    hi = i == first ? a[i] + r : std::max(hi, a[i] + r);
+// Eigenvalues of the tridiagonal matrix rows [first, m) by bisection, one at a
+// time: the caller needs the lowest few of them and the largest, not all m.
+struct TridiagEigs {
+  const std::vector<double>&a, &b;
+  int first, m;
+  double lo = 0.0, hi = 0.0, span = 1.0;
+  TridiagEigs(const std::vector<double>& a_, const std::vector<double>& b_, int first_, int m_)
+      : a(a_), b(b_), first(first_), m(m_) {
+    for (int i = first; i < m; ++i) {
+      const double r = (i > first ? std::fabs(b[i]) : 0.0) + (i + 1 < m ? std::fabs(b[i + 1]) : 0.0);
+      lo = i == first ? a[i] - r : std::min(lo, a[i] - r);
+      hi = i == first ? a[i] + r : std::max(hi, a[i] + r);
+    }
+    span = std::max(1.0, hi - lo);
   }
-  const double span = std::max(1.0, hi - lo);
-  std::vector<double> ev;
-  for (int k = 0; k < m - first; ++k) {
+  // The k-th eigenvalue, ascending from 0.
+  double at(int k) const {
     double l = lo - 1e-12 * span, r = hi + 1e-12 * span;
     for (int it = 0; it < 200 && r - l > 1e-15 * span; ++it) {
       const double mid = 0.5 * (l + r);
       if (sturm_count(a, b, first, m, mid) > k) r = mid; else l = mid;
     }
-    ev.push_back(0.5 * (l + r));
+    return 0.5 * (l + r);
   }
-  return ev;
-}
+  // Whether an eigenvalue lies within tol of x.
+  bool near(double x, double tol) const {
+    return first < m && sturm_count(a, b, first, m, x + tol) > sturm_count(a, b, first, m, x - tol);
+  }
+};
 
 }  // namespace
 
@@ -804,6 +813,7 @@ qaa_status qaa_lowest_eigenvalues(qaa_handle h, double s, int k, int max_iter, i
   char* base = static_cast<char*>(h->d_lz);
   qaa::LanczosArgs a;
   a.n = h->n;
+  a.m = h->m;
   a.s = s;
   a.iters = max_iter;
   a.random_start = start;
@@ -839,26 +849,19 @@ qaa_status qaa_lowest_eigenvalues(qaa_handle h, double s, int k, int max_iter, i
   // Lanczos matrix T_m repeats converged eigenvalues and also has spurious
   // ones; a simple eigenvalue of T_m that is also an eigenvalue of T_m without
   // its first row and column is spurious, and repeated ones count once.
-  const std::vector<double> ev = tridiag_eigs(alpha, beta, 0, m);
-  const std::vector<double> evh = m > 1 ? tridiag_eigs(alpha, beta, 1, m) : std::vector<double>();
-  double tnorm = 1.0;
-  for (double x : ev) tnorm = std::max(tnorm, std::fabs(x));
+  const TridiagEigs ev(alpha, beta, 0, m), evh(alpha, beta, 1, m);
+  double x = ev.at(0);
+  const double tnorm = std::max({1.0, std::fabs(x), std::fabs(ev.at(m - 1))});
   const double tol = 1e-9 * tnorm;  // FP64 vectors: converged copies agree far below this
   int nf = 0;
-  for (size_t i = 0; i < ev.size() && nf < k;) {
-    size_t j = i;
-    while (j + 1 < ev.size() && ev[j + 1] - ev[i] <= tol) ++j;
-    bool good = j > i;  // repeated: a converged eigenvalue
-    if (!good) {
-      good = true;
-      for (double y : evh)
-        if (std::fabs(y - ev[i]) <= tol) {
-          good = false;
-          break;
-        }
-    }
-    if (good || m == 1) evals[nf++] = ev[i];
+  for (int i = 0; i < m && nf < k;) {
+    int j = i;
+    double next = 0.0;
+    while (j + 1 < m && (next = ev.at(j + 1)) - x <= tol) ++j;
+    const bool good = j > i || !evh.near(x, tol);  // repeated: a converged eigenvalue
+    if (good || m == 1) evals[nf++] = x;
     i = j + 1;
+    x = next;
   }
   *found = nf;
   return check_device_error(h);

@@ -264,7 +264,7 @@ cudaError_t launch_persist(const LaunchCtx& lc, const PersistPlan& pp, float2* p
 // device memory.  v, vp, w: 2^n real FP64 each; E: the exported H_P diagonal;
 // partials: lanczos_partials(num_sms) doubles.
 struct LanczosArgs {
-  int n = 0;
+  int n = 0, m = 0;
   double s = 0;
   int iters = 0;
   int random_start = 0;
