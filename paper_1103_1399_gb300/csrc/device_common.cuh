@@ -43,51 +43,35 @@ __device__ __forceinline__ void reg_wht(float2 (&v)[32]) {
   }
 }
 
-// exp(-i theta H_B) on the register-index bits [0, B) of a 32-entry register
-// tile, up to a factor 2^B.  H_B = sum_i (1 - sigma^x_i)/2 (Sec. 2.1) is a sum of
-// commuting one-qubit terms, so on any block of qubits its exponential is
-// W diag(exp(-i theta popcount)) W over that block alone: B butterfly levels,
-// one multiply by tab[popcount(r)] (tab[p] = exp(-i theta p), p = 0..5, FP64
-// rounded once), B levels again.  The factor 2^B is removed by one exact
-// power-of-two scale per step.
-template <int B>
-__device__ __forceinline__ void reg_rot(float2 (&v)[32], const float2 (&tab)[6]) {
-  reg_wht<0, B>(v);
-#pragma unroll
-  for (int r = 0; r < 32; ++r) v[r] = cmul(v[r], tab[__builtin_popcount(r & ((1 << B) - 1))]);
-  reg_wht<0, B>(v);
-}
-
 // ---- one-qubit rotations in the gauge i^popcount ------------------------------
 // exp(-i theta H_B) = prod_i e^(-ih) (cos h + i sin h sigma^x_i), h = theta / 2
 // (Sec. 2.1).  With phi_x = i^popcount(x) psi_x (an exact swap and negation of
-// components) every factor is real: (u, w) <- (a u + b w, a w - b u) on the pair
-// of amplitudes whose index differs in the bit (u: bit clear), so it acts on
-// (re, im) as a packed pair.  Rows of the tangent form (a = 1, b = tan h, kept for
-// |tan h| <= 1) need one packed FMA per amplitude and qubit, against the two
-// additions and a fifth of a complex multiply of the Walsh-Hadamard sandwich,
-// and round once.  Other angles use a = cos h, b = sin h.  The norm of the rounded
-// (a, b) is taken out by the scale (a^2 + b^2)^(-n/2) = (1 + r) 2^-e: 2^-e in every step, the
-// product of the (1 + r) with the norm fold (TurnScale), so rounding a and b changes
-// the angle by less than 1e-7 of itself and the norm not at all; the phase e^(-inh), the same for
+// components) every factor is real: cos h times (u, w) <- (u + b w, w - b u), b = tan
+// h, on the pair of amplitudes whose index differs in the bit (u: bit clear), so it
+// acts on (re, im) as a packed pair: one packed FMA per amplitude and qubit, against
+// the two additions and a fifth of a complex multiply of a Walsh-Hadamard sandwich,
+// and one rounding.  Angles with |tan h| > 1 are taken in two turns of h / 2.  The
+// norm is taken out by the scale (1 + b^2)^(-n/2) per turn of the rounded b, as (1 + r)
+// 2^-e: 2^-e in every step, the product of the (1 + r) with the norm fold (TurnScale;
+// the streaming low pass puts it into its P row), so rounding b changes the angle by
+// less than 1e-7 of itself and the norm not at all; the phase e^(-inh), the same for
 // every amplitude, is left out until the last P row of a launch.  (As a factor of
 // every P row it would round the entry of E = 0, else exactly 1, in every step, and
 // with it the weight of the ground state: 2.6e-6 instead of 5e-7 after 400 steps.)
 struct RotCoef {
-  unsigned long long a, b, nb;
+  unsigned long long b, nb;
   float r, pow2;
-  bool tangent;
+  bool twice;
 };
 // row: the B row's entries 0 and 1.
 __device__ __forceinline__ RotCoef rot_coef(const float2* row) {
-  const float2 ab = row[0], sc = row[1];
+  const float2 tb = row[0], sc = row[1];
   RotCoef c;
+  c.b = f2_bits(make_float2(tb.y, tb.y));
+  c.nb = f2_bits(make_float2(-tb.y, -tb.y));
   c.r = sc.x;
   c.pow2 = sc.y;
-  c.a = f2_bits(make_float2(ab.x, ab.x));
-  c.b = f2_bits(make_float2(ab.y, ab.y));
-  c.nb = f2_bits(make_float2(-ab.y, -ab.y));
-  c.tangent = ab.x == 1.0f;
+  c.twice = tb.x == 2.0f;
   return c;
 }
 __device__ __forceinline__ float2 fma2(unsigned long long k, float2 x, float2 y) {
@@ -110,29 +94,14 @@ __device__ __forceinline__ float2 sub2(float2 x, float2 y) {
   asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(f2_bits(x)), "l"(f2_bits(y)));
   return bits_f2(d);
 }
-// Turns of the register-index bits [B0, B1) of an N-entry tile by any angle.
-template <int B0, int B1, int N>
-__device__ __forceinline__ void reg_turn_any(float2 (&v)[N], const RotCoef& c) {
-#pragma unroll
-  for (int b = B0; b < B1; ++b) {
-#pragma unroll
-    for (int r = 0; r < N; ++r) {
-      if (!(r & (1 << b))) {
-        const float2 u = v[r], w = v[r | (1 << b)];
-        v[r] = fma2(c.b, w, mul2(c.a, u));
-        v[r | (1 << b)] = fma2(c.nb, u, mul2(c.a, w));
-      }
-    }
-  }
-}
-// The same for either form of row; tangents two bits at a time:
-// on the four amplitudes of two bits
-//   (1 + tJ)(1 + tJ') v = v + t (Jv + J'v + t JJ'v),
+// Turns of the register-index bits [B0, B1) of an N-entry tile.  PAIRS: two bits at
+// a time; on the four amplitudes of two bits
+//   (1 + bJ)(1 + bJ') v = v + b (Jv + J'v + b JJ'v),
 // so an amplitude rounds once per two qubits (the inner sum's errors come times
-// t) for 2.5 packed operations instead of 2.
-template <int B0, int B1, int N>
-__device__ __forceinline__ void reg_turn(float2 (&v)[N], const RotCoef& c) {
-  if (c.tangent) {
+// b) for 2.5 packed operations instead of 2, and a dozen more registers.
+template <int B0, int B1, int N, bool PAIRS>
+__device__ __forceinline__ void turn_once(float2 (&v)[N], const RotCoef& c) {
+  if constexpr (PAIRS) {
 #pragma unroll
     for (int b = B0; b + 1 < B1; b += 2) {
       const int p = 1 << b, q = 2 << b;
@@ -148,20 +117,25 @@ __device__ __forceinline__ void reg_turn(float2 (&v)[N], const RotCoef& c) {
         }
       }
     }
-    if constexpr ((B1 - B0) % 2 == 1) {
+  }
 #pragma unroll
-      for (int r = 0; r < N; ++r) {
-        constexpr int p = 1 << (B1 - 1);
-        if (!(r & p)) {
-          const float2 u = v[r], w = v[r | p];
-          v[r] = fma2(c.b, w, u);
-          v[r | p] = fma2(c.nb, u, w);
-        }
+  for (int b = PAIRS ? B1 - (B1 - B0) % 2 : B0; b < B1; ++b) {
+#pragma unroll
+    for (int r = 0; r < N; ++r) {
+      if (!(r & (1 << b))) {
+        const float2 u = v[r], w = v[r | (1 << b)];
+        v[r] = fma2(c.b, w, u);
+        v[r | (1 << b)] = fma2(c.nb, u, w);
       }
     }
-  } else {
-    reg_turn_any<B0, B1>(v, c);
   }
+}
+// (The second turn as its own code: a loop around one would make every load of v
+// finish before it starts.)
+template <int B0, int B1, int N, bool PAIRS = true>
+__device__ __forceinline__ void reg_turn(float2 (&v)[N], const RotCoef& c) {
+  turn_once<B0, B1, N, PAIRS>(v, c);
+  if (c.twice) turn_once<B0, B1, N, PAIRS>(v, c);
 }
 
 // A register tile with the increments since its last rounding kept apart: the
@@ -184,12 +158,7 @@ struct Inc {
   }
   // Turns of the register-index bits [B0, B1); `fresh`: d is zero.
   template <int B0, int B1>
-  __device__ __forceinline__ void turn(const RotCoef& c, bool fresh = false) {
-    if (!c.tangent) {
-      settle();
-      reg_turn_any<B0, B1>(v, c);
-      return;
-    }
+  __device__ __forceinline__ void once(const RotCoef& c, bool fresh) {
 #pragma unroll
     for (int b = B0; b < B1; ++b) {
 #pragma unroll
@@ -204,9 +173,13 @@ struct Inc {
       }
     }
   }
-  // a - 1 of both halves (exact: 0.5 <= a <= 1 or the result's own rounding).
-  __device__ __forceinline__ static unsigned long long add2_bits(unsigned long long a) {
-    return f2_bits(add2(bits_f2(a), make_float2(-1.0f, -1.0f)));
+  template <int B0, int B1>
+  __device__ __forceinline__ void turn(const RotCoef& c, bool fresh = false) {
+    once<B0, B1>(c, fresh);
+    if (c.twice) {
+      settle();
+      reg_turn<B0, B1, N, false>(v, RotCoef{c.b, c.nb, c.r, c.pow2, false});
+    }
   }
 };
 
@@ -370,26 +343,34 @@ __device__ __forceinline__ unsigned extract_pair(const unsigned (&pl)[kPlanes]) 
   return w;
 }
 
-template <int R>
+// v + v z for complex v, z: four FMAs, as a multiplication takes.
+__device__ __forceinline__ float2 cadd(float2 v, float2 z) {
+  return make_float2(fmaf(-v.y, z.y, fmaf(v.x, z.x, v.x)), fmaf(v.x, z.y, fmaf(v.y, z.x, v.y)));
+}
+
+template <int R, bool MINUS1>
 struct ApplyPhaseUnroll {
   __device__ __forceinline__ static void run(float2 (&v)[32], const unsigned (&pl)[kPlanes], int nconst,
                                              const float2* __restrict__ tab) {
     const unsigned w = extract_pair<R>(pl);
-    v[R] = cmul(v[R], tab[nconst + static_cast<int>(w & 0xffffu)]);
-    v[R + 16] = cmul(v[R + 16], tab[nconst + static_cast<int>(w >> 16)]);
-    ApplyPhaseUnroll<R + 1>::run(v, pl, nconst, tab);
+    const float2 z0 = tab[nconst + static_cast<int>(w & 0xffffu)], z1 = tab[nconst + static_cast<int>(w >> 16)];
+    v[R] = MINUS1 ? cadd(v[R], z0) : cmul(v[R], z0);
+    v[R + 16] = MINUS1 ? cadd(v[R + 16], z1) : cmul(v[R + 16], z1);
+    ApplyPhaseUnroll<R + 1, MINUS1>::run(v, pl, nconst, tab);
   }
 };
-template <>
-struct ApplyPhaseUnroll<16> {
+template <bool MINUS1>
+struct ApplyPhaseUnroll<16, MINUS1> {
   __device__ __forceinline__ static void run(float2 (&)[32], const unsigned (&)[kPlanes], int, const float2*) {}
 };
 
 // v[r] <- exp(-i theta E(x_r)) v[r] where E = nconst + the bit-sliced count in
-// pl and tab[E] holds the FP32-rounded FP64 phase (the P row of the step).
+// pl and tab[E] holds the FP32-rounded FP64 phase (the P row of the step), minus 1
+// with MINUS1 (kRowsTurn).
+template <bool MINUS1 = false>
 __device__ __forceinline__ void apply_p_phase(float2 (&v)[32], const unsigned (&pl)[kPlanes], int nconst,
                                               const float2* __restrict__ tab) {
-  ApplyPhaseUnroll<0>::run(v, pl, nconst, tab);
+  ApplyPhaseUnroll<0, MINUS1>::run(v, pl, nconst, tab);
 }
 
 template <int R>

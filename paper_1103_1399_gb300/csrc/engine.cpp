@@ -65,11 +65,12 @@ struct qaa_ctx {
     const double* dt_dev;
     long long K, k0, k1;
     int wht_kind;
+    bool any_angle;
     cudaStream_t stream;
     bool operator==(const GraphKey& o) const {
       return psi == o.psi && std::memcmp(&dt, &o.dt, sizeof dt) == 0 && s_dev == o.s_dev && dt_dev == o.dt_dev &&
              K == o.K && k0 == o.k0 &&
-             k1 == o.k1 && wht_kind == o.wht_kind && stream == o.stream;
+             k1 == o.k1 && wht_kind == o.wht_kind && any_angle == o.any_angle && stream == o.stream;
     }
   } gkey{};
   // stored per-tile clause counts for the merged low passes: 0 = not yet
@@ -264,14 +265,15 @@ bool team_ready(qaa_ctx* h) {
 // range and launch it.  The graph is rebuilt when psi, the schedule, the range,
 // the variant or the stream changes.
 qaa_status evolve_graph(qaa_ctx* h, float2* psi, double dt, long long K, long long k0, long long k1, const double* s_dev,
-                 const double* dt_dev) {
+                 const double* dt_dev, bool any_angle) {
   if (!h->d_gscratch) {
     if (cudaMalloc(&h->d_gscratch, qaa::graph_scratch_bytes(h->n, h->m)) != cudaSuccess) {
       cudaGetLastError();
       return fail(QAA_E_NOMEM, "cannot allocate graph scratch");
     }
   }
-  const qaa_ctx::GraphKey key{psi, dt, s_dev, dt_dev, K, k0, k1, h->plan.wht_kind, h->stream};
+  const qaa_ctx::GraphKey key{psi, dt, s_dev, dt_dev, K, k0, k1, h->plan.wht_kind, any_angle, h->stream};
+  // (a schedule's values may change behind the same pointer: any_angle is part of the key)
   if (!h->gexec || !(key == h->gkey)) {
     if (h->gexec) {
       QAA_CK(cudaStreamSynchronize(h->stream));
@@ -289,6 +291,7 @@ qaa_status evolve_graph(qaa_ctx* h, float2* psi, double dt, long long K, long lo
     gs.dt_dev = dt_dev;
     gs.counts = stored_counts(h);
     gs.fold = h->d_fold;
+    gs.any_angle = any_angle;
     gs.K = K;
     gs.k0 = k0;
     gs.k1 = k1;
@@ -342,7 +345,8 @@ qaa_status evolve_impl(qaa_ctx* h, void* psi, double dt, long long K, long long 
   // launch-graph mode: a team needs no graph (one launch per 1024 steps); the
   // whole call counts as the graph it stands for
   const bool graph = h->launch_mode == QAA_LAUNCH_GRAPH && h->n > qaa::kOnchipMaxBits;
-  if (graph && !team) return evolve_graph(h, static_cast<float2*>(psi), dt, K, k0, k1, s_dev, dt_dev);
+  const bool any_angle = !qaa::small_angles(h->n, dt, s_host, dt_host, K, k0, k1);
+  if (graph && !team) return evolve_graph(h, static_cast<float2*>(psi), dt, K, k0, k1, s_dev, dt_dev, any_angle);
   const long long chunk = std::min(kChunkSteps, k1 - k0);
   const size_t prow = static_cast<size_t>(h->m + 1), brow = static_cast<size_t>(h->n + 1);
   st = ensure_tab(h, static_cast<size_t>(chunk + 1) * prow + static_cast<size_t>(chunk) * brow);
@@ -357,7 +361,7 @@ qaa_status evolve_impl(qaa_ctx* h, void* psi, double dt, long long K, long long 
     const long long c1 = std::min(k1, c0 + chunk);
     QAA_CK(timed(h, graph ? -1 : QAA_K_TABLES, [&] {
       return qaa::launch_tables(lc, ptab, btab, h->n, h->m, dt, s_dev, K, k0, k1, c0, c1,
-                                qaa::row_form(h->plan, team), dt_dev);
+                                qaa::row_form(h->plan), dt_dev);
     }));
     if (team) {
       QAA_CK(timed(h, graph ? -1 : QAA_K_ONCHIP, [&] {
@@ -371,7 +375,7 @@ qaa_status evolve_impl(qaa_ctx* h, void* psi, double dt, long long K, long long 
         return qaa::launch_onchip(lc, p, h->n, h->m, h->d_mv, ptab, btab, static_cast<int>(c1 - c0), c0 == k0);
       }));
     } else {
-      qaa::build_passes(h->plan, k0, k1, c0, c1, passes);
+      qaa::build_passes(h->plan, k0, k1, c0, c1, passes, any_angle);
       const unsigned* counts = stored_counts(h);
       for (const qaa::Pass& ps : passes)
         QAA_CK(timed(h, prof_kind(ps.kind), [&] {
@@ -540,9 +544,9 @@ qaa_status qaa_set_variant(qaa_handle h, int wht_kind, int q) {
                                  std::to_string(q) + " bits");
   }
   if (q != 0)
-    qaa::make_default_plan(h->n, h->plan, q, low);  // groups of at most q bits (the fewest such groups)
+    qaa::make_default_plan(h->n, h->plan, q, low, wht_kind == qaa::kRotationForm);  // groups of at most q bits (the fewest such groups)
   else
-    qaa::make_plan(h->n, h->plan, widest);
+    qaa::make_plan(h->n, h->plan, widest, wht_kind == qaa::kRotationForm);
   // a plan made (or tuned) for the other form gets the run lengths of this one
   const bool same_form = (h->plan.wht_kind == qaa::kRotationForm) == (wht_kind == qaa::kRotationForm);
   h->plan.wht_kind = wht_kind;

@@ -47,12 +47,13 @@ struct PassPlan {
 // and if no tuning override is set in the environment; otherwise the default.
 // max_q: widest strided group allowed (11 on the TMA FP32 passes; 10 for the
 // plain-load and tensor-core passes, which have no 11-bit tiles).
-void make_plan(int n, PassPlan& plan, int max_q = 11);
+// rotation: whether it is for the rotation form (some groups differ).
+void make_plan(int n, PassPlan& plan, int max_q = 11, bool rotation = true);
 // Default plan for n, with the tuning overrides QAA_PASSES, QAA_SPLIT_GROUPS,
 // QAA_PHASE_GROUP, QAA_RUN128_GROUPS, QAA_GROUP_BITS and QAA_LOW_BITS read
 // from the environment.  low: bits of the low pass, 10 or 12 (12 only for the
 // rotation form on TMA passes); 0 = QAA_LOW_BITS, else 10.
-void make_default_plan(int n, PassPlan& plan, int max_q = 11, int low = 0);
+void make_default_plan(int n, PassPlan& plan, int max_q = 11, int low = 0, bool rotation = true);
 // Run lengths per group for the plan's form (QAA_RUN128_GROUPS overrides).
 void set_default_run_c(PassPlan& plan);
 // A plan with a 12-bit low pass becomes the default plan with a 10-bit one
@@ -71,10 +72,15 @@ void set_tuned_plan(const PassPlan& plan);  // record for (current device, plan.
 bool tuned_plan(int n, PassPlan& out);
 void clear_tuned_plans();
 
+// Whether every step of the range has rows with times = 1 and e = 0 (RotCoef):
+// |h| <= pi/4 and cos^n h > 1/sqrt 2, h = dt (1 - s)/2, with a margin for rounding.
+// s_host, dt_host: K entries each, or null for the linear sweep and the uniform dt.
+bool small_angles(int n, double dt, const double* s_host, const double* dt_host, long long K, long long k0, long long k1);
+
 // Passes for steps c0 <= k < c1 of the range [k0, k1): P rows are relative to
 // the chunk (row k + 1 - c0 ends step k), B rows likewise (row k - c0).
 void build_passes(const PassPlan& plan, long long k0, long long k1, long long c0, long long c1,
-                  std::vector<Pass>& out);
+                  std::vector<Pass>& out, bool any_angle = true);
 
 // Whether the plan's evolutions run on a team of CTAs where the device can hold it.
 inline bool team_plan(const PassPlan& plan) {
@@ -82,8 +88,8 @@ inline bool team_plan(const PassPlan& plan) {
 }
 
 // The phase rows (RowForm) this plan's kernels read.
-inline int row_form(const PassPlan& plan, bool team = false) {
-  return plan.onchip || team ? kRowsTurn : (plan.wht_kind == kRotationForm ? kRowsBlock : kRowsWbw);
+inline int row_form(const PassPlan& plan) {
+  return plan.onchip || plan.wht_kind == kRotationForm ? kRowsTurn : kRowsWbw;
 }
 
 std::string describe_plan(const PassPlan& plan);
@@ -94,7 +100,7 @@ cudaError_t launch_planned_pass(const LaunchCtx& lc, const PassPlan& plan, const
                                 const ClauseLP* cl, const float2* ptab, const float2* btab, int* err,
                                 const unsigned* counts = nullptr, double* fold = nullptr);
 
-constexpr long long kChunkSteps = 1024;
+constexpr long long kChunkSteps = kTurnSpan;
 
 // Device-driven evolution of a step range in one CUDA graph (graph.cpp): a
 // WHILE conditional node whose body is kGraphUnroll Strang steps, with the
@@ -111,6 +117,7 @@ struct GraphSpec {
   const double* dt_dev = nullptr;  // per-step lengths on the device, or null for the uniform dt
   const unsigned* counts = nullptr;  // stored per-tile clause counts (launch_lp_counts), or null
   double* fold = nullptr;            // norm-fold slots (kFoldBytes), or null
+  bool any_angle = true;             // Pass::any_angle of every pass
   long long K = 0, k0 = 0, k1 = 0;
   int num_sms = 0;
   // graph scratch (graph_scratch_bytes): loop counter, kGraphUnroll + 1 P rows, kGraphUnroll B rows

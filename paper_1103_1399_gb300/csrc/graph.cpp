@@ -116,7 +116,7 @@ cudaError_t build_evolve_graph(const GraphSpec& s, cudaGraphExec_t* out) {
   e = captured_child([&]() -> cudaError_t {
     cudaError_t ec = cudaMemsetAsync(s.ctr, 0, sizeof(long long), cap.st);
     if (ec == cudaSuccess) ec = rows(0, 0, 1, 0, 0, nullptr);
-    build_passes(plan, 0, 1, 0, 0, passes);  // zero steps: the first low pass and the groups up
+    build_passes(plan, 0, 1, 0, 0, passes, s.any_angle);  // zero steps: the first low pass and the groups up
     return ec == cudaSuccess ? launch_all(lc, s, passes) : ec;
   });
   if (e != cudaSuccess) return e;
@@ -139,7 +139,7 @@ cudaError_t build_evolve_graph(const GraphSpec& s, cudaGraphExec_t* out) {
     e = capture_into(cap.st, body, [&]() -> cudaError_t {
       cudaError_t ec = rows(1, 1, kGraphUnroll, s.k0, kGraphUnroll, s.ctr);
       // kGraphUnroll merged steps: B rows 0.., P rows 1.. (build_passes' chunk convention)
-      build_passes(plan, -1, 1ll << 40, 0, kGraphUnroll, passes);
+      build_passes(plan, -1, 1ll << 40, 0, kGraphUnroll, passes, s.any_angle);
       number_low_passes(passes, 0);
       if (ec == cudaSuccess) ec = launch_all(lc, s, passes);
       if (ec == cudaSuccess) ec = launch_graph_advance(lc, s.ctr, kGraphUnroll, L * kGraphUnroll, h);
@@ -153,7 +153,7 @@ cudaError_t build_evolve_graph(const GraphSpec& s, cudaGraphExec_t* out) {
     e = captured_child([&]() -> cudaError_t {
       const long long off = L * kGraphUnroll;
       cudaError_t ec = rows(1, 1 + off, static_cast<int>(R), s.k0 + off, static_cast<int>(R), nullptr);
-      build_passes(plan, -1, 1ll << 40, 0, R, passes);
+      build_passes(plan, -1, 1ll << 40, 0, R, passes, s.any_angle);
       number_low_passes(passes, off);
       return ec == cudaSuccess ? launch_all(lc, s, passes) : ec;
     });
@@ -163,7 +163,7 @@ cudaError_t build_evolve_graph(const GraphSpec& s, cudaGraphExec_t* out) {
   // epilogue: the last step (B row of step k1 - 1, P row at position k1 - k0)
   e = captured_child([&]() -> cudaError_t {
     cudaError_t ec = rows(1, s.k1 - s.k0, 1, s.k1 - 1, 1, nullptr);
-    build_passes(plan, -1, 1, 0, 1, passes);  // one step, no first pass, ending in the last low pass
+    build_passes(plan, -1, 1, 0, 1, passes, s.any_angle);  // one step, no first pass, ending in the last low pass
     number_low_passes(passes, s.k1 - s.k0 - 1);
     return ec == cudaSuccess ? launch_all(lc, s, passes) : ec;
   });

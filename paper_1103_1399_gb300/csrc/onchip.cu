@@ -100,19 +100,22 @@ __device__ void warp_run(const RunArgs& A, unsigned char* smem) {
     cp_async_wait<kWarpRing - 1>();
     __syncwarp();
     const RotCoef c = rot_coef(s_ab + 2 * (j % kWarpRing));
-    const unsigned long long am1 = Inc<N>::add2_bits(c.a);
     if constexpr (N >= 2) x.template turn<0, (N >= 8 ? 3 : (N >= 4 ? 2 : 1))>(c, true);
+    for (bool again = c.twice;; again = false) {
 #pragma unroll
-    for (int b = 0; b < 5; ++b) {
-      if (b < n) {
-        const unsigned long long k = ((lane >> b) & 1) ? c.nb : c.b;
+      for (int b = 0; b < 5; ++b) {
+        if (b < n) {
+          const unsigned long long k = ((lane >> b) & 1) ? c.nb : c.b;
 #pragma unroll
-        for (int r = 0; r < N; ++r) {
-          const float2 s = x.at(r);
-          const float2 p = make_float2(__shfl_xor_sync(0xffffffffu, s.x, 1 << b), __shfl_xor_sync(0xffffffffu, s.y, 1 << b));
-          x.d[r] = fma2(k, p, c.tangent ? x.d[r] : fma2(am1, s, x.d[r]));
+          for (int r = 0; r < N; ++r) {
+            const float2 s = x.at(r);
+            const float2 p = make_float2(__shfl_xor_sync(0xffffffffu, s.x, 1 << b), __shfl_xor_sync(0xffffffffu, s.y, 1 << b));
+            x.d[r] = fma2(k, p, x.d[r]);
+          }
         }
       }
+      if (!again) break;
+      x.settle();
     }
     apply_rows<N>(x, e, s_p + (j % kWarpRing) * mp1);
     x.settle();

@@ -240,11 +240,12 @@ __device__ __forceinline__ double sched_s(const double* s_dev, long long K, long
 
 constexpr int kTableThreads = 256;
 
-// The rotation of step k in the kRowsTurn form (RotCoef): h = dt (1 - s)/2,
-// (a, b) = (1, tan h) where |tan h| <= 1, with flip when cos h < 0 (then the
-// factor per qubit is -1/sqrt(1 + b^2)), else (cos h, sin h); a, b as rounded to FP32.
+// The rotation of step k in the kRowsTurn form (RotCoef): h = dt (1 - s)/2 taken to
+// (-pi/2, pi/2] by a multiple of pi (flip: an odd one, which is a sign per qubit), in
+// `times` turns with b = tan(h / times), |b| <= 1, as rounded to FP32.
 struct Turn {
-  double h, a, b;
+  double h, b;
+  int times;
   bool flip;
 };
 __device__ __forceinline__ Turn turn_of(double dt, double s) {
@@ -252,15 +253,22 @@ __device__ __forceinline__ Turn turn_of(double dt, double s) {
   t.h = 0.5 * (dt * (1.0 - s));
   double sn, cs;
   sincos(t.h, &sn, &cs);
-  const bool tangent = fabs(sn) <= fabs(cs);
-  t.a = tangent ? 1.0 : static_cast<double>(static_cast<float>(cs));
-  t.b = static_cast<double>(static_cast<float>(tangent ? sn / cs : sn));
-  t.flip = tangent && cs < 0.0;
+  t.flip = cs < 0.0;
+  if (t.flip) {
+    sn = -sn;
+    cs = -cs;
+  }
+  t.times = fabs(sn) <= cs ? 1 : 2;
+  // tan(h / 2) = sin h / (1 + cos h)
+  t.b = static_cast<double>(static_cast<float>(t.times == 1 ? sn / cs : sn / (1.0 + cs)));
   return t;
 }
 
 // kRowsTurn: the sum over the steps [c0, c1) of the phase n (h + pi [flip]) that the
-// rotations leave out, by every thread of the block (FP64, fixed order).
+// rotations leave out, by every thread of the block (FP64, fixed order).  Position p
+// of a range takes it up when p is a multiple of kTurnSpan (for the steps since the
+// last one) or the end: the chunks of per-pass launches and of a launch graph's rows
+// agree on that.
 __device__ double turn_phase(double dt, const double* dt_dev, const double* s_dev, long long K, long long c0,
                              long long c1, int n) {
   if (!dt_dev && !s_dev && fabs(dt) <= 1.5)  // linear sweep, no flips: the closed form
@@ -300,11 +308,8 @@ __device__ __noinline__ float2 p_entry(double dt, const double* dt_dev, const do
   return make_float2(static_cast<float>(cs), static_cast<float>(-sn));
 }
 
-// Form kRowsBlock (rotation form): the row instead holds exp(-i dt (1 - s_k) q)
-// unscaled for q = 0..6, the rest zero: the per-block popcount phases of the
-// rotation form's 5- and 6-qubit Walsh-Hadamard sandwiches.  Form kRowsTurn:
-// entry 0 is (a, b) of turn_of, entry 1 the scale (a^2 + b^2)^(-n/2) = (1 + r) 2^-e
-// as (r, 2^-e), the rest zero; the phase e^(-inh) is part of the last P row.
+// Form kRowsTurn: entry 0 is (times, b) of turn_of, entry 1 the scale (1 +
+// b^2)^(-n times / 2) = (1 + r) 2^-e as (r, 2^-e), the rest zero.
 __device__ __noinline__ float2 b_entry(double dt, const double* dt_dev, const double* s_dev, long long K, long long k,
                                        int q, double scale, int form, int n) {
   const double s = sched_s(s_dev, K, k);
@@ -312,13 +317,9 @@ __device__ __noinline__ float2 b_entry(double dt, const double* dt_dev, const do
   if (form == kRowsTurn) {
     if (q > 1) return make_float2(0.f, 0.f);
     const Turn t = turn_of(dt, s);
-    if (q == 0) return make_float2(static_cast<float>(t.a), static_cast<float>(t.b));
-    const double lg = -0.5 * n * log2(t.a * t.a + t.b * t.b), e = rint(lg);
+    if (q == 0) return make_float2(static_cast<float>(t.times), static_cast<float>(t.b));
+    const double lg = -0.5 * n * t.times * log2(1.0 + t.b * t.b), e = rint(lg);
     return make_float2(static_cast<float>(exp2(lg - e) - 1.0), static_cast<float>(exp2(e)));
-  }
-  if (form == kRowsBlock) {
-    if (q > 6) return make_float2(0.f, 0.f);
-    scale = 1.0;
   }
   const double ph = dt * (1.0 - s) * static_cast<double>(q);
   double sn, cs;
@@ -356,22 +357,37 @@ __global__ void __launch_bounds__(kTableThreads)
 }
 
 // Rows for a launch graph: P positions p_first + j into rows dst_p0 + j of
-// prow (j < nprow), B rows of steps k_first + j into rows j of brow (j <
+// prow (j < nprow <= kTurnSpan), B rows of steps k_first + j into rows j of brow (j <
 // nbrow); with ctr non-null both starts are offset by *ctr (the graph's loop
 // counter, read by every thread; nothing here writes it).
-__global__ void graph_rows_kernel(float2* __restrict__ prow, int dst_p0, long long p_first, int nprow,
+__global__ void __launch_bounds__(kTableThreads)
+    graph_rows_kernel(float2* __restrict__ prow, int dst_p0, long long p_first, int nprow,
                                   float2* __restrict__ brow, long long k_first, int nbrow,
                                   const long long* __restrict__ ctr, int n, int m, double dt,
                                   const double* __restrict__ dt_dev, const double* __restrict__ s_dev, long long K,
                                   long long k0, long long k1, double scale, int form) {
   const long long off = ctr ? *ctr : 0;
   const long long np = static_cast<long long>(nprow) * (m + 1), nb = static_cast<long long>(nbrow) * (n + 1);
+  // the row (at most one) that takes up the phase the turns left out
+  int owed = -1;
+  double phase = 0.0;
+  if (form == kRowsTurn) {
+    for (int j = 0; j < nprow; ++j) {
+      const long long p = p_first + off + j;
+      if (p > 0 && (p % kTurnSpan == 0 || p == k1 - k0)) owed = j;
+    }
+    if (owed >= 0) {
+      const long long p = p_first + off + owed;
+      phase = turn_phase(dt, dt_dev, s_dev, K, k0 + (p - 1) / kTurnSpan * kTurnSpan, k0 + p, n);
+    }
+  }
   for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < np + nb;
        i += static_cast<long long>(gridDim.x) * blockDim.x) {
     if (i < np) {
       const long long j = i / (m + 1);
       const int e = static_cast<int>(i - j * (m + 1));
-      prow[(dst_p0 + j) * (m + 1) + e] = p_entry(dt, dt_dev, s_dev, K, k0, k1, p_first + off + j, e, form);
+      prow[(dst_p0 + j) * (m + 1) + e] =
+          p_entry(dt, dt_dev, s_dev, K, k0, k1, p_first + off + j, e, form, j == owed ? phase : 0.0);
     } else {
       const long long t = i - np;
       const long long j = t / (n + 1);
@@ -476,10 +492,10 @@ cudaError_t launch_graph_rows(const LaunchCtx& lc, float2* prow, int dst_p0, lon
                               const double* s_dev, long long K, long long k0, long long k1, int form,
                               const double* dt_dev) {
   const long long total = static_cast<long long>(nprow) * (m + 1) + static_cast<long long>(nbrow) * (n + 1);
-  long long grid = (total + 127) / 128;
+  long long grid = (total + kTableThreads - 1) / kTableThreads;
   if (grid > 2ll * lc.num_sms) grid = 2ll * lc.num_sms;
   if (grid < 1) grid = 1;
-  graph_rows_kernel<<<static_cast<unsigned>(grid), 128, 0, lc.stream>>>(
+  graph_rows_kernel<<<static_cast<unsigned>(grid), kTableThreads, 0, lc.stream>>>(
       prow, dst_p0, p_first, nprow, brow, k_first, nbrow, ctr, n, m, dt, dt_dev, s_dev, K, k0, k1,
       exp2(-static_cast<double>(n)), form);
   return cudaGetLastError();

@@ -8,6 +8,8 @@
 // step: phase group W B W, the other groups down, the low pass W P W (merging
 // the half phases of two steps), the other groups up: 2g-2 HBM round trips for
 // g groups.  n <= 14 runs entirely on chip.
+#include <algorithm>
+#include <cmath>
 #include <cstdlib>
 #include <map>
 #include <mutex>
@@ -199,13 +201,13 @@ static bool fits(const PassPlan& plan, int max_q) {
   return true;
 }
 
-void make_plan(int n, PassPlan& plan, int max_q) {
+void make_plan(int n, PassPlan& plan, int max_q, bool rotation) {
   if (n > kOnchipMaxBits && !env_overrides() && tuned_plan(n, plan) && fits(plan, max_q)) return;
-  make_default_plan(n, plan, max_q);
+  make_default_plan(n, plan, max_q, 0, rotation);
   plan.team = default_team(plan);
 }
 
-void make_default_plan(int n, PassPlan& plan, int max_q, int low) {
+void make_default_plan(int n, PassPlan& plan, int max_q, int low, bool rotation) {
   plan = PassPlan();
   plan.n = n;
   plan.onchip = n <= kOnchipMaxBits;
@@ -240,6 +242,7 @@ void make_default_plan(int n, PassPlan& plan, int max_q, int low) {
     }
     if (!ok || sum != rest) sizes.clear();
   }
+  const bool sizes_default = sizes.empty() && max_q >= 11;
   if (sizes.empty()) {
     const int ng = (rest + max_q - 1) / max_q;
     const int base = rest / ng, extra = rest % ng;
@@ -261,6 +264,14 @@ void make_default_plan(int n, PassPlan& plan, int max_q, int low) {
     const int q = plan.strided[0].q;
     plan.strided[0] = {L, q, L + q + 5};
     plan.strided[1] = {L + 5, q, L + 10};
+  }
+  // Rotation form, n = 26..29: a 10-bit group {L..L+4} + the top 5 bits (128-byte runs,
+  // 128 rows' pages per tile) and the 6 to 9 bits between, instead of two groups of 8 or
+  // 9: a 10-bit pass with its early copy moves 6.4 TB/s, a 9-bit one 5.5 (per step, n = 27
+  // 1137 -> 1081 us, n = 28 2321 -> 2170, n = 29 4626 -> 4539, n = 26 556 -> 549).
+  if (split && rotation && sizes_default && L == kLowBits && n >= 26 && n <= 29 && plan.strided.size() == 2) {
+    plan.strided[0] = {L, 10, n - 5};
+    plan.strided[1] = {L + 5, n - 5 - (L + 5), L + 10};
   }
   // Three groups at n = 33..34 (23..24 strided bits): contiguous 8-bit groups
   // put rows up to 512 MiB apart, 256 memory pages per tile.  Instead an 11-bit
@@ -291,7 +302,7 @@ void make_default_plan(int n, PassPlan& plan, int max_q, int low) {
 void narrow_low_pass(PassPlan& plan, int max_q) {
   if (plan.onchip || plan.low_bits == kLowBits) return;
   const int wk = plan.wht_kind;
-  make_default_plan(plan.n, plan, max_q, kLowBits);
+  make_default_plan(plan.n, plan, max_q, kLowBits, wk == kRotationForm);
   plan.wht_kind = wk;
   set_default_run_c(plan);
 }
@@ -322,7 +333,8 @@ void set_default_run_c(PassPlan& plan) {
 // step k is the strided groups' rotations, then the low pass's rotations and
 // the P phase at the boundary after step k (merged with the next step's first
 // half, or the last half at the end of the range): g round trips per step.
-static void build_rot_passes(const PassPlan& plan, long long k0, long long c0, long long c1, std::vector<Pass>& out) {
+static void build_rot_passes(const PassPlan& plan, long long k0, long long k1, long long c0, long long c1,
+                             std::vector<Pass>& out) {
   if (c0 == k0) out.push_back({kLpPhase, 0, 0, 0, 0, 0, 0, -1});
   for (long long k = c0; k < c1; ++k) {
     const int brow = static_cast<int>(k - c0);
@@ -330,16 +342,30 @@ static void build_rot_passes(const PassPlan& plan, long long k0, long long c0, l
       const Group& g = plan.strided[i];
       out.push_back({kSpRot, g.a, g.q, 0, plan.run_c[i], brow, g.a2});
     }
-    out.push_back({plan.low_bits == 12 ? kLpRot12 : kLpRot, 0, 0, static_cast<int>(k + 1 - c0), 0, brow, 0,
+    out.push_back({plan.low_bits == 12 ? kLpRot12 : kLpRot, k == k1 - 1 ? 1 : 0, 0, static_cast<int>(k + 1 - c0), 0, brow, 0,
                    static_cast<int>(k - k0)});
   }
 }
 
+bool small_angles(int n, double dt, const double* s_host, const double* dt_host, long long K, long long k0, long long k1) {
+  double h = 0.0;
+  if (!s_host && !dt_host) {
+    h = 0.5 * std::fabs(dt);  // |1 - s| < 1
+  } else {
+    for (long long k = k0; k < k1; ++k) {
+      const double s = s_host ? s_host[k] : (static_cast<double>(k) + 0.5) / static_cast<double>(K);
+      h = std::max(h, std::fabs(0.5 * (dt_host ? dt_host[k] : dt) * (1.0 - s)));
+    }
+  }
+  return h < 0.78 && -n * std::log2(std::cos(h)) < 0.49;
+}
+
 void build_passes(const PassPlan& plan, long long k0, long long k1, long long c0, long long c1,
-                  std::vector<Pass>& out) {
+                  std::vector<Pass>& out, bool any_angle) {
   out.clear();
   if (plan.wht_kind == kRotationForm) {
-    build_rot_passes(plan, k0, c0, c1, out);
+    build_rot_passes(plan, k0, k1, c0, c1, out);
+    for (Pass& p : out) p.any_angle = any_angle;
     return;
   }
   const int ng = static_cast<int>(plan.strided.size());
@@ -380,7 +406,7 @@ std::string describe_plan(const PassPlan& plan) {
            (team_plan(plan) ? "a cluster of 8 CTAs" : (plan.n <= 8 ? "one warp" : "one CTA")) + " (n=" + std::to_string(plan.n) + ")";
   const int ng = static_cast<int>(plan.strided.size());
   if (plan.wht_kind == kRotationForm) {
-    std::string d = "streaming, TMA loads, rotation form (H_B per 5-qubit block: W.diag.W); low pass bits [0," +
+    std::string d = "streaming, TMA loads, rotation form (H_B as one-qubit rotations); low pass bits [0," +
                     std::to_string(plan.low_bits) + ") R.P";
     for (int i = 0; i < ng; ++i) {
       const Group& g = plan.strided[i];

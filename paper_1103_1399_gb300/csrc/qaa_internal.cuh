@@ -50,16 +50,19 @@ enum PassKind : int {
   kSpW = 3,      // psi <- W_G psi over a strided group G
   kSpWBW = 4,    // psi <- W_G B(row) W_G psi over the phase group
   // Rotation form of exp(-i theta H_B) (variant 3): a product of one-qubit
-  // rotations, applied group by group, no change of basis.  TMA passes only.
-  kLpPhase = 5,  // psi <- P(prow) psi                     (first pass of a range)
-  kLpRot = 6,    // psi <- 2^-n P(prow) R_G1(brow) psi     (ends every step)
-  kSpRot = 7,    // psi <- R_G(brow) psi over a strided group (unnormalised by 2^q)
+  // rotations (RotCoef), applied group by group, no change of basis, the state in
+  // the gauge i^popcount between the passes of a range.  TMA passes only.
+  kLpPhase = 5,  // psi <- i^popcount P(prow) psi          (first pass of a range)
+  kLpRot = 6,    // psi <- P(prow) scale(brow) R_G1(brow) psi  (ends every step; the
+                 // last of a range, a = 1, also takes the gauge out)
+  kSpRot = 7,    // psi <- R_G(brow) psi over a strided group
   kLpRot12 = 8,  // kLpRot over bits 0..11: four 1024-amplitude tiles per warp quad
 };
 
 struct Pass {
   int kind;
   int a;      // strided passes: index bit of the group's lowest 5 active bits
+              // kLpRot, kLpRot12: 1 = the range's last
   int q;      // active bits (strided passes)
   int prow;   // phase-table row for P (low passes)
   int run_c;  // strided passes: 4 = 128-byte contiguous runs per tile row, 0 = default
@@ -69,6 +72,7 @@ struct Pass {
   // (-1 for the first pass of a range, -2 for no norm fold); selects the
   // norm-fold slots below
   int rel = -2;
+  bool any_angle = true;  // rotation form: whether the range has steps beyond small_angles()
 };
 
 // ---- norm fold ---------------------------------------------------------------
@@ -145,11 +149,11 @@ struct LaunchCtx {
   int num_sms;
 };
 
-// Phase rows for: the W.B.W form (B rows 2^-n exp(-i dt (1 - s_k) q), q = 0..n),
-// the 5- and 6-qubit sandwiches of the rotation form (exp(-i dt (1 - s_k) q), q =
-// 0..6, unscaled), one-qubit rotations (B entries 0 and 1: RotCoef; the phase that
-// the rotations leave out is part of the last P row; P entries e^(-i theta E) - 1).
-enum RowForm : int { kRowsWbw = 0, kRowsBlock = 1, kRowsTurn = 2 };
+// Phase rows for: the W.B.W form (B rows 2^-n exp(-i dt (1 - s_k) q), q = 0..n), one-
+// qubit rotations (B entries 0 and 1: RotCoef; the phase that the rotations leave out
+// is part of every kTurnSpan-th P row and the last; P entries e^(-i theta E) - 1).
+enum RowForm : int { kRowsWbw = 0, kRowsTurn = 2 };
+constexpr long long kTurnSpan = 1024;
 cudaError_t launch_init_uniform(const LaunchCtx& lc, float2* psi, int n);
 // Phase tables for steps c0 <= k < c1 of the range [k0, k1) of a K-step run:
 // c1-c0+1 P rows of m+1 entries and c1-c0 B rows of n+1 entries.

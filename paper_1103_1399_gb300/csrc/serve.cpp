@@ -341,6 +341,7 @@ cudaError_t issue_streaming(qaa_server* s, Req* r, cudaStream_t st) {
   if (e == cudaSuccess) e = qaa::launch_init_uniform(lc, r->psi, r->n);
   if (e == cudaSuccess && r->d_counts) e = qaa::launch_lp_counts(lc, r->d_counts, r->n, r->m, r->d_lp);
   const double dt = r->T / static_cast<double>(r->K);
+  const bool any_angle = !qaa::small_angles(r->n, dt, nullptr, nullptr, r->K, 0, r->K);
   char* team_work = r->d_team ? r->d_team + energy_bytes(r->n) : nullptr;
   if (r->d_team) {
     if (e == cudaSuccess) e = qaa::launch_hp_diag(lc, reinterpret_cast<uint16_t*>(r->d_team), r->n, r->m, r->d_lp);
@@ -359,6 +360,7 @@ cudaError_t issue_streaming(qaa_server* s, Req* r, cudaStream_t st) {
     gs.num_sms = s->num_sms;
     gs.counts = r->d_counts;
     gs.fold = r->d_fold;
+    gs.any_angle = any_angle;
     qaa::graph_scratch_split(r->d_tab, r->m, gs);
     if (e == cudaSuccess) e = qaa::build_evolve_graph(gs, &r->gexec);
     if (e == cudaSuccess) e = cudaGraphLaunch(r->gexec, st);
@@ -371,14 +373,14 @@ cudaError_t issue_streaming(qaa_server* s, Req* r, cudaStream_t st) {
   for (long long c0 = 0; e == cudaSuccess && c0 < r->K; c0 += r->chunk) {
     const long long c1 = std::min(r->K, c0 + r->chunk);
     e = qaa::launch_tables(lc, ptab, btab, r->n, r->m, dt, nullptr, r->K, 0, r->K, c0, c1,
-                           qaa::row_form(r->plan, r->d_team != nullptr));
+                           qaa::row_form(r->plan));
     if (r->d_team) {
       if (e == cudaSuccess)
         e = qaa::launch_team(lc, r->psi, r->n, r->m, reinterpret_cast<const uint16_t*>(r->d_team), ptab, btab,
                              static_cast<int>(c1 - c0), c0 == 0, team_work, r->d_fold, r->d_err);
       continue;
     }
-    qaa::build_passes(r->plan, 0, r->K, c0, c1, passes);
+    qaa::build_passes(r->plan, 0, r->K, c0, c1, passes, any_angle);
     for (const qaa::Pass& ps : passes) {
       if (e != cudaSuccess) break;
       e = qaa::launch_planned_pass(lc, r->plan, ps, r->psi, r->m, r->d_lp, ptab, btab, r->d_err, r->d_counts,

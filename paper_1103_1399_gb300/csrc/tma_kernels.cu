@@ -105,8 +105,8 @@ __host__ __device__ constexpr int tma_c(int q) { return (10 - q) > 3 ? (10 - q) 
 // [a1+5, a2), [a2+Q-5, n).  Q = 11 (C = 3, 512 threads): the sixth bit of the
 // layout-L stage is thread bit C, a lane bit, transformed by warp shuffles.
 // MODE 0: W over the group; 1: W B W (the phase group); 2: the one-qubit
-// rotations of exp(-i theta H_B) on the group's bits (rotation form: B row
-// entries 0..6 = exp(-i theta p)), unnormalised by 2^Q.
+// rotations of exp(-i theta H_B) on the group's bits (rotation form, RotCoef), all of
+// them with times = 1; 3: the same for any angle.
 //
 // Butterflies over lane bit LB: (u, w) <- (u + w, u - w) across the two lanes.
 template <int LB>
@@ -120,24 +120,40 @@ __device__ __forceinline__ void lane_wht(float2 (&v)[32], int lane) {
   }
 }
 
-// Layout-L stage over i bits 0..QB-1: registers hold i bits 0..4, a sixth bit
-// (QB = 6) is lane bit C.  MODE 2 applies the rotation-form sandwich over all
-// QB bits (its popcount counts the lane bit too).
-template <int QB, int C, int MODE>
-__device__ __forceinline__ void stage_l(float2 (&v)[32], const float2 (&rtab)[7], int lane) {
-  if constexpr (QB <= 5) {
-    if (MODE == 2) reg_rot<QB>(v, *reinterpret_cast<const float2(*)[6]>(&rtab)); else reg_wht<0, QB>(v);
-  } else {
-    static_assert(QB == 6 && C < 5, "a sixth layout-L bit must be a lane bit");
-    reg_wht<0, 5>(v);
-    lane_wht<C>(v, lane);
-    if (MODE == 2) {
-      const int hb = (lane >> C) & 1;
+// A turn (RotCoef) over lane bit LB.
+template <int LB, bool ANY>
+__device__ __forceinline__ void lane_turn(float2 (&v)[32], const RotCoef& c, int lane) {
+  const unsigned long long k = (lane >> LB) & 1 ? c.nb : c.b;
+  auto once = [&]() {
 #pragma unroll
-      for (int r = 0; r < 32; ++r) v[r] = cmul(v[r], rtab[__builtin_popcount(r) + hb]);
-      reg_wht<0, 5>(v);
-      lane_wht<C>(v, lane);
-    }
+    for (int r = 0; r < 32; ++r)
+      v[r] = fma2(k, make_float2(__shfl_xor_sync(0xffffffffu, v[r].x, 1 << LB), __shfl_xor_sync(0xffffffffu, v[r].y, 1 << LB)),
+                  v[r]);
+  };
+  once();
+  if (ANY && c.twice) once();
+}
+
+// Register bits [0, B): the turns of the rotation form (MODE 3: by any angle), or W.
+template <int B, int MODE>
+__device__ __forceinline__ void turn_or_wht(float2 (&v)[32], const RotCoef& rc) {
+  if constexpr (MODE == 3)
+    reg_turn<0, B>(v, rc);
+  else if constexpr (MODE == 2)
+    turn_once<0, B, 32, true>(v, rc);
+  else
+    reg_wht<0, B>(v);
+}
+
+// Layout-L stage over i bits 0..QB-1: registers hold i bits 0..4, a sixth bit
+// (QB = 6) is lane bit C.  MODE 2 and 3 turn the QB bits.
+template <int QB, int C, int MODE>
+__device__ __forceinline__ void stage_l(float2 (&v)[32], const RotCoef& rc, int lane) {
+  constexpr int RB = QB <= 5 ? QB : 5;
+  static_assert(QB <= 5 || (QB == 6 && C < 5), "a sixth layout-L bit must be a lane bit");
+  turn_or_wht<RB, MODE>(v, rc);
+  if constexpr (QB == 6) {
+    if (MODE >= 2) lane_turn<C, MODE == 3>(v, rc, lane); else lane_wht<C>(v, lane);
   }
 }
 
@@ -173,9 +189,8 @@ __global__ void __launch_bounds__(TmaGeom<Q, C>::NT, (TmaGeom<Q, C>::NT >= 512 ?
   if (WBW) {
     for (int i = tid; i <= n; i += blockDim.x) s_bt[i] = brow[i];
   }
-  float2 rtab[7];
-#pragma unroll
-  for (int p = 0; p < 7; ++p) rtab[p] = MODE == 2 ? brow[p] : make_float2(0.f, 0.f);
+  const float2 none[2] = {};
+  const RotCoef rc = rot_coef(MODE >= 2 ? brow : none);
   const int lane = tid & 31;
   __syncthreads();
   if (tid == 0 && static_cast<long long>(blockIdx.x) < ntiles) issue(blockIdx.x);
@@ -201,14 +216,14 @@ __global__ void __launch_bounds__(TmaGeom<Q, C>::NT, (TmaGeom<Q, C>::NT >= 512 ?
 #pragma unroll
       for (int r = 0; r < 32; ++r) v[r] = src[(r << QB) << C];
     }
-    if (MODE == 2) reg_rot<5>(v, *reinterpret_cast<const float2(*)[6]>(&rtab)); else reg_wht<0, 5>(v);  // i bits QB..QB+4
+    turn_or_wht<5, MODE>(v, rc);  // i bits QB..QB+4
     // Passes that store from layout L (plain W and the rotation form) are done
     // with the buffer once layout L is read: the next tile's copy starts there,
     // before the second butterfly stage, instead of after it (measured at
     // n = 30: plain 3.08 -> 2.83 ms, rotation with 128-byte runs 2.70 ms).  A
     // rotation pass with three 256-thread CTAs per SM ran slower with the early
     // copy (3.67 -> 4.22 ms) and keeps the late one.
-    constexpr bool kEarlyIssue = (MODE == 0 || (MODE == 2 && G::NT >= 512)) && QB > 0;
+    constexpr bool kEarlyIssue = (MODE == 0 || (MODE >= 2 && G::NT >= 512)) && QB > 0;
     auto issue_next = [&]() {
       __syncthreads();
       if (tid == 0) {
@@ -227,7 +242,7 @@ __global__ void __launch_bounds__(TmaGeom<Q, C>::NT, (TmaGeom<Q, C>::NT >= 512 ?
 #pragma unroll
       for (int r = 0; r < 32; ++r) v[r] = s_buf[sx_l + (r << C)];
       if (kEarlyIssue) issue_next();
-      stage_l<QB, C, MODE>(v, rtab, lane);  // i bits 0..QB-1
+      stage_l<QB, C, MODE>(v, rc, lane);  // i bits 0..QB-1
     }
     if (WBW) {
       // 2^-n exp(-i phi popcount(x)), x the full index
@@ -235,7 +250,7 @@ __global__ void __launch_bounds__(TmaGeom<Q, C>::NT, (TmaGeom<Q, C>::NT >= 512 ?
 #pragma unroll
       for (int r = 0; r < 32; ++r) v[r] = cmul(v[r], s_bt[pc0 + __popc(r)]);
       if (QB > 0) {
-        stage_l<QB, C, 0>(v, rtab, lane);
+        stage_l<QB, C, 0>(v, rc, lane);
         __syncthreads();
 #pragma unroll
         for (int r = 0; r < 32; ++r) s_buf[sx_l + (r << C)] = v[r];
@@ -281,15 +296,22 @@ __global__ void __launch_bounds__(TmaGeom<Q, C>::NT, (TmaGeom<Q, C>::NT >= 512 ?
 constexpr int kLpRowT = 33;
 constexpr int kLpSlotsT = 32 * kLpRowT;
 constexpr int kLpTmaWarps = 8;
+constexpr int kLpSplitWarps = 6;
 
+// split: 0 = one buffer per warp, the clause tables always there; 1 = a landing buffer
+// beside it; 2 = one buffer; 1 and 2 with the clause tables only when the counts are
+// not stored.
 struct LpTmaLayout {
-  size_t off_pt, off_warp, per_warp, off_bar, total;
-  __host__ __device__ explicit LpTmaLayout(int m) {
-    off_pt = 16u * static_cast<size_t>(m);
+  size_t off_pt, off_warp, off_act, per_warp, off_bar, total;
+  __host__ __device__ explicit LpTmaLayout(int m, int split = 0, bool stored = false) {
+    const int warps = split ? kLpSplitWarps : kLpTmaWarps;
+    const bool tables = !split || !stored;
+    off_pt = tables ? 16u * static_cast<size_t>(m) : 0u;
     off_warp = (off_pt + 8u * static_cast<size_t>(m + 1) + 127u) & ~static_cast<size_t>(127);
-    per_warp = (8u * kLpSlotsT + 8u * static_cast<size_t>(m + 16) + 127u) & ~static_cast<size_t>(127);
-    off_bar = off_warp + per_warp * kLpTmaWarps;
-    total = off_bar + 8u * kLpTmaWarps;
+    off_act = 8u * kLpSlotsT + (split == 1 ? 8192u : 0u);
+    per_warp = (off_act + (tables ? 8u * static_cast<size_t>(m + 16) : 0u) + 127u) & ~static_cast<size_t>(127);
+    off_bar = off_warp + per_warp * warps;
+    total = off_bar + 8u * warps;
   }
 };
 
@@ -315,8 +337,10 @@ __device__ __forceinline__ void xpose_y2x_t(float2 (&v)[32], float2* __restrict_
 }
 
 // KIND kLpPhase / kLpRot / kLpRot12: the rotation form (P alone; the
-// rotations of bits 0..9, or 0..11 with warp quads, then 2^-n P), with B row
-// entries 0..5 = exp(-i theta p).
+// rotations of bits 0..9, or 0..11 with warp quads, then their scale and P), P rows
+// as e^(-i theta E) - 1 (ANY: steps with two turns or a scale below 1/sqrt 2 among
+// them; as a branch of the one kernel they cost 200 bytes of spills).  The first pass of a range brings the state into the gauge
+// i^popcount, the last (LAST) takes it out: exact.
 // Stored per-tile counts: load_counts (device_common.cuh).
 
 // Warp quads (kLpRot12): warps 4k..4k+3 of a CTA sync on named barrier 1 + k
@@ -339,50 +363,46 @@ __device__ __forceinline__ void quad_sync(int quad) {
     asm volatile("bar.sync 1, 128;" ::: "memory");
 }
 
-// exp(-i theta H_B) on index bits 10 and 11 of four 1024-amplitude tiles held
-// in the quad's shared buffers (tile k of the quad = bits 10..11 equal to k):
-// W diag(exp(-i theta popcount)) W on the two bits, up to the factor 4.
-__device__ __forceinline__ void quad_rot2(float2* const (&b)[4], const float2 (&tab)[6], int t) {
+// The turns of index bits 10 and 11 over four 1024-amplitude tiles held in the
+// quad's shared buffers (tile k of the quad = bits 10..11 equal to k).
+__device__ __forceinline__ void quad_turn2(float2* const (&b)[4], const RotCoef& c, int t) {
 #pragma unroll 2
   for (int o = t; o < 1024; o += 128) {
-    float2 a0 = b[0][o], a1 = b[1][o], a2 = b[2][o], a3 = b[3][o];
-    butterfly(a0, a1);
-    butterfly(a2, a3);
-    butterfly(a0, a2);
-    butterfly(a1, a3);
-    a0 = cmul(a0, tab[0]);
-    a1 = cmul(a1, tab[1]);
-    a2 = cmul(a2, tab[1]);
-    a3 = cmul(a3, tab[2]);
-    butterfly(a0, a1);
-    butterfly(a2, a3);
-    butterfly(a0, a2);
-    butterfly(a1, a3);
-    b[0][o] = a0;
-    b[1][o] = a1;
-    b[2][o] = a2;
-    b[3][o] = a3;
+    float2 v[4] = {b[0][o], b[1][o], b[2][o], b[3][o]};
+    reg_turn<0, 2>(v, c);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) b[k][o] = v[k];
   }
 }
 
-template <int KIND>
-__global__ void __launch_bounds__(kLpTmaWarps * 32, 2)
+//
+// SPLIT (the rotation form's merged passes): six warps per CTA.  1, while the state
+// fits in L2: a landing buffer beside the transposes', and the next tile's copy starts as
+// soon as this one is in registers: n = 24 56 -> 47 us.  2, beyond it: the copy starts
+// after this tile's arithmetic, and 12 instead of 16 warps per SM: more reads in flight
+// among the writes make DRAM slower, not faster (n = 30: 2.99 ms with the early copy or
+// with 16 warps, 2.83 ms so; n = 26: 194 -> 182 us).
+// The grid does not depend on the shared memory, so that counts stored or not give
+// the same partial sums of the norm fold.
+template <int KIND, bool LAST = false, bool ANY = false, int SPLIT = 0>
+__global__ void __launch_bounds__((SPLIT ? kLpSplitWarps : kLpTmaWarps) * 32, 2)
     lp_tma_kernel(float2* __restrict__ psi, int m, const ClauseLP* __restrict__ cl, const float2* __restrict__ prow,
-                  const float2* __restrict__ brow, int n, long long ntiles, int* __restrict__ err,
+                  const float2* __restrict__ brow, long long ntiles, int* __restrict__ err,
                   const unsigned* __restrict__ counts, const NormFold nf) {
   constexpr bool kRegLow = KIND != kLpFirst && KIND != kLpPhase;  // phase applied in layout Y
   extern __shared__ __align__(1024) unsigned char smem[];
-  const LpTmaLayout L(m);
+  const LpTmaLayout L(m, SPLIT, counts != nullptr);
+  constexpr int kWarps = SPLIT ? kLpSplitWarps : kLpTmaWarps;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   ClauseLP* s_cl = reinterpret_cast<ClauseLP*>(smem);
   float2* s_pt = reinterpret_cast<float2*>(smem + L.off_pt);
   unsigned char* wbase = smem + L.off_warp + L.per_warp * warp;
   float2* s_buf = reinterpret_cast<float2*>(wbase);  // dense tile, then padded transposes
-  uint2* s_act = reinterpret_cast<uint2*>(wbase + 8u * kLpSlotsT);
+  uint2* s_act = reinterpret_cast<uint2*>(wbase + L.off_act);
   uint64_t* s_bar = reinterpret_cast<uint64_t*>(smem + L.off_bar) + warp;
-
-  const long long step = static_cast<long long>(gridDim.x) * kLpTmaWarps;
-  const long long first = static_cast<long long>(blockIdx.x) * kLpTmaWarps + warp;
+  float2* s_land = SPLIT == 1 ? reinterpret_cast<float2*>(wbase + 8u * kLpSlotsT) : s_buf;  // where the tile arrives
+  const long long step = static_cast<long long>(gridDim.x) * kWarps;
+  const long long first = static_cast<long long>(blockIdx.x) * kWarps + warp;
   if (lane == 0) {
     mbar_init(s_bar, 1);
     fence_mbar_init();
@@ -390,22 +410,25 @@ __global__ void __launch_bounds__(kLpTmaWarps * 32, 2)
   __syncwarp();
   if (lane == 0 && first < ntiles) {
     mbar_expect_tx(s_bar, 8192u);
-    bulk_load(s_buf, psi + (first << kLowBits), 8192u, s_bar);
+    bulk_load(s_land, psi + (first << kLowBits), 8192u, s_bar);
   }
-  for (int i = threadIdx.x; i < m; i += blockDim.x) s_cl[i] = cl[i];
-  // the rotation form's last pass of a step also removes the 2^n of its rotations (exact)
+  const bool stored = kRegLow && counts != nullptr;
+  if (!SPLIT || !stored) {
+    for (int i = threadIdx.x; i < m; i += blockDim.x) s_cl[i] = cl[i];
+  }
   constexpr bool kRot = KIND == kLpRot || KIND == kLpRot12;
   constexpr bool kQuad = KIND == kLpRot12;
-  // and every merged pass folds in the norm correction of the previous step
+  constexpr bool kMinus1 = kRot || KIND == kLpPhase;
+  // every merged pass folds in the norm correction of the previous step; the
+  // rotation form's row 1 + z becomes (1 + k) (1 + z) with the scale of the turns
   const float fd = fold_factor_block(nf);
-  const float psc = kRot ? __int_as_float((127 - n) << 23) : 1.0f;  // 2^-n exactly (n <= 34)
+  __shared__ float2 s_row[2];  // read again for every tile: registers are short
+  if (kRot && threadIdx.x < 2) s_row[threadIdx.x] = brow[threadIdx.x];
+  const float rs = kRot ? brow[1].x : 0.f, k1 = fmaf(rs, fd, rs + fd);
   for (int i = threadIdx.x; i <= m; i += blockDim.x) {
     const float2 pv = prow[i];
-    s_pt[i] = fold_apply(make_float2(pv.x * psc, pv.y * psc), fd);
+    s_pt[i] = kRot ? make_float2(fmaf(k1, pv.x, pv.x) + k1, fmaf(k1, pv.y, pv.y)) : (kMinus1 ? pv : fold_apply(pv, fd));
   }
-  float2 rtab[6];
-#pragma unroll
-  for (int p = 0; p < 6; ++p) rtab[p] = kRot ? brow[p] : make_float2(0.f, 0.f);
   // kLpRot12: the quad's four tile buffers (tile first + k of the quad in warp 4q + k's buffer)
   const int quad = warp >> 2;
   float2* qbuf[4];
@@ -416,7 +439,6 @@ __global__ void __launch_bounds__(kLpTmaWarps * 32, 2)
 
   int nconst = 0, npad = 0;
   unsigned pl[kPlanes];
-  const bool stored = kRegLow && counts != nullptr;
   if (first < ntiles) {
     if (stored) {
       load_counts(counts, first, lane, pl, nconst);
@@ -436,25 +458,47 @@ __global__ void __launch_bounds__(kLpTmaWarps * 32, 2)
     }
     if (kQuad) {
       // all four tiles are in (the barrier above): bits 10..11 across them
-      quad_rot2(qbuf, rtab, threadIdx.x & 127);
+      quad_turn2(qbuf, rot_coef(s_row), threadIdx.x & 127);
       fence_proxy_async();  // these writes precede the next bulk copies into the buffers
       quad_sync(quad);
     }
     float2 v[32];
     {
-      const float2* src = s_buf + lane;
+      const float2* src = s_land + lane;
 #pragma unroll
       for (int r = 0; r < 32; ++r) v[r] = src[32 * r];
     }
     __syncwarp();
+    const long long tn = tile + step;
+    auto next = [&]() {
+      if (lane == 0 && tn < ntiles) {
+        fence_proxy_async();
+        mbar_expect_tx(s_bar, 8192u);
+        bulk_load(s_land, psi + (tn << kLowBits), 8192u, s_bar);
+      }
+    };
+    if (SPLIT == 1) next();
     if (KIND == kLpPhase) {
-      apply_p_phase(v, pl, nconst, s_pt);
+      apply_p_phase<true>(v, pl, nconst, s_pt);
+      const int pc = __popcll(tile) + __popc(lane);
+#pragma unroll
+      for (int r = 0; r < 32; ++r) v[r] = times_i(v[r], pc + __popc(r));
     } else if (kRot) {
-      reg_rot<5>(v, rtab);
+      turn_or_wht<5, ANY ? 3 : 2>(v, rot_coef(s_row));
       xpose_x2y_t(v, s_buf, lane);
-      reg_rot<5>(v, rtab);
-      apply_p_phase(v, pl, nconst, s_pt);
+      if (ANY) {
+        const unsigned long long pw = f2_bits(make_float2(s_row[1].y, s_row[1].y));  // 2^-e
+#pragma unroll
+        for (int r = 0; r < 32; ++r) v[r] = mul2(pw, v[r]);
+      }
+      turn_or_wht<5, ANY ? 3 : 2>(v, rot_coef(s_row));
+      apply_p_phase<true>(v, pl, nconst, s_pt);
       xpose_y2x_t(v, s_buf, lane);
+      if (LAST) {
+        const int pc = __popcll(tile) + __popc(lane);
+#pragma unroll
+        for (int r = 0; r < 32; ++r) v[r] = times_i(v[r], -(pc + __popc(r)));
+      }
     } else if (KIND == kLpFirst) {
       apply_p_phase(v, pl, nconst, s_pt);
       reg_wht<0, 5>(v);
@@ -470,15 +514,10 @@ __global__ void __launch_bounds__(kLpTmaWarps * 32, 2)
       xpose_y2x_t(v, s_buf, lane);
       if (KIND == kLpMerge) reg_wht<0, 5>(v);
     }
-    const long long tn = tile + step;
-    if (lane == 0 && tn < ntiles) {
-      fence_proxy_async();
-      mbar_expect_tx(s_bar, 8192u);
-      bulk_load(s_buf, psi + (tn << kLowBits), 8192u, s_bar);
-    }
+    if (SPLIT != 1) next();
     float2* g = psi + (tile << kLowBits) + lane;
 #pragma unroll
-    for (int r = 0; r < 32; ++r) g[32 * r] = v[r];
+    for (int r = 0; r < 32; ++r) __stcs(&g[32 * r], v[r]);
     if (nf.out) nacc = df_add1(nacc, tile_norm(v));
     if (tn < ntiles) {
       if (stored) {
@@ -662,7 +701,8 @@ static cudaError_t launch_sp_tma_c(const LaunchCtx& lc, float2* psi, int n, int 
                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
   const long long ntiles = 1ll << (n - Q - C);
-  auto kern = mode == 1 ? sp_tma_kernel<Q, C, 1> : (mode == 2 ? sp_tma_kernel<Q, C, 2> : sp_tma_kernel<Q, C, 0>);
+  auto kern = mode == 1 ? sp_tma_kernel<Q, C, 1>
+                        : (mode == 2 ? sp_tma_kernel<Q, C, 2> : (mode == 3 ? sp_tma_kernel<Q, C, 3> : sp_tma_kernel<Q, C, 0>));
   cudaError_t e = allow_smem(reinterpret_cast<const void*>(kern), G::smem);
   if (e != cudaSuccess) return e;
   int occ = 0;
@@ -811,26 +851,48 @@ cudaError_t launch_lp_counts(const LaunchCtx& lc, unsigned* counts, int n, int m
   return cudaGetLastError();
 }
 
-template <int KIND>
+template <int KIND, bool LAST = false, bool ANY = false, int SPLIT = 0>
 static cudaError_t launch_lp_tma(const LaunchCtx& lc, float2* psi, int n, int m, const ClauseLP* cl,
                                  const float2* prow, const float2* brow, int* err, const unsigned* counts,
                                  const NormFold& nf) {
   const long long ntiles = 1ll << (n - kLowBits);
-  const LpTmaLayout L(m);
-  auto kern = lp_tma_kernel<KIND>;
-  cudaError_t e = allow_smem(reinterpret_cast<const void*>(kern), LpTmaLayout(QAA_MAX_CLAUSES_DEV).total);
+  const LpTmaLayout L(m, SPLIT, counts != nullptr);
+  constexpr int kWarps = SPLIT ? kLpSplitWarps : kLpTmaWarps;
+  auto kern = lp_tma_kernel<KIND, LAST, ANY, SPLIT>;
+  cudaError_t e = allow_smem(reinterpret_cast<const void*>(kern), LpTmaLayout(QAA_MAX_CLAUSES_DEV, SPLIT, false).total);
   if (e != cudaSuccess) return e;
-  int occ = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kLpTmaWarps * 32, L.total);
-  if (e != cudaSuccess) return e;
-  if (occ < 1) occ = 1;
+  int occ = 2;
+  if (!SPLIT) {
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kWarps * 32, L.total);
+    if (e != cudaSuccess) return e;
+    if (occ < 1) occ = 1;
+  }
   long long grid = static_cast<long long>(occ) * lc.num_sms;
-  const long long need = (ntiles + kLpTmaWarps - 1) / kLpTmaWarps;
+  const long long need = (ntiles + kWarps - 1) / kWarps;
   if (grid > need) grid = need;
   if (grid > kFoldSlot - 1) grid = kFoldSlot - 1;  // one norm-fold partial per CTA
-  kern<<<static_cast<unsigned>(grid), kLpTmaWarps * 32, L.total, lc.stream>>>(psi, m, cl, prow, brow, n, ntiles,
+  kern<<<static_cast<unsigned>(grid), kWarps * 32, L.total, lc.stream>>>(psi, m, cl, prow, brow, ntiles,
                                                                               err, counts, nf);
   return cudaGetLastError();
+}
+
+template <int KIND>
+static cudaError_t launch_lp_rot(const LaunchCtx& lc, const Pass& p, float2* psi, int n, int m, const ClauseLP* cl,
+                                 const float2* prow, const float2* brow, int* err, const unsigned* counts,
+                                 const NormFold& nf) {
+  if (p.any_angle)
+    return p.a ? launch_lp_tma<KIND, true, true>(lc, psi, n, m, cl, prow, brow, err, counts, nf)
+               : launch_lp_tma<KIND, false, true>(lc, psi, n, m, cl, prow, brow, err, counts, nf);
+  if constexpr (KIND == kLpRot) {
+    if (n >= 26)
+      return p.a ? launch_lp_tma<KIND, true, false, 2>(lc, psi, n, m, cl, prow, brow, err, counts, nf)
+                 : launch_lp_tma<KIND, false, false, 2>(lc, psi, n, m, cl, prow, brow, err, counts, nf);
+    return p.a ? launch_lp_tma<KIND, true, false, 1>(lc, psi, n, m, cl, prow, brow, err, counts, nf)
+               : launch_lp_tma<KIND, false, false, 1>(lc, psi, n, m, cl, prow, brow, err, counts, nf);
+  } else {
+    return p.a ? launch_lp_tma<KIND, true>(lc, psi, n, m, cl, prow, brow, err, counts, nf)
+               : launch_lp_tma<KIND>(lc, psi, n, m, cl, prow, brow, err, counts, nf);
+  }
 }
 
 cudaError_t launch_pass_tma(const LaunchCtx& lc, const Pass& p, float2* psi, int n, int m, const ClauseLP* cl,
@@ -844,14 +906,15 @@ cudaError_t launch_pass_tma(const LaunchCtx& lc, const Pass& p, float2* psi, int
     case kLpMerge: return launch_lp_tma<kLpMerge>(lc, psi, n, m, cl, prow, nullptr, err, counts, nf);
     case kLpLast: return launch_lp_tma<kLpLast>(lc, psi, n, m, cl, prow, nullptr, err, counts, nf);
     case kLpPhase: return launch_lp_tma<kLpPhase>(lc, psi, n, m, cl, prow, nullptr, err, nullptr, nf);
-    case kLpRot: return launch_lp_tma<kLpRot>(lc, psi, n, m, cl, prow, brow, err, counts, nf);
+    case kLpRot:
+      return launch_lp_rot<kLpRot>(lc, p, psi, n, m, cl, prow, brow, err, counts, nf);
     case kLpRot12:
       if (n < 12) return cudaErrorInvalidValue;
-      return launch_lp_tma<kLpRot12>(lc, psi, n, m, cl, prow, brow, err, counts, nf);
+      return launch_lp_rot<kLpRot12>(lc, p, psi, n, m, cl, prow, brow, err, counts, nf);
     case kSpW:
     case kSpWBW:
     case kSpRot: {
-      const int wbw = p.kind == kSpWBW ? 1 : (p.kind == kSpRot ? 2 : 0);
+      const int wbw = p.kind == kSpWBW ? 1 : (p.kind == kSpRot ? (p.any_angle ? 3 : 2) : 0);
       switch (p.q) {
         case 5: return launch_sp_tma<5>(lc, psi, n, p.a, p.a2, wbw, brow, err, c_req);
         case 6: return launch_sp_tma<6>(lc, psi, n, p.a, p.a2, wbw, brow, err, c_req);
