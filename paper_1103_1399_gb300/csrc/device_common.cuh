@@ -396,6 +396,11 @@ __device__ __forceinline__ void energies(int (&e)[32], const uint2* __restrict__
 }
 
 
+// Overlapped launches (launch_overlapped): let the next kernel's blocks in as soon as
+// there is room, and wait until the kernel before this one is complete.
+__device__ __forceinline__ void let_next_in() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // The device's global nanosecond timer (the PTX special register %globaltimer).
 __device__ __forceinline__ unsigned long long global_ns() {
   unsigned long long t;

@@ -354,6 +354,8 @@ qaa_status evolve_impl(qaa_ctx* h, void* psi, double dt, long long K, long long 
   float2* ptab = h->d_tab;
   float2* btab = h->d_tab + static_cast<size_t>(chunk + 1) * prow;
   const qaa::LaunchCtx lc = lctx(h);
+  qaa::LaunchCtx pass_lc = lc;
+  pass_lc.overlap = qaa::overlap_passes(h->n);
   float2* p = static_cast<float2*>(psi);
   std::vector<qaa::Pass> passes;
   ProfSpan span(graph ? h : nullptr, QAA_K_GRAPH);
@@ -379,7 +381,7 @@ qaa_status evolve_impl(qaa_ctx* h, void* psi, double dt, long long K, long long 
       const unsigned* counts = stored_counts(h);
       for (const qaa::Pass& ps : passes)
         QAA_CK(timed(h, prof_kind(ps.kind), [&] {
-          return qaa::launch_planned_pass(lc, h->plan, ps, p, h->m, h->d_lp, ptab, btab, h->d_err, counts,
+          return qaa::launch_planned_pass(pass_lc, h->plan, ps, p, h->m, h->d_lp, ptab, btab, h->d_err, counts,
                                           h->d_fold);
         }));
     }

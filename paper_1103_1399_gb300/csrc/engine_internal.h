@@ -100,6 +100,12 @@ cudaError_t launch_planned_pass(const LaunchCtx& lc, const PassPlan& plan, const
                                 const ClauseLP* cl, const float2* ptab, const float2* btab, int* err,
                                 const unsigned* counts = nullptr, double* fold = nullptr);
 
+// Whether the passes' launches overlap (LaunchCtx::overlap): while the state fits in L2
+// and a pass takes tens of microseconds (n = 23: 55.4 -> 52.3 us per step).  Beyond, the
+// next pass's blocks take the room of this one's last and the passes run slower (n = 26
+// 538 -> 543 us, n = 30 8.7 -> 9.3 ms).
+inline bool overlap_passes(int n) { return n < 26; }
+
 constexpr long long kChunkSteps = kTurnSpan;
 
 // Device-driven evolution of a step range in one CUDA graph (graph.cpp): a

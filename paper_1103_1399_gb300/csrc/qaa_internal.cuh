@@ -147,7 +147,27 @@ __host__ __device__ inline NormFold fold_for(double* slots, const Pass& p, int F
 struct LaunchCtx {
   cudaStream_t stream;
   int num_sms;
+  bool overlap = false;  // the streaming passes' launches may overlap (launch_overlapped)
 };
+
+// A launch whose blocks may become resident while the kernel before it on the
+// stream drains; the kernel waits for that one's completion itself
+// (griddepcontrol.wait, before it touches anything another kernel writes).
+template <class... P, class... A>
+inline cudaError_t launch_overlapped(const LaunchCtx& lc, void (*kern)(P...), unsigned grid, unsigned block, size_t smem,
+                                     A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = lc.stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = lc.overlap ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
 
 // Phase rows for: the W.B.W form (B rows 2^-n exp(-i dt (1 - s_k) q), q = 0..n), one-
 // qubit rotations (B entries 0 and 1: RotCoef; the phase that the rotations leave out

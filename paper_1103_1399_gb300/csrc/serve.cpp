@@ -335,7 +335,7 @@ cudaError_t mark_start(qaa_server* s, Req* r, cudaStream_t st) {
 // a team of CTAs (one launch per 1024 steps), one launch graph for the whole run,
 // or one launch per pass.
 cudaError_t issue_streaming(qaa_server* s, Req* r, cudaStream_t st) {
-  const qaa::LaunchCtx lc{st, s->num_sms};
+  const qaa::LaunchCtx lc{st, s->num_sms}, pass_lc{st, s->num_sms, qaa::overlap_passes(r->n)};
   cudaError_t e = mark_start(s, r, st);
   if (e == cudaSuccess) e = upload_tables(s, r, st);
   if (e == cudaSuccess) e = qaa::launch_init_uniform(lc, r->psi, r->n);
@@ -383,7 +383,7 @@ cudaError_t issue_streaming(qaa_server* s, Req* r, cudaStream_t st) {
     qaa::build_passes(r->plan, 0, r->K, c0, c1, passes, any_angle);
     for (const qaa::Pass& ps : passes) {
       if (e != cudaSuccess) break;
-      e = qaa::launch_planned_pass(lc, r->plan, ps, r->psi, r->m, r->d_lp, ptab, btab, r->d_err, r->d_counts,
+      e = qaa::launch_planned_pass(pass_lc, r->plan, ps, r->psi, r->m, r->d_lp, ptab, btab, r->d_err, r->d_counts,
                                    r->d_fold);
     }
   }

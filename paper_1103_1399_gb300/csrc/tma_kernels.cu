@@ -181,10 +181,12 @@ __global__ void __launch_bounds__(TmaGeom<Q, C>::NT, (TmaGeom<Q, C>::NT >= 512 ?
                 static_cast<int>(T >> (lo_bits + mid_bits)), s_bar);
   };
 
+  let_next_in();
   if (tid == 0) {
     mbar_init(s_bar, 1);
     fence_mbar_init();
   }
+  wait_previous();
   constexpr bool WBW = MODE == 1;
   if (WBW) {
     for (int i = tid; i <= n; i += blockDim.x) s_bt[i] = brow[i];
@@ -403,11 +405,13 @@ __global__ void __launch_bounds__((SPLIT ? kLpSplitWarps : kLpTmaWarps) * 32, 2)
   float2* s_land = SPLIT == 1 ? reinterpret_cast<float2*>(wbase + 8u * kLpSlotsT) : s_buf;  // where the tile arrives
   const long long step = static_cast<long long>(gridDim.x) * kWarps;
   const long long first = static_cast<long long>(blockIdx.x) * kWarps + warp;
+  let_next_in();
   if (lane == 0) {
     mbar_init(s_bar, 1);
     fence_mbar_init();
   }
   __syncwarp();
+  wait_previous();
   if (lane == 0 && first < ntiles) {
     mbar_expect_tx(s_bar, 8192u);
     bulk_load(s_land, psi + (first << kLowBits), 8192u, s_bar);
@@ -711,8 +715,7 @@ static cudaError_t launch_sp_tma_c(const LaunchCtx& lc, float2* psi, int n, int 
   if (occ < 1) occ = 1;
   long long grid = static_cast<long long>(occ) * lc.num_sms;
   if (grid > ntiles) grid = ntiles;
-  kern<<<static_cast<unsigned>(grid), G::NT, G::smem, lc.stream>>>(psi, map, n, a1, a2, brow, ntiles, err);
-  return cudaGetLastError();
+  return launch_overlapped(lc, kern, static_cast<unsigned>(grid), G::NT, G::smem, psi, map, n, a1, a2, brow, ntiles, err);
 }
 
 // The correlation pass over the bits [a, a+5) and [a2, a2+q-5) (a2 = a + 5 for
@@ -871,9 +874,8 @@ static cudaError_t launch_lp_tma(const LaunchCtx& lc, float2* psi, int n, int m,
   const long long need = (ntiles + kWarps - 1) / kWarps;
   if (grid > need) grid = need;
   if (grid > kFoldSlot - 1) grid = kFoldSlot - 1;  // one norm-fold partial per CTA
-  kern<<<static_cast<unsigned>(grid), kWarps * 32, L.total, lc.stream>>>(psi, m, cl, prow, brow, ntiles,
-                                                                              err, counts, nf);
-  return cudaGetLastError();
+  return launch_overlapped(lc, kern, static_cast<unsigned>(grid), kWarps * 32, L.total, psi, m, cl, prow, brow, ntiles, err,
+                           counts, nf);
 }
 
 template <int KIND>
