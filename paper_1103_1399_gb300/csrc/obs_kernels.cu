@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(kObsWarps * 32)
   __syncthreads();
   const int N = n < kLowBits ? (1 << n) : (1 << kLowBits);  // amplitudes per tile that exist
   double d_norm = 0.0, d_hp = 0.0, d_gp = 0.0, d_gc = 0.0, d_corr = 0.0;
-  for (long long tile = static_cast<long long>(blockIdx.x) * kObsWarps + warp; tile < ntiles;
+  for (long long tile = static_cast<long long>(warp) * gridDim.x + blockIdx.x; tile < ntiles;
        tile += static_cast<long long>(gridDim.x) * kObsWarps) {
     const float2* g = psi + (static_cast<unsigned long long>(tile) << kLowBits);
     float2 v[32];
@@ -306,7 +306,7 @@ __global__ void __launch_bounds__(kObsWarps * 32, 2)
   uint64_t* s_bar = reinterpret_cast<uint64_t*>(smem + L.off_bar) + warp;
   double* s_red = reinterpret_cast<double*>(smem + L.off_red);
   const long long step = static_cast<long long>(gridDim.x) * kObsWarps;
-  const long long first = static_cast<long long>(blockIdx.x) * kObsWarps + warp;
+  const long long first = static_cast<long long>(warp) * gridDim.x + blockIdx.x;  // a small state's tiles on many SMs
   if (lane == 0) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(obs_smem(s_bar)), "r"(1) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -415,31 +415,36 @@ __global__ void __launch_bounds__(256)
 }
 
 // result[0..4] = norm, <H_P>, ground, count, C.  Regions 0..4 come from the low
-// kernel; regions 5.. are the strided correlation kernels (added to C).  With
-// stamp, the device time at the end (global_ns) is written there.
-__global__ void __launch_bounds__(256)
+// kernel; regions 5.. are the strided correlation kernels (added to C).  One warp
+// per quantity, each in a fixed order (five block-wide trees one after the other took
+// 13.8 us, most of a small state's observables).  err (not null): the error word,
+// written to result[5] beside them.  result may be pinned host memory.  With stamp, the
+// device time at the end (global_ns) is written there.
+__global__ void __launch_bounds__(32 * kObsQuant)
     obs_reduce_kernel(const double* __restrict__ partials, int nparts, int nregions, double* __restrict__ result,
-                      unsigned long long* __restrict__ stamp) {
-  __shared__ double s[256];
-  for (int q = 0; q < kObsQuant; ++q) {
-    double t = 0.0;
-    const int last = (q == kObsQuant - 1) ? nregions : q + 1;
-    for (int reg = q; reg < last; ++reg) {
-      for (int i = threadIdx.x; i < nparts; i += blockDim.x) t += partials[static_cast<size_t>(reg) * nparts + i];
-    }
-    s[threadIdx.x] = t;
-    __syncthreads();
-    for (int h = blockDim.x >> 1; h > 0; h >>= 1) {
-      if (static_cast<int>(threadIdx.x) < h) s[threadIdx.x] += s[threadIdx.x + h];
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) result[q] = s[0];
-    __syncthreads();
+                      const int* __restrict__ err, unsigned long long* __restrict__ stamp) {
+  const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int last = (q == kObsQuant - 1) ? nregions : q + 1;
+  double t = 0.0;
+  for (int reg = q; reg < last; ++reg) {
+    double u = 0.0;
+#pragma unroll 4
+    for (int i = lane; i < nparts; i += 32) u += partials[static_cast<size_t>(reg) * nparts + i];
+    t += u;
   }
-  if (stamp && threadIdx.x == 0) *stamp = global_ns();
+  t = warp_sum(t);
+  if (lane == 0) result[q] = t;
+  if (threadIdx.x == 0) {
+    if (err) result[5] = static_cast<double>(*err);
+    if (stamp) *stamp = global_ns();
+  }
 }
 
-static int obs_grid(int num_sms) { return 2 * num_sms; }
+// CTAs (and partials per region): two per SM, or one per tile of a small state.
+static int obs_grid(int num_sms, int n = 64) {
+  const int most = 2 * num_sms;
+  return n <= kLowBits ? 1 : (n - kLowBits < 12 && (1 << (n - kLowBits)) < most ? 1 << (n - kLowBits) : most);
+}
 
 // Correlation passes over bits [10, n): contiguous groups of 5..10 bits (as
 // even as possible) on the TMA tile passes, else groups of at most 5 bits with
@@ -493,8 +498,8 @@ cudaError_t launch_hp_diag(const LaunchCtx& lc, uint16_t* out, int n, int m, con
 
 cudaError_t launch_observables(const LaunchCtx& lc, const float2* psi, int n, int m, const ClauseLP* cl,
                                double* partials, double* result, const unsigned* counts, int* err_word,
-                               unsigned long long* stamp) {
-  const int P = obs_grid(lc.num_sms);
+                               unsigned long long* stamp, bool err_to_result) {
+  const int P = obs_grid(lc.num_sms, n);
   const long long ntiles = n > kLowBits ? (1ll << (n - kLowBits)) : 1ll;
   const bool stored = counts != nullptr && n > kLowBits;
   cudaError_t err;
@@ -525,7 +530,8 @@ cudaError_t launch_observables(const LaunchCtx& lc, const float2* psi, int n, in
     }
     if (err != cudaSuccess) return err;
   }
-  obs_reduce_kernel<<<1, 256, 0, lc.stream>>>(partials, P, kObsQuant + cp.ng, result, stamp);
+  obs_reduce_kernel<<<1, 32 * kObsQuant, 0, lc.stream>>>(partials, P, kObsQuant + cp.ng, result,
+                                                         err_to_result ? err_word : nullptr, stamp);
   return cudaGetLastError();
 }
 

@@ -230,11 +230,12 @@ cudaError_t launch_hp_diag(const LaunchCtx& lc, uint16_t* out, int n, int m, con
 // {norm, <H_P>, ground_prob, ground_count, sum of pair correlations} on the device.
 size_t obs_partials_len(int n, int num_sms);
 // counts (optional): the stored per-tile clause counts of launch_lp_counts.
-// err: the bounded-wait error word of the TMA correlation passes.
+// err: the bounded-wait error word of the TMA correlation passes, copied to result[5]
+// with err_to_result.  result may be pinned host memory.
 cudaError_t launch_observables(const LaunchCtx& lc, const float2* psi, int n, int m,
                                const ClauseLP* cl, double* partials, double* result,
                                const unsigned* counts = nullptr, int* err = nullptr,
-                               unsigned long long* stamp = nullptr);
+                               unsigned long long* stamp = nullptr, bool err_to_result = false);
 // One thread writes the device's nanosecond timer to *stamp (the start of a
 // served request's device interval; the observables' last kernel writes its end).
 cudaError_t launch_stamp(const LaunchCtx& lc, unsigned long long* stamp);
