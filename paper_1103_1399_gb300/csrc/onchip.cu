@@ -21,7 +21,7 @@
 // a 400-step run, before and after: n = 6 1.76 / 0.48, n = 9 1.83 / 0.77, n = 11
 // 3.09 / 1.19 (from n = 12 on a single run takes a cluster, team.cu; batches keep one
 // CTA per instance).
-// Phase rows come through a ring of cp.async copies issued kRing - 1 steps ahead.
+// Phase rows come through a ring of cp.async copies issued kCtaRing - 1 steps ahead.
 #include "tile.cuh"
 
 namespace qaa {
@@ -55,16 +55,14 @@ __device__ __forceinline__ void fetch_rows(const RunArgs& A, float2* s_p, float2
 }
 
 // ------------------------------------------------------------ one warp ------
-constexpr int kWarpRing = 8;
-
+// A lane's entries of the phase rows depend on its energies only, so they are
+// loaded straight into registers, kAhead steps before their use.
 template <int N>
 __device__ void warp_run(const RunArgs& A, unsigned char* smem) {
+  constexpr int kAhead = N >= 8 ? 2 : 4;
   const int lane = threadIdx.x & 31;
   const int n = A.n, mp1 = A.m + 1;
-  float2* s_ab = reinterpret_cast<float2*>(smem);
-  float2* s_p = s_ab + 2 * kWarpRing;
-  ClauseMV* s_cl = reinterpret_cast<ClauseMV*>(smem + ((8u * (2 * kWarpRing + kWarpRing * mp1) + 15u) & ~15u));
-  for (int j = 0; j < kWarpRing - 1; ++j) fetch_rows<32, kWarpRing>(A, s_p, s_ab, j, lane);
+  ClauseMV* s_cl = reinterpret_cast<ClauseMV*>(smem);
   for (int c = lane; c < A.m; c += 32) s_cl[c] = A.cl[c];
   const bool mine = lane < (1 << n);  // n < 5: the other lanes hold zeros
   Inc<N> x;
@@ -76,14 +74,24 @@ __device__ void warp_run(const RunArgs& A, unsigned char* smem) {
   int ev[N];
 #pragma unroll
   for (int r = 0; r < N; ++r) ev[r] = 0;
+#pragma unroll 4
   for (int c = 0; c < A.m; ++c) {
     const unsigned mk = static_cast<unsigned>(s_cl[c].mask), vl = static_cast<unsigned>(s_cl[c].viol);
 #pragma unroll
     for (int r = 0; r < N; ++r) ev[r] += (static_cast<unsigned>(lane + 32 * r) & mk) == vl;
   }
-  unsigned e[(N + 1) / 2];
+  float2 z[kAhead][N], row[kAhead][2];
+  auto load = [&](int k, int j) {
+    if (j >= A.nsteps) return;
+    const float2* p = A.ptab + static_cast<size_t>(j + 1) * mp1;
+    const float2* b = A.btab + static_cast<size_t>(j) * (n + 1);
 #pragma unroll
-  for (int r = 0; r < N; r += 2) e[r / 2] = static_cast<unsigned>(8 * ev[r]) | (r + 1 < N ? static_cast<unsigned>(8 * ev[r + 1 < N ? r + 1 : r]) << 16 : 0u);
+    for (int r = 0; r < N; ++r) z[k][r] = __ldg(p + ev[r]);
+    row[k][0] = __ldg(b);
+    row[k][1] = __ldg(b + 1);
+  };
+#pragma unroll
+  for (int k = 0; k < kAhead; ++k) load(k, k);
   auto warp_norm = [&]() { return warp_sum(norm_of<N>(v)); };
   const DFloat nref = warp_norm();
   const int pc = __popc(lane);
@@ -95,35 +103,42 @@ __device__ void warp_run(const RunArgs& A, unsigned char* smem) {
   }
   x.zero();
   TurnScale ts;
-  for (int j = 0; j < A.nsteps; ++j) {
-    fetch_rows<32, kWarpRing>(A, s_p, s_ab, j + kWarpRing - 1, lane);
-    cp_async_wait<kWarpRing - 1>();
-    __syncwarp();
-    const RotCoef c = rot_coef(s_ab + 2 * (j % kWarpRing));
-    if constexpr (N >= 2) x.template turn<0, (N >= 8 ? 3 : (N >= 4 ? 2 : 1))>(c, true);
-    for (bool again = c.twice;; again = false) {
+  for (int j0 = 0; j0 < A.nsteps; j0 += kAhead) {
 #pragma unroll
-      for (int b = 0; b < 5; ++b) {
-        if (b < n) {
-          const unsigned long long k = ((lane >> b) & 1) ? c.nb : c.b;
+    for (int k = 0; k < kAhead; ++k) {
+      const int j = j0 + k;
+      if (j >= A.nsteps) break;
+      const RotCoef c = rot_coef(row[k]);
+      if constexpr (N >= 2) x.template turn<0, (N >= 8 ? 3 : (N >= 4 ? 2 : 1))>(c, true);
+      auto lanes = [&]() {
 #pragma unroll
-          for (int r = 0; r < N; ++r) {
-            const float2 s = x.at(r);
-            const float2 p = make_float2(__shfl_xor_sync(0xffffffffu, s.x, 1 << b), __shfl_xor_sync(0xffffffffu, s.y, 1 << b));
-            x.d[r] = fma2(k, p, x.d[r]);
+        for (int b = 0; b < 5; ++b) {
+          if (b < n) {
+            const unsigned long long kk = ((lane >> b) & 1) ? c.nb : c.b;
+#pragma unroll
+            for (int r = 0; r < N; ++r) {
+              const float2 s = x.at(r);
+              x.d[r] = fma2(kk, make_float2(__shfl_xor_sync(0xffffffffu, s.x, 1 << b), __shfl_xor_sync(0xffffffffu, s.y, 1 << b)),
+                            x.d[r]);
+            }
           }
         }
+      };
+      lanes();
+      if (c.twice) {
+        x.settle();
+        lanes();
       }
-      if (!again) break;
+#pragma unroll
+      for (int r = 0; r < N; ++r) x.d[r] = cmac(x.d[r], x.at(r), z[k][r]);
+      load(k, j + kAhead);
       x.settle();
+      scale_pow2<N>(v, c.pow2);
+      // every fold_period(n)-th step and the last
+      ts.step(c.r);
+      if ((j + 1) % fold_period(1) == 0 || j + 1 == A.nsteps)
+        scale_by<N>(v, __shfl_sync(0xffffffffu, ts.fold(nref, warp_norm()), 0));
     }
-    apply_rows<N>(x, e, s_p + (j % kWarpRing) * mp1);
-    x.settle();
-    scale_pow2<N>(v, c.pow2);
-    // every fold_period(n)-th step and the last
-    ts.step(c.r);
-    if ((j + 1) % fold_period(n) == 0 || j + 1 == A.nsteps) scale_by<N>(v, __shfl_sync(0xffffffffu, ts.fold(nref, warp_norm()), 0));
-    __syncwarp();
   }
   if (mine) {
 #pragma unroll
@@ -131,9 +146,7 @@ __device__ void warp_run(const RunArgs& A, unsigned char* smem) {
   }
 }
 
-size_t warp_smem(int m) {
-  return ((8u * (2 * kWarpRing + static_cast<size_t>(kWarpRing) * (m + 1)) + 15u) & ~static_cast<size_t>(15)) + 16u * m;
-}
+size_t warp_smem(int m) { return 16u * static_cast<size_t>(m); }
 
 // ------------------------------------------------------------- one CTA ------
 constexpr int kCtaRing = 4;
