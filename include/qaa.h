@@ -97,7 +97,8 @@ qaa_status qaa_set_stream(qaa_handle h, void* cuda_stream);
 
 /*
  * qaa_set_variant -- choose the Walsh-Hadamard implementation of the
- * streaming passes (n >= 15; the on-chip path for n <= 14 is always FP32).
+ * streaming passes (n >= 15; the on-chip path for n <= 14 is always FP32).  A call with an explicit
+ * variant runs the passes also where the default is a team of CTAs (15 <= n <= 21).
  *   wht_kind 0: FP32 CUDA-core butterflies, the whole-register W.B.W form.
  *            1: the W.B.W form with every transform on the tensor cores
  *               (tcgen05): each group of <= 10 qubits in two 5-qubit stages,
@@ -188,7 +189,8 @@ qaa_status qaa_forget_tuned_plans(void);
 
 /*
  * qaa_set_launch_mode -- how qaa_evolve* issue the streaming passes (n >= 15;
- * the on-chip path for n <= 14 is one launch per chunk either way).
+ * sizes whose state stays in the registers of a warp, a CTA or a team of
+ * CTAs (n <= 21 by default) take one launch per chunk either way).
  *   QAA_LAUNCH_PASSES (0, default): one kernel launch per pass from the host.
  *   QAA_LAUNCH_GRAPH  (1): one CUDA graph per step range, launched once: a
  *     WHILE conditional node whose body is 8 Strang steps, the phase rows of
@@ -216,7 +218,7 @@ qaa_status qaa_init_uniform(qaa_handle h, void* psi);
  * For n >= 15 on the TMA passes the handle stores, on the first evolution,
  * the bit-sliced violated-clause counts of every 1024-amplitude tile (as many
  * bit planes as the instance's largest count needs, at most 10: 1.25 bytes
- * per amplitude, 0.88 for the 30-qubit benchmark instance), allocated once at
+ * per amplitude, 0.75 for the 30-qubit benchmark instance), allocated once at
  * the largest size (1.25 GiB at n = 30), so that later low passes read them
  * instead of counting again; if that memory cannot be allocated the passes
  * count on the fly (the same values).  QAA_LP_COUNTS=0 turns the store off.
@@ -355,8 +357,8 @@ qaa_status qaa_observables_noalloc(int n, const int32_t* clauses, int m, const v
  * at a time).  Requests keep their states resident in a device arena that the
  * server reserves once, are admitted when their memory block and a result slot
  * are free, run in continuous batches (every admitted request with n <= 14 in
- * one launch of the batched on-chip evolver; larger ones as streaming passes on
- * a pool of streams, overlapped), and report host-clock timestamps for latency.
+ * one launch of the batched on-chip evolver; larger ones by a team of
+ * CTAs or as streaming passes on a pool of streams, overlapped), and report host-clock timestamps for latency.
  * Each request evolves from the uniform superposition over T with `steps`
  * Strang steps (as qaa_evolve) and returns the observables of the final state.
  * All functions are thread safe.
@@ -429,7 +431,7 @@ typedef enum {
   QAA_K_STRIDED = 3,       /* strided group pass: W                         */
   QAA_K_STRIDED_PHASE = 4, /* top group pass: W, popcount phase, W          */
   QAA_K_TABLES = 5,        /* FP64 phase-table generation                   */
-  QAA_K_ONCHIP = 6,        /* whole-run on-chip evolver (n <= 14)           */
+  QAA_K_ONCHIP = 6,        /* whole-run evolvers: one warp, CTA or CTA team */
   QAA_K_OBSERVE = 7,       /* observable reductions (all kernels of a call) */
   QAA_K_DIAG = 8,          /* E(x) export                                   */
   QAA_K_INIT = 9,          /* uniform-state initialisation                  */

@@ -7,7 +7,9 @@
 // are transformed before it (ascending) and after it (descending).  Per Strang
 // step: phase group W B W, the other groups down, the low pass W P W (merging
 // the half phases of two steps), the other groups up: 2g-2 HBM round trips for
-// g groups.  n <= 14 runs entirely on chip.
+// g groups.  In the rotation form (the default) no pass changes basis and a step is
+// g round trips.  n <= 14 runs entirely on chip, n <= 21 by default in the registers
+// of a team of CTAs (team.cu).
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
@@ -293,7 +295,7 @@ void make_default_plan(int n, PassPlan& plan, int max_q, int low, bool rotation)
     if (v >= 0 && v < ng) plan.phase_group = v;
   }
   // The form of the H_B factor: on the TMA FP32 passes the rotation form
-  // (W.diag.W on every 5-qubit block inside each pass: g round trips per
+  // (one-qubit turns inside each pass: g round trips per
   // step), otherwise the W.B.W form (2g - 2).
   plan.wht_kind = plan.use_tma ? kRotationForm : 0;
   set_default_run_c(plan);

@@ -10,11 +10,12 @@
 // block until its observables are read back.
 //
 // Work: admitted requests with n <= 14 are gathered into one launch of the
-// batched on-chip evolver (one CTA per request, whole run in shared memory);
+// batched on-chip evolver (one CTA per request);
 // requests with 15 <= n <= 17 get one persistent cooperative launch each
 // (persist.cu) on a few SMs, several running side by side; larger requests go
-// to issuer threads, each with its own stream, which launch the streaming
-// passes of the request's plan.  Completion is observed with one
+// to issuer threads, each with its own stream, which launch the request's team
+// evolver (n <= 21, its scratch at most a sixteenth of the arena) or the
+// streaming passes of its plan.  Completion is observed with one
 // event per request; the worker then reads the FP64 observables from a pinned
 // slot and releases the memory.
 //

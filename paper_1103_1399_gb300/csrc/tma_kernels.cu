@@ -1,14 +1,13 @@
 // TMA-pipelined streaming passes (n >= 15).  Same arithmetic as the passes in
 // pass_kernels.cu; what changes is how the state moves between HBM and the SM.
 //
-// * Strided passes (W over a group of Q index bits, or W B W over the top
-//   group): persistent CTAs, two dense 2^(Q+C)-amplitude tile buffers filled by
-//   4-D cp.async.bulk.tensor loads that complete on an mbarrier.  While a tile
-//   is transformed in registers, the TMA engine already fetches the tile after
-//   next into the other buffer.  Results go straight from registers to HBM.
-// * Low passes (W P W over bits 0..9): every warp owns two 8 KiB buffers filled
-//   by 1-D cp.async.bulk copies; the clause fold and bit-sliced count for a tile
-//   run while its data is still in flight.
+// * Strided passes (one-qubit turns or W over a group of Q index bits, or W B W
+//   over the top group): persistent CTAs, one dense 2^(Q+C)-amplitude tile buffer
+//   filled by 5-D cp.async.bulk.tensor loads that complete on an mbarrier and
+//   reused for the transposes.  Results go straight from registers to HBM.
+// * Low passes (turns then P, or W P W, over bits 0..9): every warp's tiles come
+//   by 1-D cp.async.bulk copies, in the rotation form into a landing buffer of
+//   their own.
 //
 // Every wait on an mbarrier is bounded; on expiry the kernel records an error
 // word that the host reports as QAA_E_TIMEOUT, and all threads of the block (or
@@ -212,13 +211,20 @@ __global__ void __launch_bounds__(TmaGeom<Q, C>::NT, (TmaGeom<Q, C>::NT >= 512 ?
     const unsigned long long ut = static_cast<unsigned long long>(T);
     const unsigned long long xbase = ((ut & lo_mask) << C) | (((ut >> lo_bits) & mid_mask) << (a1 + 5)) |
                                      ((ut >> (lo_bits + mid_bits)) << (a2 + QB));
+    // An 11-bit rotation pass takes layout L first and stores from layout H: a warp's
+    // store then covers four rows 2^a1 apart, on one page, instead of four rows of the
+    // upper range (n = 32 14.5 -> 12.5 ms a pass, n = 31 6.2 -> 6.6).
+    constexpr bool kLFirst = Q == 11 && MODE >= 2;
     float2 v[32];
     {
-      const float2* src = s_buf + h_off;
+      const float2* src = s_buf + (kLFirst ? j + (th << (C + 5)) : h_off);
 #pragma unroll
-      for (int r = 0; r < 32; ++r) v[r] = src[(r << QB) << C];
+      for (int r = 0; r < 32; ++r) v[r] = src[kLFirst ? r << C : (r << QB) << C];
     }
-    turn_or_wht<5, MODE>(v, rc);  // i bits QB..QB+4
+    if (kLFirst)
+      stage_l<QB, C, MODE>(v, rc, lane);  // i bits 0..QB-1
+    else
+      turn_or_wht<5, MODE>(v, rc);  // i bits QB..QB+4
     // Passes that store from layout L (plain W and the rotation form) are done
     // with the buffer once layout L is read: the next tile's copy starts there,
     // before the second butterfly stage, instead of after it (measured at
@@ -239,12 +245,15 @@ __global__ void __launch_bounds__(TmaGeom<Q, C>::NT, (TmaGeom<Q, C>::NT >= 512 ?
     if (QB > 0) {
       __syncthreads();  // dense tile fully read
 #pragma unroll
-      for (int r = 0; r < 32; ++r) s_buf[sx_h + G::slot((r << QB) << C)] = v[r];
+      for (int r = 0; r < 32; ++r) s_buf[kLFirst ? sx_l + (r << C) : sx_h + G::slot((r << QB) << C)] = v[r];
       __syncthreads();
 #pragma unroll
-      for (int r = 0; r < 32; ++r) v[r] = s_buf[sx_l + (r << C)];
+      for (int r = 0; r < 32; ++r) v[r] = s_buf[kLFirst ? sx_h + G::slot((r << QB) << C) : sx_l + (r << C)];
       if (kEarlyIssue) issue_next();
-      stage_l<QB, C, MODE>(v, rc, lane);  // i bits 0..QB-1
+      if (kLFirst)
+        turn_or_wht<5, MODE>(v, rc);  // i bits QB..QB+4
+      else
+        stage_l<QB, C, MODE>(v, rc, lane);  // i bits 0..QB-1
     }
     if (WBW) {
       // 2^-n exp(-i phi popcount(x)), x the full index
@@ -264,7 +273,7 @@ __global__ void __launch_bounds__(TmaGeom<Q, C>::NT, (TmaGeom<Q, C>::NT >= 512 ?
     }
     // the buffer is free: fetch the next tile while this one is stored
     if (!kEarlyIssue) issue_next();
-    if (WBW || QB == 0) {
+    if (WBW || QB == 0 || kLFirst) {
       // layout H: i = th + (r << QB); th = i bits 0..QB-1: bits 0..4 lie at a1.., bit 5 (QB = 6) at a2
       float2* dst = psi + xbase + j + (static_cast<unsigned long long>(th & 31) << a1) +
                     (static_cast<unsigned long long>(th >> 5) << a2);
@@ -685,6 +694,13 @@ static CUtensorMapL2promotion l2_promotion(int c) {
   }
 }
 
+// CTAs of a rotation pass beyond L2 (n >= 26): 18/19 of the SMs' room, a multiple of 16
+// (144 strided and 288 low-pass CTAs).  With every SM at work the reads and writes in
+// flight get in each other's way in DRAM; an odd count parts the neighbouring tiles that
+// share 256-byte lines.  n = 30, strided pass of one 512-thread CTA per SM: 152 CTAs 2.73 ms,
+// 148 2.68, 144 2.67, 136 2.68, 143 2.97; low pass: 304 CTAs 2.86 ms, 287 2.84, 272 2.82.
+static long long dram_grid(long long full) { return full * 18 / 19 / 16 * 16; }
+
 template <int Q, int C>
 static cudaError_t launch_sp_tma_c(const LaunchCtx& lc, float2* psi, int n, int a1, int a2, int mode,
                                    const float2* brow, int* err) {
@@ -714,6 +730,7 @@ static cudaError_t launch_sp_tma_c(const LaunchCtx& lc, float2* psi, int n, int 
   if (e != cudaSuccess) return e;
   if (occ < 1) occ = 1;
   long long grid = static_cast<long long>(occ) * lc.num_sms;
+  if (n >= 26 && mode >= 2 && Q == 10 && C == 4 && dram_grid(grid) > 0) grid = dram_grid(grid);
   if (grid > ntiles) grid = ntiles;
   return launch_overlapped(lc, kern, static_cast<unsigned>(grid), G::NT, G::smem, psi, map, n, a1, a2, brow, ntiles, err);
 }
@@ -784,23 +801,6 @@ int tma_run_bytes(int q, int run_c) {
   return 8 << c;
 }
 
-// The stored counts of every tile (layout Y), computed once per instance in
-// two launches of the same fold and count: MEASURE raises the header's plane
-// count P to the bits of the largest count any lane holds, then the second
-// launch stores P planes and the constant part of every tile.
-template <bool MEASURE>
-__global__ void __launch_bounds__(kLpTmaWarps * 32)
-    lp_counts_kernel(int m, const ClauseLP* __restrict__ cl, unsigned* __restrict__ counts, long long ntiles,
-                     unsigned planes_off) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  ClauseLP* s_cl = reinterpret_cast<ClauseLP*>(smem);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  uint2* s_act = reinterpret_cast<uint2*>(smem + 16u * m) + warp * (m + 16);
-  for (int i = threadIdx.x; i < m; i += blockDim.x) s_cl[i] = cl[i];
-  __syncthreads();
-  const int P = MEASURE ? kPlanes : static_cast<int>(counts[0]);
-  unsigned* planes = counts + planes_off;
-  if (!MEASURE && blockIdx.x == 0 && threadIdx.x == 0) counts[1] = planes_off;
 // Takes the smallest of the warp's 1024 bit-sliced counts out of all of them and
 // returns it: what is left of a tile's counts often needs a plane less (7 -> 6 for the
 // 30-qubit benchmark instance, 0.13 of 18.1 GB per low pass).
@@ -825,6 +825,23 @@ __device__ __forceinline__ int take_min(unsigned (&pl)[kPlanes]) {
   return least;
 }
 
+// The stored counts of every tile (layout Y), computed once per instance in
+// two launches of the same fold and count: MEASURE raises the header's plane
+// count P to the bits of the largest count any lane holds, then the second
+// launch stores P planes and the constant part of every tile.
+template <bool MEASURE>
+__global__ void __launch_bounds__(kLpTmaWarps * 32)
+    lp_counts_kernel(int m, const ClauseLP* __restrict__ cl, unsigned* __restrict__ counts, long long ntiles,
+                     unsigned planes_off) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  ClauseLP* s_cl = reinterpret_cast<ClauseLP*>(smem);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  uint2* s_act = reinterpret_cast<uint2*>(smem + 16u * m) + warp * (m + 16);
+  for (int i = threadIdx.x; i < m; i += blockDim.x) s_cl[i] = cl[i];
+  __syncthreads();
+  const int P = MEASURE ? kPlanes : static_cast<int>(counts[0]);
+  unsigned* planes = counts + planes_off;
+  if (!MEASURE && blockIdx.x == 0 && threadIdx.x == 0) counts[1] = planes_off;
   unsigned used = 0u;  // OR of every plane word this lane computed, by plane
   for (long long tile = static_cast<long long>(blockIdx.x) * kLpTmaWarps + warp; tile < ntiles;
        tile += static_cast<long long>(gridDim.x) * kLpTmaWarps) {
@@ -833,6 +850,7 @@ __device__ __forceinline__ int take_min(unsigned (&pl)[kPlanes]) {
     __syncwarp();
     fold_tile<true>(s_cl, m, static_cast<unsigned>(tile), lane, s_act, nconst, npad);
     count_active(s_act, npad, 1u << lane, pl);
+    nconst += take_min(pl);
     if (MEASURE) {
 #pragma unroll
       for (int b = 0; b < kPlanes; ++b) used |= pl[b] != 0u ? (1u << b) : 0u;
@@ -850,7 +868,6 @@ __device__ __forceinline__ int take_min(unsigned (&pl)[kPlanes]) {
   }
 }
 
-    nconst += take_min(pl);
 static long long counts_planes_offset(long long ntiles) {
   return kCountHeaderWords + ((ntiles + 31) / 32) * 32;
 }
@@ -896,6 +913,7 @@ static cudaError_t launch_lp_tma(const LaunchCtx& lc, float2* psi, int n, int m,
     if (occ < 1) occ = 1;
   }
   long long grid = static_cast<long long>(occ) * lc.num_sms;
+  if (SPLIT == 2 && dram_grid(grid) > 0) grid = dram_grid(grid);
   const long long need = (ntiles + kWarps - 1) / kWarps;
   if (grid > need) grid = need;
   if (grid > kFoldSlot - 1) grid = kFoldSlot - 1;  // one norm-fold partial per CTA
