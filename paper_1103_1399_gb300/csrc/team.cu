@@ -17,9 +17,9 @@
 // The exchange:
 // * CLUSTER (8 CTAs of one cluster): st.async into the partners' shared memory,
 //   counted by the receiver's mbarrier (a cluster barrier per step instead: 1.79
-//   against 1.51 us per step at n = 13).  Two receive buffers in turn: what a CTA has
-//   received in step j - 1 its partners sent after their last read of the buffer
-//   that it writes in step j.
+//   against 1.51 us per step at n = 13).  Two receive buffers in turn, for nothing else
+//   (team_schedule.h): what a CTA has received in step j its partners sent after a
+//   barrier behind their reads of step j - 1's buffer, which it fills in step j + 1.
 // * grid (a cooperative launch): 64-bit words in global memory (L2) that say by
 //   themselves whether they have arrived (kEmpty), so the exchange costs one store
 //   and the polling of one load; with a grid barrier between stores and loads (a
@@ -31,6 +31,7 @@
 // Norm fold as in the streaming passes (NormFold), with the reference kept in the
 // handle's fold slot across launches of a range: the sum measured after a step
 // travels with the next exchange and corrects the P after it.
+#include "team_schedule.h"
 #include "tile.cuh"
 
 namespace qaa {
@@ -165,9 +166,9 @@ struct TeamGeom : CtaGeom<T, R> {
   static constexpr int kOut = kSplit ? kTop : kMid;   // window that sends
   static_assert(D >= 0 && (!kSplit || D >= R), "incoming bits must lie in TOP and MID");
   static_assert(!CLUSTER || C <= 3, "portable clusters of 8 CTAs");
-  // cluster: a transpose buffer and two receive buffers (the current one serves
-  // the second transpose); grid: two transpose buffers, one for 2^14 amplitudes
-  static constexpr int kBufs = CLUSTER ? 3 : (T <= 13 ? 2 : 1);
+  // cluster: two transpose and two receive buffers; grid: two transpose buffers, one
+  // for 2^14 amplitudes
+  static constexpr int kBufs = CLUSTER ? kClusterBuffers : (T <= 13 ? 2 : 1);
   // grid: self-validating words, with a warp of its own for the fence that orders
   // the emptied slots; 512 threads with 32 amplitudes each (2^14 per CTA) use the
   // grid barrier: the words' second set of stores and registers cost more there
@@ -323,9 +324,8 @@ __global__ void __launch_bounds__(TeamGeom<T, R, C, CLUSTER>::kThreads, (TeamGeo
   for (int j = 0; j < A.nsteps; ++j) {
     const RotCoef c = rot_coef(s_ab + 2 * (j % kTeamRing));
     const float2* prow = s_p + (j % kTeamRing) * mp1;
-    // the receive buffer of the previous step (cluster): free for the second transpose
-    float2* b0 = CLUSTER ? buffer(0) : buffer(b);
-    float2* b1 = CLUSTER ? buffer(1 + ((j + 1) & 1)) : buffer(G::kBufs == 2 ? b ^ 1 : 0);
+    float2* b0 = buffer(CLUSTER ? cluster_transpose(j, 0) : b);
+    float2* b1 = buffer(CLUSTER ? cluster_transpose(j, 1) : (G::kBufs == 2 ? b ^ 1 : 0));
     auto middle = [&]() {  // barrier between a put and a get; with one buffer another before the next put
       cp_async_wait<0>();
       team_sync<NT>();
@@ -383,7 +383,7 @@ __global__ void __launch_bounds__(TeamGeom<T, R, C, CLUSTER>::kThreads, (TeamGeo
       constexpr int ls = win_step<T, R, kOut>();
       constexpr int dm = (1 << D) - 1;
       if constexpr (CLUSTER) {
-        float2* dst = buffer(1 + (j & 1)) + G::slot((l0 & dm) | static_cast<int>(cta) << D);
+        float2* dst = buffer(cluster_receive(j)) + G::slot((l0 & dm) | static_cast<int>(cta) << D);
 #pragma unroll
         for (int r = 0; r < N; ++r)
           peer_send(peer_smem(dst, (l0 >> D) + ((r * ls) >> D)) + 8u * G::slot((r * ls) & dm), v[r],
@@ -391,7 +391,7 @@ __global__ void __launch_bounds__(TeamGeom<T, R, C, CLUSTER>::kThreads, (TeamGeo
         if (!recv_wait(s_bar + (j & 1), (j >> 1) & 1)) late = true;
         if (__syncthreads_or(late)) break;
         if (tid == 0 && j + 2 < A.nsteps) expect(j + 2);
-        get<T, R, kTop>(v, buffer(1 + (j & 1)), tid);
+        get<T, R, kTop>(v, buffer(cluster_receive(j)), tid);
       } else {
         // three buffers in turn (words), two with the grid barrier
         float2* xb = A.xbuf + (static_cast<size_t>(G::kWords ? j % 3 : j & 1) << A.n);

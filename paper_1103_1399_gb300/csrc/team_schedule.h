@@ -1,0 +1,22 @@
+// Which buffer of a team's exchange each step uses (team.cu), in one place so that a
+// host program can check the order of every pair of accesses.
+#pragma once
+
+#ifdef __CUDACC__
+#define QAA_HD __host__ __device__
+#else
+#define QAA_HD
+#endif
+
+namespace qaa {
+
+// Cluster form, shared memory of one CTA: two buffers for its own transposes, then two
+// that its partners fill, in turn by step.  The transposes stay out of what the partners
+// fill: a partner that has its words of step j may send step j + 1 while other threads
+// of this CTA still read their last transpose of step j (each partner's words come
+// from some of the threads only).
+constexpr int kClusterBuffers = 4;
+QAA_HD constexpr int cluster_transpose(int j, int k) { return (void)j, k; }  // k: 0, 1
+QAA_HD constexpr int cluster_receive(int j) { return 2 + (j & 1); }
+
+}  // namespace qaa

@@ -1,0 +1,114 @@
+// Host check of the team evolver's exchange buffers (team_schedule.h): every write of a
+// buffer is ordered against every other access of it.
+//
+// Cluster form: two CTAs of two threads each, thread t of either sending to CTA t (the
+// sparsest pattern the kernel has: a CTA's words for one partner come from some of its
+// threads only).  The accesses of several steps are laid out as the kernel makes them;
+// a happens-before relation is closed over program order, the CTA's barriers and the
+// arrival of sent words (a wait orders the waiting CTA behind the threads that sent to
+// it, no others).  Prints "ok" and exits 0, else prints the first violation and exits 1.
+#include <cstdio>
+#include <vector>
+
+#include "team_schedule.h"
+
+namespace {
+
+constexpr int kSteps = 7;
+
+struct Event {
+  int cta, thread, step;
+  const char* what;
+  int mem_cta, buffer;  // memory accessed; buffer -1: none
+  bool write;
+};
+
+struct Graph {
+  std::vector<Event> ev;
+  std::vector<std::vector<int>> next;
+  int last[2][3];
+  Graph() {
+    for (auto& c : last)
+      for (int& t : c) t = -1;
+  }
+  int add(const Event& e) {
+    ev.push_back(e);
+    next.emplace_back();
+    const int i = static_cast<int>(ev.size()) - 1;
+    int& l = last[e.cta][e.thread];
+    if (l >= 0) next[l].push_back(i);
+    return l = i;
+  }
+  // a barrier among the threads [0, nt) of every CTA
+  void barrier(int j, int nt) {
+    for (int c = 0; c < 2; ++c) {
+      std::vector<int> in, out;
+      for (int t = 0; t < nt; ++t) in.push_back(add({c, t, j, "arrive", c, -1, false}));
+      for (int t = 0; t < nt; ++t) out.push_back(add({c, t, j, "leave", c, -1, false}));
+      for (int a : in)
+        for (int b : out) next[a].push_back(b);
+    }
+  }
+  std::vector<char> after(int i) const {
+    std::vector<char> seen(ev.size(), 0);
+    std::vector<int> todo{i};
+    while (!todo.empty()) {
+      const int k = todo.back();
+      todo.pop_back();
+      for (int m : next[k])
+        if (!seen[m]) seen[m] = 1, todo.push_back(m);
+    }
+    return seen;
+  }
+  int check(const char* form) const {
+    std::vector<std::vector<char>> reach;
+    for (size_t i = 0; i < ev.size(); ++i) reach.push_back(after(static_cast<int>(i)));
+    for (size_t a = 0; a < ev.size(); ++a)
+      for (size_t b = a + 1; b < ev.size(); ++b) {
+        const Event &x = ev[a], &y = ev[b];
+        if (x.buffer < 0 || x.buffer != y.buffer || x.mem_cta != y.mem_cta || !(x.write || y.write)) continue;
+        // threads write parts of their own of one transpose or exchange
+        if (x.write && y.write && x.step == y.step && x.what == y.what) continue;
+        if (!reach[a][b] && !reach[b][a]) {
+          std::printf("%s: buffer %d of CTA %d: %s of CTA %d thread %d step %d and %s of CTA %d thread %d step %d unordered\n", form,
+                      x.buffer, x.mem_cta, x.what, x.cta, x.thread, x.step, y.what, y.cta, y.thread, y.step);
+          return 1;
+        }
+      }
+    return 0;
+  }
+};
+
+int cluster() {
+  Graph g;
+  auto all = [&](int j, const char* what, int buffer, bool write) {
+    for (int c = 0; c < 2; ++c)
+      for (int t = 0; t < 2; ++t) g.add({c, t, j, what, c, buffer, write});
+  };
+  for (int j = 0; j < kSteps; ++j) {
+    for (int k = 0; k < 2; ++k) {
+      all(j, k ? "put 1" : "put 0", qaa::cluster_transpose(j, k), true);
+      g.barrier(j, 2);
+      all(j, k ? "get 1" : "get 0", qaa::cluster_transpose(j, k), false);
+    }
+    int sent[2][2];  // [receiver][sender]
+    for (int c = 0; c < 2; ++c)
+      for (int t = 0; t < 2; ++t) sent[t][c] = g.add({c, t, j, "send", t, qaa::cluster_receive(j), true});
+    for (int c = 0; c < 2; ++c)
+      for (int t = 0; t < 2; ++t) {
+        const int w = g.add({c, t, j, "wait", c, -1, false});
+        for (int s = 0; s < 2; ++s) g.next[sent[c][s]].push_back(w);
+      }
+    g.barrier(j, 2);
+    all(j, "get received", qaa::cluster_receive(j), false);
+  }
+  return g.check("cluster");
+}
+
+}  // namespace
+
+int main() {
+  if (cluster()) return 1;
+  std::puts("ok");
+  return 0;
+}
