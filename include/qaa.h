@@ -208,6 +208,13 @@ qaa_status qaa_forget_tuned_plans(void);
 #define QAA_LAUNCH_GRAPH 1
 qaa_status qaa_set_launch_mode(qaa_handle h, int mode);
 
+/* Fault injection for tests: fault 1, on a handle whose evolutions run on a team of
+ * CTAs (12 <= n <= 21 by default; else QAA_E_STATE): in the next evolution one CTA
+ * withholds what it sends in the first exchange.  The others' bounded waits run out,
+ * every CTA returns, psi is undefined, the next call that reads a result from the
+ * device reports QAA_E_TIMEOUT, and the handle stays usable.  Nothing traps or faults. */
+qaa_status qaa_inject(qaa_handle h, int fault);
+
 /* psi[x] = 2^(-n/2) for all x: the ground state of H_B (Sec. 2.1).  Asynchronous. */
 qaa_status qaa_init_uniform(qaa_handle h, void* psi);
 

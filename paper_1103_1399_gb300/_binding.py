@@ -56,6 +56,7 @@ SIGNATURES = {
     "qaa_set_stream": (_c_int, [_vp, _vp]),
     "qaa_set_variant": (_c_int, [_vp, _c_int, _c_int]),
     "qaa_set_launch_mode": (_c_int, [_vp, _c_int]),
+    "qaa_inject": (_c_int, [_vp, _c_int]),
     "qaa_evolve_substeps": (_c_int, [_vp, _vp, ctypes.POINTER(ctypes.c_double), ctypes.POINTER(ctypes.c_double),
                                      ctypes.c_int64]),
     "qaa_evolve_order4": (_c_int, [_vp, _vp, ctypes.c_double, ctypes.c_int64]),
@@ -212,6 +213,10 @@ class Instance:
     def set_launch_mode(self, mode):
         """0: one launch per pass; 1: one CUDA graph per evolve range (qaa_set_launch_mode)."""
         _check(lib.qaa_set_launch_mode(self._h, int(mode)))
+
+    def inject(self, fault):
+        """Fault injection for tests (qaa_inject)."""
+        _check(lib.qaa_inject(self._h, int(fault)))
 
     def init_uniform(self, psi):
         _check_state(self, psi)

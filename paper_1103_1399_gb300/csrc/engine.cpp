@@ -10,6 +10,7 @@
 #include <mutex>
 #include <new>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "engine_internal.h"
@@ -82,6 +83,7 @@ struct qaa_ctx {
   // (the device cannot hold the team, or no memory)
   char* d_team = nullptr;
   int team_state = 0;
+  bool team_lose = false;  // qaa_inject: the next team launch loses an exchange
   // Lanczos workspace (qaa_lowest_eigenvalues), allocated on first use
   void* d_lz = nullptr;
   size_t lz_bytes = 0;
@@ -367,7 +369,8 @@ qaa_status evolve_impl(qaa_ctx* h, void* psi, double dt, long long K, long long 
     if (team) {
       QAA_CK(timed(h, graph ? -1 : QAA_K_ONCHIP, [&] {
         return qaa::launch_team(lc, p, h->n, h->m, reinterpret_cast<const uint16_t*>(h->d_team), ptab, btab,
-                                static_cast<int>(c1 - c0), c0 == k0, h->d_team + energy_bytes(h->n), h->d_fold, h->d_err);
+                                static_cast<int>(c1 - c0), c0 == k0, h->d_team + energy_bytes(h->n), h->d_fold, h->d_err,
+                                std::exchange(h->team_lose, false));
       }));
       continue;
     }
@@ -876,6 +879,14 @@ qaa_status qaa_set_launch_mode(qaa_handle h, int mode) {
   if (mode != QAA_LAUNCH_PASSES && mode != QAA_LAUNCH_GRAPH)
     return fail(QAA_E_ARG, "unknown launch mode (0 = per-pass launches, 1 = launch graph)");
   h->launch_mode = mode;
+  return QAA_OK;
+}
+
+qaa_status qaa_inject(qaa_handle h, int fault) {
+  if (!h) return fail(QAA_E_ARG, "null handle");
+  if (fault != 1) return fail(QAA_E_ARG, "unknown fault (1 = an exchange of the evolving team is lost)");
+  if (!qaa::team_plan(h->plan)) return fail(QAA_E_STATE, "this handle's plan does not run on a team of CTAs");
+  h->team_lose = true;
   return QAA_OK;
 }
 

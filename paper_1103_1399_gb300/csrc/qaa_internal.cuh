@@ -218,13 +218,14 @@ cudaError_t launch_onchip_batch(const LaunchCtx& lc, const OnchipJob* jobs_dev, 
 // 12 <= n <= 21.  energy: E(x) as launch_hp_diag writes it; rows of the kRowsTurn
 // form; work: team_bytes(n) of device scratch, team_reset before its first launch
 // and after one that ran out of time (every complete launch leaves it reset);
-// fold: the range's norm-fold slots (first = the launch starts the range).
+// fold: the range's norm-fold slots (first = the launch starts the range).  lose: the
+// injected fault of qaa_inject.
 constexpr int kTeamMinBits = 12, kTeamMaxBits = 21;
 bool team_fits(int n, int m, int num_sms);
 size_t team_bytes(int n);
 cudaError_t team_reset(const LaunchCtx& lc, int n, void* work);
 cudaError_t launch_team(const LaunchCtx& lc, float2* psi, int n, int m, const uint16_t* energy, const float2* ptab,
-                        const float2* btab, int nsteps, bool first, void* work, double* fold, int* err);
+                        const float2* btab, int nsteps, bool first, void* work, double* fold, int* err, bool lose = false);
 cudaError_t launch_hp_diag(const LaunchCtx& lc, uint16_t* out, int n, int m, const ClauseLP* cl);
 // Observables: partials has room for obs_partials_len(n) doubles; result is 5 doubles
 // {norm, <H_P>, ground_prob, ground_count, sum of pair correlations} on the device.

@@ -39,7 +39,10 @@ namespace qaa {
 namespace {
 
 constexpr int kTeamRing = 3;  // phase rows in flight: this step's and two ahead
-constexpr int kTeamPolls = 1 << 21;  // about two seconds
+// Polls of a wait before it gives up, by default and with an injected fault.  The cluster
+// form must not give up while words sent to it are in flight (its CTAs return after
+// giving up): even the smaller limit takes hundreds of times a word's flight.
+constexpr int kTeamPolls = 1 << 21, kTeamPollsInjected = 1 << 12;
 
 struct TeamArgs {
   float2* psi;
@@ -52,7 +55,9 @@ struct TeamArgs {
   float2* ref;     // the range's reference norm (double-float)
   int* err;
   int n, m, nsteps;
+  int polls;       // limit of every wait on another CTA
   bool first;      // the launch starts a range: apply P row 0, take the reference
+  bool lose;       // injected fault: CTA 0 withholds its first exchange
 };
 
 __device__ __forceinline__ unsigned cluster_rank() {
@@ -67,9 +72,6 @@ __device__ __forceinline__ uint32_t peer_smem(const void* p, unsigned rank) {
   uint32_t a;
   asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(p))), "r"(rank));
   return a;
-}
-__device__ __forceinline__ void peer_store(uint32_t a, float2 v) {
-  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
 }
 
 // The grid exchange: amplitudes go through global memory as 64-bit words that say
@@ -87,12 +89,12 @@ __device__ __forceinline__ void word_store(float2* p, unsigned long long x) {
 }
 // Take N words at p, p + step, ...; false when the wait ran out.
 template <int N>
-__device__ __forceinline__ bool take_words(float2 (&v)[N], float2* p, int step) {
+__device__ __forceinline__ bool take_words(float2 (&v)[N], float2* p, int step, int polls) {
   unsigned long long x[N];
 #pragma unroll
   for (int r = 0; r < N; ++r) x[r] = word_load(p + r * step);
   bool wait = true;
-  for (int i = 0; wait && i < kTeamPolls; ++i) {
+  for (int i = 0; wait && i < polls; ++i) {
     wait = false;
 #pragma unroll
     for (int r = 0; r < N; ++r)
@@ -110,14 +112,15 @@ __device__ __forceinline__ bool take_words(float2 (&v)[N], float2* p, int step) 
 }
 // The other grid exchange: plain stores, a grid barrier, plain loads.  Every
 // CTA's stores before its `round`-th call are visible to this one after it; false
-// when the wait ran out.  The counter only grows within a launch.
-__device__ __forceinline__ bool grid_barrier(unsigned* count, unsigned round, int tid, int* s_ok) {
+// when the wait ran out.  The counter only grows within a launch.  `arrive`: false for
+// the injected fault.
+__device__ __forceinline__ bool grid_barrier(unsigned* count, unsigned round, bool arrive, int polls, int tid, int* s_ok) {
   __syncthreads();
   if (tid == 0) {
     const unsigned target = round * gridDim.x;
-    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
+    if (arrive) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
     int ok = 0;
-    for (int i = 0; i < kTeamPolls && !ok; ++i) {
+    for (int i = 0; i < polls && !ok; ++i) {
       unsigned c;
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(count) : "memory");
       ok = c >= target;
@@ -144,8 +147,8 @@ __device__ __forceinline__ void peer_send(uint32_t a, float2 v, uint32_t bar) {
                "f"(v.y), "r"(bar)
                : "memory");
 }
-__device__ __forceinline__ bool recv_wait(uint64_t* bar, uint32_t parity) {
-  for (long long i = 0; i < kTeamPolls; ++i) {
+__device__ __forceinline__ bool recv_wait(uint64_t* bar, uint32_t parity, int polls) {
+  for (int i = 0; i < polls; ++i) {
     uint32_t ok;
     asm volatile(
         "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
@@ -270,7 +273,7 @@ __global__ void __launch_bounds__(TeamGeom<T, R, C, CLUSTER>::kThreads, (TeamGeo
       if (tid < 32) {
         for (int i = tid; i < TEAM; i += 32) {
           float2 p[1];
-          if (!take_words<1>(p, A.part + (end * TEAM + cta) * TEAM + i, 0)) s_late = 1;
+          if (!take_words<1>(p, A.part + (end * TEAM + cta) * TEAM + i, 0, A.polls)) s_late = 1;
           t = df_add(t, DFloat{p[0].x, p[0].y});
         }
         t = warp_sum(t);
@@ -382,14 +385,18 @@ __global__ void __launch_bounds__(TeamGeom<T, R, C, CLUSTER>::kThreads, (TeamGeo
       const int l0 = win_base<T, R, kOut>(tid);
       constexpr int ls = win_step<T, R, kOut>();
       constexpr int dm = (1 << D) - 1;
+      const bool lost = A.lose && cta == 0 && j == 0;
       if constexpr (CLUSTER) {
         float2* dst = buffer(cluster_receive(j)) + G::slot((l0 & dm) | static_cast<int>(cta) << D);
+        if (!lost) {
 #pragma unroll
-        for (int r = 0; r < N; ++r)
-          peer_send(peer_smem(dst, (l0 >> D) + ((r * ls) >> D)) + 8u * G::slot((r * ls) & dm), v[r],
-                    peer_smem(s_bar + (j & 1), (l0 >> D) + ((r * ls) >> D)));
-        if (!recv_wait(s_bar + (j & 1), (j >> 1) & 1)) late = true;
-        if (__syncthreads_or(late)) break;
+          for (int r = 0; r < N; ++r)
+            peer_send(peer_smem(dst, (l0 >> D) + ((r * ls) >> D)) + 8u * G::slot((r * ls) & dm), v[r],
+                      peer_smem(s_bar + (j & 1), (l0 >> D) + ((r * ls) >> D)));
+        }
+        // the CTA goes on or gives up as one: words may arrive as some threads' waits run out
+        late = __syncthreads_or(!recv_wait(s_bar + (j & 1), (j >> 1) & 1, A.polls)) != 0;
+        if (late) break;
         if (tid == 0 && j + 2 < A.nsteps) expect(j + 2);
         get<T, R, kTop>(v, buffer(cluster_receive(j)), tid);
       } else {
@@ -401,15 +408,17 @@ __global__ void __launch_bounds__(TeamGeom<T, R, C, CLUSTER>::kThreads, (TeamGeo
           if (j >= 2) {  // the fence warp is done with step j - 2
             if (j & 1) bar_sync<4, NT + 32>(); else bar_sync<3, NT + 32>();
           }
+          if (!lost) {
 #pragma unroll
-          for (int r = 0; r < N; ++r)
-            word_store(dst + ((static_cast<size_t>((r * ls) >> D) << T) + ((r * ls) & dm)), f2_bits(v[r]));
-          if (!take_words<N>(v, src, win_step<T, R, kTop>())) s_late = 1;
+            for (int r = 0; r < N; ++r)
+              word_store(dst + ((static_cast<size_t>((r * ls) >> D) << T) + ((r * ls) & dm)), f2_bits(v[r]));
+          }
+          if (!take_words<N>(v, src, win_step<T, R, kTop>(), A.polls)) s_late = 1;
           bar_arrive<2, NT + 32>();
         } else {
 #pragma unroll
           for (int r = 0; r < N; ++r) __stcg(dst + ((static_cast<size_t>((r * ls) >> D) << T) + ((r * ls) & dm)), v[r]);
-          if (!grid_barrier(A.count, static_cast<unsigned>(j) + 1u, tid, &s_ok)) {
+          if (!grid_barrier(A.count, static_cast<unsigned>(j) + 1u, !lost, A.polls, tid, &s_ok)) {
             late = true;
             break;
           }
@@ -468,7 +477,7 @@ __global__ void __launch_bounds__(TeamGeom<T, R, C, CLUSTER>::kThreads, (TeamGeo
     team_sync<NT>();
     if (tid < 32) publish(2, 1);
     if (CLUSTER) {
-      if (!recv_wait(s_bar + 2, 0)) late = true;
+      late = __syncthreads_or(!recv_wait(s_bar + 2, 0, A.polls)) != 0;
     }
     scale_by<N>(v, ts.fold(ref, collect(1)));
     if (!CLUSTER) late = *static_cast<volatile int*>(&s_late) != 0;
@@ -588,7 +597,7 @@ bool team_fits(int n, int m, int num_sms) {
 }
 
 cudaError_t launch_team(const LaunchCtx& lc, float2* psi, int n, int m, const uint16_t* energy, const float2* ptab,
-                        const float2* btab, int nsteps, bool first, void* work, double* fold, int* err) {
+                        const float2* btab, int nsteps, bool first, void* work, double* fold, int* err, bool lose) {
   if (nsteps < 1) return cudaErrorInvalidValue;
   char* w = static_cast<char*>(work);
   TeamArgs A;
@@ -604,7 +613,9 @@ cudaError_t launch_team(const LaunchCtx& lc, float2* psi, int n, int m, const ui
   A.n = n;
   A.m = m;
   A.nsteps = nsteps;
+  A.polls = lose ? kTeamPollsInjected : kTeamPolls;
   A.first = first;
+  A.lose = lose;
   switch (n) {
 #define QAA_CASE(T, R, C, K) \
   case T + C:                \
