@@ -24,9 +24,8 @@
 //   themselves whether they have arrived (kEmpty), so the exchange costs one store
 //   and the polling of one load; with a grid barrier between stores and loads (a
 //   release, an atomic, an acquire and the loads in sequence) n = 16 took 3.10
-//   instead of 2.70 us per step.  Three buffers in turn: a slot emptied in step j is
-//   written again in step j + 3 by a CTA that has received data this CTA sent in step
-//   j + 2, after the fence warp's fence that follows the emptying.
+//   instead of 2.70 us per step.  The slots are used in turn (team_schedule.h): a warp
+//   of its own runs the fences that order a slot's emptying before its next word.
 //
 // Norm fold as in the streaming passes (NormFold), with the reference kept in the
 // handle's fold slot across launches of a range: the sum measured after a step
@@ -49,7 +48,7 @@ struct TeamArgs {
   const uint16_t* energy;  // E(x)
   const float2* ptab;
   const float2* btab;
-  float2* xbuf;    // grid: 2 x 2^n amplitudes
+  float2* xbuf;    // grid: the exchange buffers, 2^n amplitudes each
   float2* part;    // grid: [receiver][sender] norm partials of the steps, then of the end
   unsigned* count; // grid barrier: arrivals, zeroed before the launch
   float2* ref;     // the range's reference norm (double-float)
@@ -217,11 +216,11 @@ __global__ void __launch_bounds__(TeamGeom<T, R, C, CLUSTER>::kThreads, (TeamGeo
     if (tid == 0) s_late = 0;
     __syncthreads();
     if (G::kWords && tid >= NT) {
-      // the fence warp: kEmpty stores of step j are visible to the whole device
-      // before any amplitude of step j + 2 leaves this CTA
+      // the fence warp: takes and kEmpty stores of step j come before any amplitude of
+      // step j + kWordFenceLag leaves this CTA
       for (int j = 0; j < A.nsteps; ++j) {
         bar_sync<2, NT + 32>();
-        if (*static_cast<volatile int*>(&s_late) || j + 2 >= A.nsteps) return;
+        if (*static_cast<volatile int*>(&s_late) || j + kWordFenceLag >= A.nsteps) return;
         __threadfence();
         if (j & 1) bar_arrive<4, NT + 32>(); else bar_arrive<3, NT + 32>();
       }
@@ -400,12 +399,12 @@ __global__ void __launch_bounds__(TeamGeom<T, R, C, CLUSTER>::kThreads, (TeamGeo
         if (tid == 0 && j + 2 < A.nsteps) expect(j + 2);
         get<T, R, kTop>(v, buffer(cluster_receive(j)), tid);
       } else {
-        // three buffers in turn (words), two with the grid barrier
-        float2* xb = A.xbuf + (static_cast<size_t>(G::kWords ? j % 3 : j & 1) << A.n);
+        float2* xb = A.xbuf + (static_cast<size_t>(G::kWords ? word_buffer(j) : j & 1) << A.n);
         float2* dst = xb + (static_cast<size_t>(l0 >> D) << T) + ((l0 & dm) | static_cast<int>(cta) << D);
         float2* src = xb + (static_cast<size_t>(cta) << T) + win_base<T, R, kTop>(tid);
         if constexpr (G::kWords) {
-          if (j >= 2) {  // the fence warp is done with step j - 2
+          if (j >= kWordFenceLag) {  // the fence warp is done with step j - kWordFenceLag
+            static_assert(kWordFenceLag == 2, "one barrier per parity");
             if (j & 1) bar_sync<4, NT + 32>(); else bar_sync<3, NT + 32>();
           }
           if (!lost) {
@@ -576,7 +575,7 @@ bool fits(int num_sms, int m) {
 constexpr size_t kTeamHead = 2u * 65536u * sizeof(float2);
 size_t team_bytes(int n) {
   if (n <= 14) return 0;
-  return kTeamHead + 256 + (static_cast<size_t>(n <= 20 ? 24 : 16) << n);
+  return kTeamHead + 256 + (static_cast<size_t>(8 * (n <= 20 ? kWordBuffers : 2)) << n);
 }
 
 cudaError_t team_reset(const LaunchCtx& lc, int n, void* work) {

@@ -19,4 +19,15 @@ constexpr int kClusterBuffers = 4;
 QAA_HD constexpr int cluster_transpose(int j, int k) { return (void)j, k; }  // k: 0, 1
 QAA_HD constexpr int cluster_receive(int j) { return 2 + (j & 1); }
 
+// Word form, global memory: buffers in turn by step.  A receiver empties a slot in step
+// j, after it has taken the word; its sender stores the next word there in step j +
+// kWordBuffers.  Behind the takes and emptyings of step j a warp of each CTA runs a
+// fence, and the CTA's stores of step j + kWordFenceLag wait for it.  The emptying is
+// before the next store if a fence of the receiver, words sent behind it and a fence of
+// the sender behind those words' arrival lie in between: twice the lag.
+constexpr int kWordBuffers = 4;
+constexpr int kWordFenceLag = 2;
+QAA_HD constexpr int word_buffer(int j) { return j % kWordBuffers; }
+static_assert(kWordBuffers >= 2 * kWordFenceLag, "a fence on both sides between the emptying of a slot and its next use");
+
 }  // namespace qaa

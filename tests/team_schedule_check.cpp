@@ -6,15 +6,21 @@
 // threads only).  The accesses of several steps are laid out as the kernel makes them;
 // a happens-before relation is closed over program order, the CTA's barriers and the
 // arrival of sent words (a wait orders the waiting CTA behind the threads that sent to
-// it, no others).  Prints "ok" and exits 0, else prints the first violation and exits 1.
+// it, no others).
+//
+// Word form: the same two CTAs, each with a third thread that runs the fences.  Between
+// CTAs only a fence before the sent words and a fence behind their arrival order
+// anything: the arrival itself is a relaxed load.
+// Prints "ok" and exits 0, else prints the first violation and exits 1.
 #include <cstdio>
+#include <utility>
 #include <vector>
 
 #include "team_schedule.h"
 
 namespace {
 
-constexpr int kSteps = 7;
+constexpr int kSteps = 11;
 
 struct Event {
   int cta, thread, step;
@@ -26,6 +32,7 @@ struct Event {
 struct Graph {
   std::vector<Event> ev;
   std::vector<std::vector<int>> next;
+  std::vector<std::pair<int, int>> own;  // a store and the take that waits for its word
   int last[2][3];
   Graph() {
     for (auto& c : last)
@@ -69,7 +76,9 @@ struct Graph {
         if (x.buffer < 0 || x.buffer != y.buffer || x.mem_cta != y.mem_cta || !(x.write || y.write)) continue;
         // threads write parts of their own of one transpose or exchange
         if (x.write && y.write && x.step == y.step && x.what == y.what) continue;
-        if (!reach[a][b] && !reach[b][a]) {
+        bool word = false;
+        for (const auto& p : own) word = word || (p.first == static_cast<int>(a) && p.second == static_cast<int>(b));
+        if (!word && !reach[a][b] && !reach[b][a]) {
           std::printf("%s: buffer %d of CTA %d: %s of CTA %d thread %d step %d and %s of CTA %d thread %d step %d unordered\n", form,
                       x.buffer, x.mem_cta, x.what, x.cta, x.thread, x.step, y.what, y.cta, y.thread, y.step);
           return 1;
@@ -105,10 +114,40 @@ int cluster() {
   return g.check("cluster");
 }
 
+int words() {
+  Graph g;
+  int fence[2][kSteps], leave[2][kSteps];  // the fence warp's fence and its release of step j
+  int sent[2][2];                          // [receiver][sender], this step's
+  for (int j = 0; j < kSteps; ++j) {
+    g.barrier(j, 2);  // of the transposes
+    if (j >= qaa::kWordFenceLag)
+      for (int c = 0; c < 2; ++c)
+        for (int t = 0; t < 2; ++t) g.next[leave[c][j - qaa::kWordFenceLag]].push_back(g.add({c, t, j, "await fence", c, -1, false}));
+    // slot of a buffer: by sender; thread s of the receiver takes the words of CTA s
+    auto slot = [&](int sender) { return 2 * qaa::word_buffer(j) + sender; };
+    for (int c = 0; c < 2; ++c)
+      for (int t = 0; t < 2; ++t) sent[t][c] = g.add({c, t, j, "store", t, slot(c), true});
+    for (int c = 0; c < 2; ++c)
+      for (int t = 0; t < 2; ++t) g.own.push_back({sent[c][t], g.add({c, t, j, "take and empty", c, slot(t), true})});
+    // the threads arrive, the fence warp waits for them
+    for (int c = 0; c < 2; ++c) {
+      const int a0 = g.add({c, 0, j, "arrive", c, -1, false}), a1 = g.add({c, 1, j, "arrive", c, -1, false});
+      fence[c][j] = g.add({c, 2, j, "fence", c, -1, false});
+      g.next[a0].push_back(fence[c][j]);
+      g.next[a1].push_back(fence[c][j]);
+    }
+    for (int c = 0; c < 2; ++c) leave[c][j] = g.add({c, 2, j, "release", c, -1, false});
+  }
+  // a fence of the sender before a word it sends, and a fence of the receiver behind it
+  for (int r = 0; r < 2; ++r)
+    for (int j = qaa::kWordFenceLag; j < kSteps; ++j) g.next[fence[1 - r][j - qaa::kWordFenceLag]].push_back(fence[r][j]);
+  return g.check("words");
+}
+
 }  // namespace
 
 int main() {
-  if (cluster()) return 1;
+  if (cluster() || words()) return 1;
   std::puts("ok");
   return 0;
 }
