@@ -138,11 +138,44 @@ __device__ __forceinline__ void reg_turn(float2 (&v)[N], const RotCoef& c) {
   if (c.twice) turn_once<B0, B1, N, PAIRS>(v, c);
 }
 
+template <int N>
+__device__ __forceinline__ void scale_by(float2 (&v)[N], float k) {
+  const unsigned long long kk = f2_bits(make_float2(k, k));
+#pragma unroll
+  for (int r = 0; r < N; ++r) v[r] = fma2(kk, v[r], v[r]);
+}
+template <int N>
+__device__ __forceinline__ void scale_pow2(float2 (&v)[N], float p) {
+  if (p == 1.0f) return;
+  const unsigned long long pp = f2_bits(make_float2(p, p));
+#pragma unroll
+  for (int r = 0; r < N; ++r) v[r] = mul2(pp, v[r]);
+}
+
 // A register tile with the increments since its last rounding kept apart: the
 // value is v + d.  A step's turns and phases are small changes, so d is computed to
-// 2^-24 of itself and an amplitude rounds once per settle() instead of once or
-// twice per turn and phase.  Where most of the weight sits in a few amplitudes
+// 2^-24 of itself, where rounding the amplitude in every turn and phase would round it
+// to 2^-24 of itself each time.  Where most of the weight sits in a few amplitudes
 // their rounding is the error of the ground-state probability and of <H_P>.
+//
+// What a rounding leaves out, at most 2^-24 of the value, is kept in 8 bits of itself (a
+// bfloat16 pair).
+__device__ __forceinline__ unsigned pack_rest(float2 e) {
+  unsigned p;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p) : "f"(e.y), "f"(e.x));
+  return p;
+}
+__device__ __forceinline__ float2 unpack_rest(unsigned p) {
+  return make_float2(__uint_as_float(p << 16), __uint_as_float(p & 0xffff0000u));
+}
+template <int N>
+__device__ __forceinline__ void scale_rest(unsigned (&rest)[N], float f) {
+#pragma unroll
+  for (int r = 0; r < N; ++r) {
+    const float2 e = unpack_rest(rest[r]);
+    rest[r] = pack_rest(make_float2(f * e.x, f * e.y));
+  }
+}
 template <int N>
 struct Inc {
   float2 v[N], d[N];
@@ -156,11 +189,61 @@ struct Inc {
     for (int r = 0; r < N; ++r) v[r] = at(r);
     zero();
   }
-  // Turns of the register-index bits [B0, B1); `fresh`: d is zero.
+  // v <- the rounded v + d, d <- what the rounding left out (exact for |d| <= |v|).
+  __device__ __forceinline__ void carry() {
+#pragma unroll
+    for (int r = 0; r < N; ++r) {
+      const float2 t = at(r);
+      d[r] = sub2(d[r], sub2(t, v[r]));
+      v[r] = t;
+    }
+  }
+  // Before v alone leaves the thread: v <- the rounded v + d + left, left <- what the
+  // rounding left out, d <- 0.
+  __device__ __forceinline__ void leave(unsigned (&left)[N]) {
+#pragma unroll
+    for (int r = 0; r < N; ++r) {
+      const float2 s = add2(d[r], unpack_rest(left[r])), t = add2(v[r], s);
+      left[r] = pack_rest(sub2(s, sub2(t, v[r])));
+      v[r] = t;
+    }
+    zero();
+  }
+  // The value times 1 + k.
+  __device__ __forceinline__ void grow(float k) {
+    const unsigned long long kk = f2_bits(make_float2(k, k));
+#pragma unroll
+    for (int r = 0; r < N; ++r) d[r] = fma2(kk, at(r), d[r]);
+  }
+  // The value times a power of two.
+  __device__ __forceinline__ void scale(float p) {
+    scale_pow2<N>(v, p);
+    scale_pow2<N>(d, p);
+  }
+  // Turns of the register-index bits [B0, B1), two at a time as in turn_once; `fresh`:
+  // d is zero.
   template <int B0, int B1>
   __device__ __forceinline__ void once(const RotCoef& c, bool fresh) {
 #pragma unroll
-    for (int b = B0; b < B1; ++b) {
+    for (int b = B0; b + 1 < B1; b += 2) {
+      const int p = 1 << b, q = 2 << b;
+#pragma unroll
+      for (int r = 0; r < N; ++r) {
+        if (!(r & (p | q))) {
+          const bool first = fresh && b == B0;
+          const float2 a0 = first ? v[r] : at(r), a1 = first ? v[r | p] : at(r | p);
+          const float2 a2 = first ? v[r | q] : at(r | q), a3 = first ? v[r | p | q] : at(r | p | q);
+          const float2 s = add2(a1, a2), e = sub2(a3, a0);
+          const float2 i0 = fma2(c.b, a3, s), i1 = fma2(c.nb, a2, e), i2 = fma2(c.nb, a1, e), i3 = fma2(c.nb, a0, s);
+          d[r] = first ? mul2(c.b, i0) : fma2(c.b, i0, d[r]);
+          d[r | p] = first ? mul2(c.b, i1) : fma2(c.b, i1, d[r | p]);
+          d[r | q] = first ? mul2(c.b, i2) : fma2(c.b, i2, d[r | q]);
+          d[r | p | q] = first ? mul2(c.nb, i3) : fma2(c.nb, i3, d[r | p | q]);
+        }
+      }
+    }
+#pragma unroll
+    for (int b = B1 - (B1 - B0) % 2; b < B1; ++b) {
 #pragma unroll
       for (int r = 0; r < N; ++r) {
         if (!(r & (1 << b))) {
@@ -538,20 +621,6 @@ struct TurnScale {
     return k;
   }
 };
-template <int N>
-__device__ __forceinline__ void scale_by(float2 (&v)[N], float k) {
-  const unsigned long long kk = f2_bits(make_float2(k, k));
-#pragma unroll
-  for (int r = 0; r < N; ++r) v[r] = fma2(kk, v[r], v[r]);
-}
-template <int N>
-__device__ __forceinline__ void scale_pow2(float2 (&v)[N], float p) {
-  if (p == 1.0f) return;
-  const unsigned long long pp = f2_bits(make_float2(p, p));
-#pragma unroll
-  for (int r = 0; r < N; ++r) v[r] = mul2(pp, v[r]);
-}
-
 // Write the block's partial: the double-float sum of one pair per thread in a
 // fixed order; block 0 also writes the partial count.  Contains
 // __syncthreads: every thread of the block must call it.

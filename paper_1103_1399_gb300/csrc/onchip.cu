@@ -18,8 +18,8 @@
 // n = 12, by the latency of a step's two barriers.  The earlier form (W B W in
 // columns of 32 amplitudes, 24 butterfly levels, four shared-memory rounds and
 // P rows from global memory) had 2^(n-5) threads busy.  Measured, us per step of
-// a 400-step run, before and after: n = 6 1.76 / 0.48, n = 9 1.83 / 0.77, n = 11
-// 3.09 / 1.19 (from n = 12 on a single run takes a cluster, team.cu; batches keep one
+// a 400-step run, before and after: n = 6 1.76 / 0.33, n = 9 1.83 / 0.79, n = 11
+// 3.00 / 1.36 (1.19 when the increments were rounded away at every window; from n = 12 on a single run takes a cluster, team.cu; batches keep one
 // CTA per instance).
 // Phase rows come through a ring of cp.async copies issued kCtaRing - 1 steps ahead.
 #include "tile.cuh"
@@ -92,16 +92,16 @@ __device__ void warp_run(const RunArgs& A, unsigned char* smem) {
   };
 #pragma unroll
   for (int k = 0; k < kAhead; ++k) load(k, k);
-  auto warp_norm = [&]() { return warp_sum(norm_of<N>(v)); };
+  auto warp_norm = [&]() { return warp_sum(norm_of<N>(x)); };
+  x.zero();
   const DFloat nref = warp_norm();
   const int pc = __popc(lane);
 #pragma unroll
   for (int r = 0; r < N; ++r) v[r] = times_i(v[r], pc + __popc(r));
   if (A.first_p) {
 #pragma unroll
-    for (int r = 0; r < N; ++r) v[r] = add2(v[r], cmac(make_float2(0.f, 0.f), v[r], A.ptab[ev[r]]));
+    for (int r = 0; r < N; ++r) x.d[r] = cmac(x.d[r], v[r], A.ptab[ev[r]]);
   }
-  x.zero();
   TurnScale ts;
   for (int j0 = 0; j0 < A.nsteps; j0 += kAhead) {
 #pragma unroll
@@ -109,7 +109,7 @@ __device__ void warp_run(const RunArgs& A, unsigned char* smem) {
       const int j = j0 + k;
       if (j >= A.nsteps) break;
       const RotCoef c = rot_coef(row[k]);
-      if constexpr (N >= 2) x.template turn<0, (N >= 8 ? 3 : (N >= 4 ? 2 : 1))>(c, true);
+      if constexpr (N >= 2) x.template turn<0, (N >= 8 ? 3 : (N >= 4 ? 2 : 1))>(c);
       auto lanes = [&]() {
 #pragma unroll
         for (int b = 0; b < 5; ++b) {
@@ -132,17 +132,17 @@ __device__ void warp_run(const RunArgs& A, unsigned char* smem) {
 #pragma unroll
       for (int r = 0; r < N; ++r) x.d[r] = cmac(x.d[r], x.at(r), z[k][r]);
       load(k, j + kAhead);
-      x.settle();
-      scale_pow2<N>(v, c.pow2);
+      x.carry();
+      x.scale(c.pow2);
       // every fold_period(n)-th step and the last
       ts.step(c.r);
       if ((j + 1) % fold_period(1) == 0 || j + 1 == A.nsteps)
-        scale_by<N>(v, __shfl_sync(0xffffffffu, ts.fold(nref, warp_norm()), 0));
+        x.grow(__shfl_sync(0xffffffffu, ts.fold(nref, warp_norm()), 0));
     }
   }
   if (mine) {
 #pragma unroll
-    for (int r = 0; r < N; ++r) A.psi[lane + 32 * r] = times_i(v[r], -(pc + __popc(r)));
+    for (int r = 0; r < N; ++r) A.psi[lane + 32 * r] = times_i(x.at(r), -(pc + __popc(r)));
   }
 }
 
@@ -195,7 +195,7 @@ __device__ void window_energies(const ClauseMV* __restrict__ cl, int m, uint4* s
 template <int T, int R>
 __host__ __device__ inline size_t cta_smem(int m) {
   using G = CtaGeom<T, R>;
-  const size_t buf = (8u * static_cast<size_t>(G::SLOTS) * (G::kTwoBuffers ? 2 : 1) + 15u) & ~static_cast<size_t>(15);
+  const size_t buf = (tile_bytes<T, R, (R < 5)>() * (G::kTwoBuffers ? 2 : 1) + 15u) & ~static_cast<size_t>(15);
   const size_t ent = 16u * static_cast<size_t>((m + 15) & ~15);  // the buffers hold the clause tables first
   return (buf > ent ? buf : ent) + 8u * kCtaRing * static_cast<size_t>(m + 3);
 }
@@ -232,13 +232,13 @@ __device__ void cta_run(const RunArgs& A, unsigned char* smem) {
   unsigned et[N / 2], em[N / 2];
   window_energies<R, NT>(A.cl, A.m, reinterpret_cast<uint4*>(smem), T - R, xt, tid, et);
   window_energies<R, NT>(A.cl, A.m, reinterpret_cast<uint4*>(smem), R, xm, tid, em);
-  const DFloat nref = cta_norm<NT>(norm_of<N>(v), s_w, tid);  // also ends the use of s_buf as the clause tables
+  x.zero();
+  const DFloat nref = cta_norm<NT>(norm_of<N>(x), s_w, tid);  // also ends the use of s_buf as the clause tables
 #pragma unroll
   for (int r = 0; r < N; ++r) v[r] = times_i(v[r], __popc(xt) + __popc(r));
-  if (A.first_p) apply_rows<N>(v, et, A.ptab);
-  x.zero();
+  if (A.first_p) x.phase(et, A.ptab);
   float2* b0 = s_buf;
-  float2* b1 = s_buf + (G::kTwoBuffers ? G::SLOTS : 0);
+  float2* b1 = s_buf + (G::kTwoBuffers ? tile_bytes<T, R, (R < 5)>() / 8 : 0);
   TurnScale ts;
   cp_async_wait<1>();
   team_sync<NT>();  // the first rotation is in
@@ -249,47 +249,40 @@ __device__ void cta_run(const RunArgs& A, unsigned char* smem) {
     const bool down = !(j & 1);
     if (down) {
       x.template turn<0, R>(c);
-      x.settle();
-      put<T, R, kTop>(v, b0, tid);
+      put_tile<T, R, kTop>(x, b0, tid);
     } else {
       x.template turn<0, T - 2 * R>(c);
-      x.settle();
-      put<T, R, kMid>(v, b0, tid);
+      put_tile<T, R, kMid>(x, b0, tid);
     }
     cp_async_wait<1>();  // rows up to step j + 1, visible to all beyond the barrier
     team_sync<NT>();
     fetch_rows<NT, kCtaRing>(A, s_p, s_ab, j + kCtaRing - 1, tid);  // into the slot of step j - 1, which all have left
-    get<T, R, kBot>(v, b0, tid);
+    get_tile<T, R, kBot>(x, b0, tid);
     if (!G::kTwoBuffers) team_sync<NT>();
-    x.template turn<0, R>(c, true);
-    x.settle();
-    put<T, R, kBot>(v, b1, tid);
+    x.template turn<0, R>(c);
+    put_tile<T, R, kBot>(x, b1, tid);
     team_sync<NT>();
     if (down) {
-      get<T, R, kMid>(v, b1, tid);
-      x.template turn<0, T - 2 * R>(c, true);
+      get_tile<T, R, kMid>(x, b1, tid);
+      x.template turn<0, T - 2 * R>(c);
       x.phase(em, prow);
     } else {
-      get<T, R, kTop>(v, b1, tid);
-      x.template turn<0, R>(c, true);
+      get_tile<T, R, kTop>(x, b1, tid);
+      x.template turn<0, R>(c);
       x.phase(et, prow);
     }
-    if (c.pow2 != 1.0f) {
-      x.settle();
-      scale_pow2<N>(v, c.pow2);
-    }
+    x.carry();
+    if (c.pow2 != 1.0f) x.scale(c.pow2);
     ts.step(c.r);
-    if ((j + 1) % fold_period(T) == 0 || j + 1 == A.nsteps) {
-      x.settle();
-      scale_by<N>(v, ts.fold(nref, cta_norm<NT>(norm_of<N>(v), s_w, tid)));
-    }
+    if ((j + 1) % fold_period(T) == 0 || j + 1 == A.nsteps)
+      x.grow(ts.fold(nref, cta_norm<NT>(norm_of<N>(x), s_w, tid)));
   }
   if (A.nsteps & 1) {
 #pragma unroll
-    for (int r = 0; r < N; ++r) A.psi[xm + (r << R)] = times_i(v[r], -(__popc(xm) + __popc(r)));
+    for (int r = 0; r < N; ++r) A.psi[xm + (r << R)] = times_i(x.at(r), -(__popc(xm) + __popc(r)));
   } else {
 #pragma unroll
-    for (int r = 0; r < N; ++r) A.psi[xt + (r << (T - R))] = times_i(v[r], -(__popc(xt) + __popc(r)));
+    for (int r = 0; r < N; ++r) A.psi[xt + (r << (T - R))] = times_i(x.at(r), -(__popc(xt) + __popc(r)));
   }
 }
 

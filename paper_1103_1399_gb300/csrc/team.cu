@@ -168,9 +168,6 @@ struct TeamGeom : CtaGeom<T, R> {
   static constexpr int kOut = kSplit ? kTop : kMid;   // window that sends
   static_assert(D >= 0 && (!kSplit || D >= R), "incoming bits must lie in TOP and MID");
   static_assert(!CLUSTER || C <= 3, "portable clusters of 8 CTAs");
-  // cluster: two transpose and two receive buffers; grid: two transpose buffers, one
-  // for 2^14 amplitudes
-  static constexpr int kBufs = CLUSTER ? kClusterBuffers : (T <= 13 ? 2 : 1);
   // grid: self-validating words, with a warp of its own for the fence that orders
   // the emptied slots; 512 threads with 32 amplitudes each (2^14 per CTA) use the
   // grid barrier: the words' second set of stores and registers cost more there
@@ -178,13 +175,27 @@ struct TeamGeom : CtaGeom<T, R> {
   static constexpr bool kWords = !CLUSTER && G::NT < 512;
   static constexpr int kThreads = G::NT + (kWords ? 32 : 0);
   static constexpr int kPerSm = C >= 8 ? 2 : 1;
-  static constexpr bool kInc = R < 5 && kPerSm == 1;  // registers for the increments
+  // increments beside the values where there are registers for them (two CTAs per SM
+  // with a fence warp each leave 96 per thread)
+  static constexpr bool kInc = R < 5 && kPerSm == 1;
+  // What the rounding before the exchange leaves out stays in registers and is taken up
+  // two steps on, when the amplitude is in the same layout, thread and register again.
+  // Its turn in between is ignored: at angles that are not small it is one more error of
+  // the size of the rounding.  The scales of the steps in between are not: they reach
+  // 2^-n.
+  static constexpr bool kLeft = kInc && kPerSm == 1;
+  // transpose buffers: two where they fit (one barrier per transpose instead of two);
+  // the cluster's receive buffers lie behind them
+  static constexpr int kBufs = (kPerSm == 2 && kInc) || T > 13 ? 1 : 2;
+  static_assert(!CLUSTER || kBufs == 2, "team_schedule.h");
+  static constexpr size_t kTile = (tile_bytes<T, R, kInc>() + 15u) / 16u * 16u;
+  static constexpr size_t kBytes = kTile * kBufs + (CLUSTER ? (kClusterBuffers - 2) * 8u * static_cast<size_t>(G::SLOTS) : 0u);
 };
 
 template <int T, int R, int C, bool CLUSTER>
 size_t team_smem(int m) {
   using G = TeamGeom<T, R, C, CLUSTER>;
-  return 8u * static_cast<size_t>(G::SLOTS) * G::kBufs + 8u * kTeamRing * static_cast<size_t>(m + 3);
+  return G::kBytes + 8u * kTeamRing * static_cast<size_t>(m + 3);
 }
 
 template <int T, int R, int C, bool CLUSTER>
@@ -201,7 +212,7 @@ __global__ void __launch_bounds__(TeamGeom<T, R, C, CLUSTER>::kThreads, (TeamGeo
   const unsigned cta = CLUSTER ? cluster_rank() : blockIdx.x;
   const int mp1 = A.m + 1;
   float2* s_buf = reinterpret_cast<float2*>(smem);
-  float2* s_ab = s_buf + static_cast<size_t>(G::SLOTS) * G::kBufs;
+  float2* s_ab = s_buf + G::kBytes / 8;
   float2* s_p = s_ab + 2 * kTeamRing;
   auto fetch = [&](int j) {
     if (j < A.nsteps) {
@@ -248,7 +259,7 @@ __global__ void __launch_bounds__(TeamGeom<T, R, C, CLUSTER>::kThreads, (TeamGeo
 
   // a warp's sum of |v|^2 for the CTA's partial
   auto measure = [&]() {
-    const DFloat t = warp_sum(norm_of<N>(v));
+    const DFloat t = warp_sum(norm_of<N>(x));
     if ((tid & 31) == 0) s_w[tid >> 5] = t;
   };
   // the CTA's partial to every CTA of the team (one warp, after a barrier since measure)
@@ -290,11 +301,11 @@ __global__ void __launch_bounds__(TeamGeom<T, R, C, CLUSTER>::kThreads, (TeamGeo
     const float2 r = __ldcg(A.ref);
     ref = DFloat{r.x, r.y};
   }
+  x.zero();
   measure();
 #pragma unroll
   for (int r = 0; r < N; ++r) v[r] = times_i(v[r], pc + __popc(r));
-  if (A.first) apply_rows<N>(v, ea, A.ptab);
-  x.zero();
+  if (A.first) x.phase(ea, A.ptab);
 
   // the bytes that arrive in step j
   auto expect = [&](int j) {
@@ -320,7 +331,11 @@ __global__ void __launch_bounds__(TeamGeom<T, R, C, CLUSTER>::kThreads, (TeamGeo
 
   // transposes through one or two buffers; `b` alternates so that one barrier is enough
   int b = 0;
-  auto buffer = [&](int k) { return s_buf + static_cast<size_t>(G::SLOTS) * k; };
+  auto buffer = [&](int k) { return s_buf + G::kTile / 8 * k; };
+  auto receive = [&](int j) {  // cluster
+    return s_buf + G::kTile / 8 * 2 + static_cast<size_t>(G::SLOTS) * (cluster_receive(j) - 2);
+  };
+  unsigned left[2][G::kLeft ? N : 1] = {};  // by layout
   bool late = false;
   TurnScale ts;
   for (int j = 0; j < A.nsteps; ++j) {
@@ -338,8 +353,7 @@ __global__ void __launch_bounds__(TeamGeom<T, R, C, CLUSTER>::kThreads, (TeamGeo
     };
     if constexpr (!G::kSplit) {
       x.template turn<0, R>(c);
-      x.settle();
-      put<T, R, kTop>(v, b0, tid);
+      put_tile<T, R, kTop>(x, b0, tid);
       middle();
       if (G::kWords && late) {
         bar_arrive<2, NT + 32>();  // the fence warp may be waiting for this step's
@@ -347,20 +361,17 @@ __global__ void __launch_bounds__(TeamGeom<T, R, C, CLUSTER>::kThreads, (TeamGeo
       }
       if (pending && tid < 32) publish(j & 1, 0);
       fetch(j + kTeamRing - 1);
-      get<T, R, kBot>(v, b0, tid);
+      get_tile<T, R, kBot>(x, b0, tid);
       reuse();
-      x.template turn<0, R>(c, true);
-      x.settle();
-      put<T, R, kBot>(v, b1, tid);
+      x.template turn<0, R>(c);
+      put_tile<T, R, kBot>(x, b1, tid);
       team_sync<NT>();
-      get<T, R, kMid>(v, b1, tid);
+      get_tile<T, R, kMid>(x, b1, tid);
       reuse();
-      x.template turn<0, T - 2 * R>(c, true);
-      x.settle();
+      x.template turn<0, T - 2 * R>(c);
     } else {
       x.template turn<0, T - 2 * R>(c);
-      x.settle();
-      put<T, R, kMid>(v, b0, tid);
+      put_tile<T, R, kMid>(x, b0, tid);
       middle();
       if (G::kWords && late) {
         bar_arrive<2, NT + 32>();  // the fence warp may be waiting for this step's
@@ -368,17 +379,22 @@ __global__ void __launch_bounds__(TeamGeom<T, R, C, CLUSTER>::kThreads, (TeamGeo
       }
       if (pending && tid < 32) publish(j & 1, 0);
       fetch(j + kTeamRing - 1);
-      get<T, R, kBot>(v, b0, tid);
+      get_tile<T, R, kBot>(x, b0, tid);
       reuse();
-      x.template turn<0, R>(c, true);
-      x.settle();
-      put<T, R, kBot>(v, b1, tid);
+      x.template turn<0, R>(c);
+      put_tile<T, R, kBot>(x, b1, tid);
       team_sync<NT>();
-      get<T, R, kTop>(v, b1, tid);
+      get_tile<T, R, kTop>(x, b1, tid);
       reuse();
-      x.template turn<0, R>(c, true);
-      x.settle();
+      x.template turn<0, R>(c);
     }
+    // only the values leave: the one rounding of an amplitude per step
+    if constexpr (!G::kLeft)
+      x.settle();
+    else if (j & 1)
+      x.leave(left[1]);
+    else
+      x.leave(left[0]);
     // exchange: tile index l -> CTA l >> D, slot (l mod 2^D) | cta << D
     {
       const int l0 = win_base<T, R, kOut>(tid);
@@ -386,7 +402,7 @@ __global__ void __launch_bounds__(TeamGeom<T, R, C, CLUSTER>::kThreads, (TeamGeo
       constexpr int dm = (1 << D) - 1;
       const bool lost = A.lose && cta == 0 && j == 0;
       if constexpr (CLUSTER) {
-        float2* dst = buffer(cluster_receive(j)) + G::slot((l0 & dm) | static_cast<int>(cta) << D);
+        float2* dst = receive(j) + G::slot((l0 & dm) | static_cast<int>(cta) << D);
         if (!lost) {
 #pragma unroll
           for (int r = 0; r < N; ++r)
@@ -397,7 +413,7 @@ __global__ void __launch_bounds__(TeamGeom<T, R, C, CLUSTER>::kThreads, (TeamGeo
         late = __syncthreads_or(!recv_wait(s_bar + (j & 1), (j >> 1) & 1, A.polls)) != 0;
         if (late) break;
         if (tid == 0 && j + 2 < A.nsteps) expect(j + 2);
-        get<T, R, kTop>(v, buffer(cluster_receive(j)), tid);
+        get<T, R, kTop>(v, receive(j), tid);
       } else {
         float2* xb = A.xbuf + (static_cast<size_t>(G::kWords ? word_buffer(j) : j & 1) << A.n);
         float2* dst = xb + (static_cast<size_t>(l0 >> D) << T) + ((l0 & dm) | static_cast<int>(cta) << D);
@@ -440,27 +456,27 @@ __global__ void __launch_bounds__(TeamGeom<T, R, C, CLUSTER>::kThreads, (TeamGeo
       x.template turn<R - C, R>(c, true);
     } else {
       x.template turn<0, R>(c, true);
-      x.settle();
       float2* b2 = buffer(b);
-      put<T, R, kTop>(v, b2, tid);
+      put_tile<T, R, kTop>(x, b2, tid);
       team_sync<NT>();
-      get<T, R, kMid>(v, b2, tid);
+      get_tile<T, R, kMid>(x, b2, tid);
       reuse();
-      x.template turn<D - R, T - 2 * R>(c, true);
+      x.template turn<D - R, T - 2 * R>(c);
       if (G::kBufs == 2) b ^= 1;
     }
     if (j & 1)
       x.phase(ea, prow);
     else
       x.phase(eb, prow);
-    if (c.pow2 != 1.0f || k != 0.f) {
-      x.settle();
-      scale_pow2<N>(v, c.pow2);
-      scale_by<N>(v, k);
+    if (c.pow2 != 1.0f) x.scale(c.pow2);
+    if (k != 0.f) x.grow(k);
+    if (G::kLeft && (c.pow2 != 1.0f || k != 0.f)) {
+      const float f = fmaf(c.pow2, k, c.pow2);
+      scale_rest(left[0], f);
+      scale_rest(left[1], f);
     }
     ts.step(c.r);
     if ((j + 1) % fold_period(T + C) == 0 && j + 1 < A.nsteps) {
-      x.settle();
       measure();
       pending = true;
     }
@@ -471,24 +487,23 @@ __global__ void __launch_bounds__(TeamGeom<T, R, C, CLUSTER>::kThreads, (TeamGeo
     late = late || *static_cast<volatile int*>(&s_late) != 0;
   }
   if (!late) {  // the same in every thread of the CTA
-    x.settle();
     measure();
     team_sync<NT>();
     if (tid < 32) publish(2, 1);
     if (CLUSTER) {
       late = __syncthreads_or(!recv_wait(s_bar + 2, 0, A.polls)) != 0;
     }
-    scale_by<N>(v, ts.fold(ref, collect(1)));
+    x.grow(ts.fold(ref, collect(1)));
     if (!CLUSTER) late = *static_cast<volatile int*>(&s_late) != 0;
   }
   if (late && (CLUSTER || tid == 0)) atomicExch(A.err, 2);
   if (CLUSTER) cluster_barrier();  // no CTA leaves while another may still store into its shared memory
   if (A.nsteps & 1) {
 #pragma unroll
-    for (int r = 0; r < N; ++r) A.psi[index_b(lp + r * lstep)] = times_i(v[r], -(pc + __popc(r)));
+    for (int r = 0; r < N; ++r) A.psi[index_b(lp + r * lstep)] = times_i(x.at(r), -(pc + __popc(r)));
   } else {
 #pragma unroll
-    for (int r = 0; r < N; ++r) A.psi[xa + r * lstep] = times_i(v[r], -(pc + __popc(r)));
+    for (int r = 0; r < N; ++r) A.psi[xa + r * lstep] = times_i(x.at(r), -(pc + __popc(r)));
   }
 }
 
@@ -551,8 +566,8 @@ bool fits(int num_sms, int m) {
 
 // The team of each n: tile bits T, register bits R, CTA bits C.  Small tiles win
 // up to the exchange's latency.  us per step of a 200-step run, the launch included,
-// of the choices tried (with single turns; the rounding of Inc and of the paired
-// turns adds 5 to 15 %):
+// of the choices tried (with single turns; the increments beside the amplitudes and
+// the paired turns add up to 30 %):
 //   n = 12 cluster (9,3) 1.20, one CTA 1.39      n = 13 cluster (10,4) 1.51, one CTA 2.39
 //   n = 14 cluster (11,4) 2.01, grid (9,3) 2.05, (10,4) 2.39, one CTA 4.79
 //   n = 15 grid (9,3) 2.08, (10,4) 2.49, (11,4) 2.62, cluster (12,4) 3.09
@@ -561,9 +576,15 @@ bool fits(int num_sms, int m) {
 //   n = 19 grid (12,4) 4.08, (13,5) 6.51
 //   n = 20 grid (12,4) with two CTAs per SM 6.36, (13,5) 6.65    n = 21 grid (14,5) 11.5
 // The kernels as they are, 400 steps, against the streaming passes (n = 12..14: the
-// earlier one-CTA kernel): n = 12 1.26 / 3.23, 13 1.69 / 4.85, 14 2.16 / 8.60, 15 2.15 /
-// 12.4, 16 2.94 / 12.5, 17 3.06 / 13.2, 18 3.45 / 14.6, 19 4.44 / 14.8, 20 6.77 / 19.0,
-// 21 13.1 / 25.1; the state's error against 64 bits 1.0e-6 / 3.0e-6 (n = 16).
+// earlier one-CTA kernel): n = 12 1.40 / 3.16, 13 1.88 / 4.85, 14 2.41 / 8.60, 15 2.30 /
+// 12.4, 16 3.04 / 12.4, 17 3.49 / 13.2, 18 3.71 / 14.6, 19 5.16 / 14.7, 20 6.58 / 18.8,
+// 21 12.3 / 24.9; the state's error against 64 bits 2e-7 / 3.2e-6 (n = 16).
+// Without the increments in the transposes (an amplitude rounded at every window) n = 16
+// took 2.94, n = 19 4.44, with four times the error of <H_P> and of the ground
+// probability; with what a rounding leaves out packed into 4 bytes instead n = 16 3.51,
+// n = 19 5.08.  n = 20 and 21 have no registers for them (n = 20 so 9.1): every pair of
+// turns rounds, and the errors are about half of the streaming passes' (n = 20, 200
+// steps, rms of 8 instances: state 1.2e-6, <H_P> 9e-8, ground probability 3.9e-7).
 // n <= 11 stays with one CTA (0.94 at n = 11 against 1.07 in a cluster); 2^22
 // amplitudes do not fit in the registers.
 #define QAA_TEAMS(X)                                                                                       \

@@ -59,33 +59,39 @@ struct Tile;
 template <int N>
 struct Tile<N, false> {
   float2 v[N];
+  __device__ __forceinline__ float2 at(int r) const { return v[r]; }
   template <int B0, int B1>
   __device__ __forceinline__ void turn(const RotCoef& c, bool = false) {
     reg_turn<B0, B1>(v, c);
   }
   __device__ __forceinline__ void phase(const unsigned (&e)[(N + 1) / 2], const float2* prow) { apply_rows<N>(v, e, prow); }
+  __device__ __forceinline__ void carry() {}
   __device__ __forceinline__ void settle() {}
   __device__ __forceinline__ void zero() {}
+  __device__ __forceinline__ void grow(float k) { scale_by<N>(v, k); }
+  __device__ __forceinline__ void scale(float p) { scale_pow2<N>(v, p); }
 };
 template <int N>
 struct Tile<N, true> : Inc<N> {
   __device__ __forceinline__ void phase(const unsigned (&e)[(N + 1) / 2], const float2* prow) { apply_rows<N>(*this, e, prow); }
 };
 
-// |v|^2 over a thread's amplitudes as a double-float: every square as its FP32
-// product and that product's exact error, the products summed by TwoSum.  A plain
-// FP32 sum would be biased by up to 4e-7 on a uniform state (every thread adds the
-// same numbers and rounds the same way), and with it the norm a run is held to.
-template <int N>
-__device__ __forceinline__ DFloat norm_of(const float2 (&v)[N]) {
+// |x|^2 over a thread's N amplitudes (an Inc's as rounded) as a double-float: every
+// square as its FP32 product and that product's exact error, the products summed by
+// TwoSum.  A plain FP32 sum would be biased by up to 4e-7 on a uniform state (every
+// thread adds the same numbers and rounds the same way), and with it the norm a run
+// is held to.
+template <int N, class X>
+__device__ __forceinline__ DFloat norm_of(const X& x) {
   float s = 0.f, e = 0.f;
 #pragma unroll
   for (int r = 0; r < N; ++r) {
+    const float2 v = x.at(r);
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
-      const float x = k ? v[r].y : v[r].x;
-      const float p = x * x, t = s + p, bb = t - s;
-      e += ((s - (t - bb)) + (p - bb)) + fmaf(x, x, -p);
+      const float a = k ? v.y : v.x;
+      const float p = a * a, t = s + p, bb = t - s;
+      e += ((s - (t - bb)) + (p - bb)) + fmaf(a, a, -p);
       s = t;
     }
   }
@@ -136,6 +142,24 @@ __device__ __forceinline__ void get(float2 (&v)[1 << R], const float2* buf, int 
   const float2* p = buf + G::slot(win_base<T, R, W>(tid));
 #pragma unroll
   for (int r = 0; r < (1 << R); ++r) v[r] = p[G::slot(r * win_step<T, R, W>())];
+}
+// A tile's transposes: the increments, where there are any, travel with the values
+// (behind them in the buffer).  Rounding them into the values at every transpose
+// instead (three or four roundings per step) made the error of <H_P> as large as that of
+// turns rounded one by one: n = 16, 400 steps, 3.9e-7 rms over 8 instances; so 6e-8.
+template <int T, int R, bool INC>
+__host__ __device__ constexpr size_t tile_bytes() {
+  return (INC ? 16u : 8u) * static_cast<size_t>(CtaGeom<T, R>::SLOTS);
+}
+template <int T, int R, int W, bool INC>
+__device__ __forceinline__ void put_tile(const Tile<1 << R, INC>& x, float2* buf, int tid) {
+  put<T, R, W>(x.v, buf, tid);
+  if constexpr (INC) put<T, R, W>(x.d, buf + CtaGeom<T, R>::SLOTS, tid);
+}
+template <int T, int R, int W, bool INC>
+__device__ __forceinline__ void get_tile(Tile<1 << R, INC>& x, const float2* buf, int tid) {
+  get<T, R, W>(x.v, buf, tid);
+  if constexpr (INC) get<T, R, W>(x.d, buf + CtaGeom<T, R>::SLOTS, tid);
 }
 
 }  // namespace qaa
