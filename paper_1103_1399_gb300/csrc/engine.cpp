@@ -550,6 +550,7 @@ qaa_status qaa_set_variant(qaa_handle h, int wht_kind, int q) {
     qaa::make_default_plan(h->n, h->plan, q, low, wht_kind == qaa::kRotationForm);  // groups of at most q bits (the fewest such groups)
   else
     qaa::make_plan(h->n, h->plan, widest, wht_kind == qaa::kRotationForm);
+  h->plan.team = false;  // a variant is a form of the passes, also where the default (or a tuned) plan is a team
   // a plan made (or tuned) for the other form gets the run lengths of this one
   const bool same_form = (h->plan.wht_kind == qaa::kRotationForm) == (wht_kind == qaa::kRotationForm);
   h->plan.wht_kind = wht_kind;

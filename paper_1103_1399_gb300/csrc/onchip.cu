@@ -19,8 +19,8 @@
 // columns of 32 amplitudes, 24 butterfly levels, four shared-memory rounds and
 // P rows from global memory) had 2^(n-5) threads busy.  Measured, us per step of
 // a 400-step run, before and after: n = 6 1.76 / 0.33, n = 9 1.83 / 0.79, n = 11
-// 3.00 / 1.36 (1.19 when the increments were rounded away at every window; from n = 12 on a single run takes a cluster, team.cu; batches keep one
-// CTA per instance).
+// 3.00 / 1.36 (1.19 when the increments were rounded away at every window; from n =
+// 12 on a single run takes a cluster, team.cu; batches keep one CTA per instance).
 // Phase rows come through a ring of cp.async copies issued kCtaRing - 1 steps ahead.
 #include "tile.cuh"
 
