@@ -213,7 +213,7 @@ struct qaa_server {
   // default: on the n ~ U{10..22} mix it measured 202-210 solves/s (4 or 8
   // issuers) against 219 with per-pass launches from 4 issuers -- the graph
   // makes one request's steps faster but several n = 20..22 requests then
-  // contend for L2 and HBM at once.
+  // contend for L2 and HBM at once.  Requests that run on a team of CTAs have none.
   bool use_graphs = false;
   int graph_max_bits = 0;  // streamed requests with n <= this run as one launch graph
   // small-request batches
@@ -758,7 +758,7 @@ qaa_status qaa_submit(qaa_server* s, int n, const int32_t* clauses, int m, doubl
     if (!r->plan.onchip && !r->persist && r->plan.use_tma && n > qaa::kOnchipMaxBits && !(env && std::atoi(env) == 0))
       r->counts_bytes = qaa::lp_counts_bytes(n);
   }
-  // A team's scratch is three times the state: only where it is a small part of
+  // A team's scratch is four times the state: only where it is a small part of
   // the arena, so that it never decides whether a request fits.
   if (!r->plan.onchip && !r->persist && qaa::team_plan(r->plan) && qaa::team_fits(n, m, s->num_sms)) {
     const size_t tb = energy_bytes(n) + qaa::team_bytes(n);
