@@ -105,7 +105,16 @@ __host__ __device__ constexpr int tma_c(int q) { return (10 - q) > 3 ? (10 - q) 
 // layout-L stage is thread bit C, a lane bit, transformed by warp shuffles.
 // MODE 0: W over the group; 1: W B W (the phase group); 2: the one-qubit
 // rotations of exp(-i theta H_B) on the group's bits (rotation form, RotCoef), all of
-// them with times = 1; 3: the same for any angle.
+// them with times = 1; 3: the same for any angle.  LFIRST (rotations of 11 bits): layout
+// L comes first and the results are stored from layout H.  A warp's store of an 11-bit
+// tile covers four rows: from layout L four of the upper range, 2^a2 apart, from layout H
+// four of the lower one.  Where the upper range steps over memory pages (a2 >= kPageBits)
+// layout H is the better one to store from, and better still behind a fence and a barrier,
+// so that a tile's rows are written together (without the fence the last turns move
+// behind the barrier, between the stores); elsewhere layout L is.  ms a pass, stored from H
+// / L: n = 32 (a2 = 26 and 20) 11.5 (12.2 without the fence, 12.5 without both) / 12.8, n =
+// 33 25.4 / 26.5 (the mean of its three groups); n = 31 (a2 = 15; both groups) 6.18 / 6.07.
+constexpr int kPageBits = 18;  // 2 MiB of amplitudes
 //
 // Butterflies over lane bit LB: (u, w) <- (u + w, u - w) across the two lanes.
 template <int LB>
@@ -156,7 +165,7 @@ __device__ __forceinline__ void stage_l(float2 (&v)[32], const RotCoef& rc, int 
   }
 }
 
-template <int Q, int C, int MODE>
+template <int Q, int C, int MODE, bool LFIRST = false>
 __global__ void __launch_bounds__(TmaGeom<Q, C>::NT, (TmaGeom<Q, C>::NT >= 512 ? 1 : (TmaGeom<Q, C>::NT >= 256 ? 3 : 4)))
     sp_tma_kernel(float2* __restrict__ psi, const __grid_constant__ CUtensorMap tmap, int n, int a1, int a2,
                   const float2* __restrict__ brow, long long ntiles, int* __restrict__ err) {
@@ -211,17 +220,13 @@ __global__ void __launch_bounds__(TmaGeom<Q, C>::NT, (TmaGeom<Q, C>::NT >= 512 ?
     const unsigned long long ut = static_cast<unsigned long long>(T);
     const unsigned long long xbase = ((ut & lo_mask) << C) | (((ut >> lo_bits) & mid_mask) << (a1 + 5)) |
                                      ((ut >> (lo_bits + mid_bits)) << (a2 + QB));
-    // An 11-bit rotation pass takes layout L first and stores from layout H: a warp's
-    // store then covers four rows 2^a1 apart, on one page, instead of four rows of the
-    // upper range (n = 32 14.5 -> 12.5 ms a pass, n = 31 6.2 -> 6.6).
-    constexpr bool kLFirst = Q == 11 && MODE >= 2;
     float2 v[32];
     {
-      const float2* src = s_buf + (kLFirst ? j + (th << (C + 5)) : h_off);
+      const float2* src = s_buf + (LFIRST ? j + (th << (C + 5)) : h_off);
 #pragma unroll
-      for (int r = 0; r < 32; ++r) v[r] = src[kLFirst ? r << C : (r << QB) << C];
+      for (int r = 0; r < 32; ++r) v[r] = src[LFIRST ? r << C : (r << QB) << C];
     }
-    if (kLFirst)
+    if (LFIRST)
       stage_l<QB, C, MODE>(v, rc, lane);  // i bits 0..QB-1
     else
       turn_or_wht<5, MODE>(v, rc);  // i bits QB..QB+4
@@ -245,12 +250,12 @@ __global__ void __launch_bounds__(TmaGeom<Q, C>::NT, (TmaGeom<Q, C>::NT >= 512 ?
     if (QB > 0) {
       __syncthreads();  // dense tile fully read
 #pragma unroll
-      for (int r = 0; r < 32; ++r) s_buf[kLFirst ? sx_l + (r << C) : sx_h + G::slot((r << QB) << C)] = v[r];
+      for (int r = 0; r < 32; ++r) s_buf[LFIRST ? sx_l + (r << C) : sx_h + G::slot((r << QB) << C)] = v[r];
       __syncthreads();
 #pragma unroll
-      for (int r = 0; r < 32; ++r) v[r] = s_buf[kLFirst ? sx_h + G::slot((r << QB) << C) : sx_l + (r << C)];
+      for (int r = 0; r < 32; ++r) v[r] = s_buf[LFIRST ? sx_h + G::slot((r << QB) << C) : sx_l + (r << C)];
       if (kEarlyIssue) issue_next();
-      if (kLFirst)
+      if (LFIRST)
         turn_or_wht<5, MODE>(v, rc);  // i bits QB..QB+4
       else
         stage_l<QB, C, MODE>(v, rc, lane);  // i bits 0..QB-1
@@ -273,7 +278,11 @@ __global__ void __launch_bounds__(TmaGeom<Q, C>::NT, (TmaGeom<Q, C>::NT >= 512 ?
     }
     // the buffer is free: fetch the next tile while this one is stored
     if (!kEarlyIssue) issue_next();
-    if (WBW || QB == 0 || kLFirst) {
+    if (LFIRST) {
+      __threadfence_block();
+      __syncthreads();
+    }
+    if (WBW || QB == 0 || LFIRST) {
       // layout H: i = th + (r << QB); th = i bits 0..QB-1: bits 0..4 lie at a1.., bit 5 (QB = 6) at a2
       float2* dst = psi + xbase + j + (static_cast<unsigned long long>(th & 31) << a1) +
                     (static_cast<unsigned long long>(th >> 5) << a2);
@@ -699,6 +708,8 @@ static CUtensorMapL2promotion l2_promotion(int c) {
 // flight get in each other's way in DRAM; an odd count parts the neighbouring tiles that
 // share 256-byte lines.  n = 30, strided pass of one 512-thread CTA per SM: 152 CTAs 2.73 ms,
 // 148 2.68, 144 2.67, 136 2.68, 143 2.97; low pass: 304 CTAs 2.86 ms, 287 2.84, 272 2.82.
+// Not where every row of a tile lies on a page of its own (a1 >= kPageBits, n = 31): there a
+// CTA's own chain counts, 152 CTAs 18.5 ms a step, 144 18.9, 136 19.3.
 static long long dram_grid(long long full) { return full * 18 / 19 / 16 * 16; }
 
 template <int Q, int C>
@@ -723,6 +734,9 @@ static cudaError_t launch_sp_tma_c(const LaunchCtx& lc, float2* psi, int n, int 
   const long long ntiles = 1ll << (n - Q - C);
   auto kern = mode == 1 ? sp_tma_kernel<Q, C, 1>
                         : (mode == 2 ? sp_tma_kernel<Q, C, 2> : (mode == 3 ? sp_tma_kernel<Q, C, 3> : sp_tma_kernel<Q, C, 0>));
+  if constexpr (Q == 11) {
+    if (mode >= 2 && a2 >= kPageBits) kern = mode == 2 ? sp_tma_kernel<Q, C, 2, true> : sp_tma_kernel<Q, C, 3, true>;
+  }
   cudaError_t e = allow_smem(reinterpret_cast<const void*>(kern), G::smem);
   if (e != cudaSuccess) return e;
   int occ = 0;
@@ -730,7 +744,7 @@ static cudaError_t launch_sp_tma_c(const LaunchCtx& lc, float2* psi, int n, int 
   if (e != cudaSuccess) return e;
   if (occ < 1) occ = 1;
   long long grid = static_cast<long long>(occ) * lc.num_sms;
-  if (n >= 26 && mode >= 2 && Q == 10 && C == 4 && dram_grid(grid) > 0) grid = dram_grid(grid);
+  if (n >= 26 && mode >= 2 && Q == 10 && C == 4 && a1 < kPageBits && dram_grid(grid) > 0) grid = dram_grid(grid);
   if (grid > ntiles) grid = ntiles;
   return launch_overlapped(lc, kern, static_cast<unsigned>(grid), G::NT, G::smem, psi, map, n, a1, a2, brow, ntiles, err);
 }
