@@ -25,7 +25,8 @@
 //   and the polling of one load; with a grid barrier between stores and loads (a
 //   release, an atomic, an acquire and the loads in sequence) n = 16 took 3.10
 //   instead of 2.70 us per step.  The slots are used in turn (team_schedule.h): a warp
-//   of its own runs the fences that order a slot's emptying before its next word.
+//   of its own (with two CTAs per SM: thread 0) runs the fences that order a slot's
+//   emptying before its next word.
 //
 // Norm fold as in the streaming passes (NormFold), with the reference kept in the
 // handle's fold slot across launches of a range: the sum measured after a step
@@ -173,22 +174,24 @@ struct TeamGeom : CtaGeom<T, R> {
   // grid barrier: the words' second set of stores and registers cost more there
   // than the barrier (n = 21: 13.1 against 11.5 us per step)
   static constexpr bool kWords = !CLUSTER && G::NT < 512;
-  static constexpr int kThreads = G::NT + (kWords ? 32 : 0);
   static constexpr int kPerSm = C >= 8 ? 2 : 1;
-  // increments beside the values where there are registers for them (two CTAs per SM
-  // with a fence warp each leave 96 per thread)
-  static constexpr bool kInc = R < 5 && kPerSm == 1;
+  static constexpr bool kFenceWarp = kWords && kPerSm == 1;
+  static constexpr int kThreads = G::NT + (kFenceWarp ? 32 : 0);
+  // increments beside the values where there are registers for them; they go through
+  // the transposes too where the tile is the SM's only one (two: rounded at every window)
+  static constexpr bool kInc = R < 5;
+  static constexpr bool kCarry = kInc && kPerSm == 1;
   // What the rounding before the exchange leaves out stays in registers and is taken up
   // two steps on, when the amplitude is in the same layout, thread and register again.
   // Its turn in between is ignored: at angles that are not small it is one more error of
   // the size of the rounding.  The scales of the steps in between are not: they reach
   // 2^-n.
-  static constexpr bool kLeft = kInc && kPerSm == 1;
+  static constexpr bool kLeft = kCarry;
   // transpose buffers: two where they fit (one barrier per transpose instead of two);
   // the cluster's receive buffers lie behind them
-  static constexpr int kBufs = (kPerSm == 2 && kInc) || T > 13 ? 1 : 2;
+  static constexpr int kBufs = T > 13 ? 1 : 2;
   static_assert(!CLUSTER || kBufs == 2, "team_schedule.h");
-  static constexpr size_t kTile = (tile_bytes<T, R, kInc>() + 15u) / 16u * 16u;
+  static constexpr size_t kTile = (tile_bytes<T, R, kCarry>() + 15u) / 16u * 16u;
   static constexpr size_t kBytes = kTile * kBufs + (CLUSTER ? (kClusterBuffers - 2) * 8u * static_cast<size_t>(G::SLOTS) : 0u);
 };
 
@@ -226,7 +229,7 @@ __global__ void __launch_bounds__(TeamGeom<T, R, C, CLUSTER>::kThreads, (TeamGeo
   if constexpr (!CLUSTER) {
     if (tid == 0) s_late = 0;
     __syncthreads();
-    if (G::kWords && tid >= NT) {
+    if (G::kFenceWarp && tid >= NT) {
       // the fence warp: takes and kEmpty stores of step j come before any amplitude of
       // step j + kWordFenceLag leaves this CTA
       for (int j = 0; j < A.nsteps; ++j) {
@@ -347,46 +350,47 @@ __global__ void __launch_bounds__(TeamGeom<T, R, C, CLUSTER>::kThreads, (TeamGeo
       cp_async_wait<0>();
       team_sync<NT>();
       if (G::kWords) late = *static_cast<volatile int*>(&s_late) != 0;
+      if (G::kWords && !G::kFenceWarp && tid == 0) __threadfence();  // behind step j - 1
     };
     auto reuse = [&]() {
       if (G::kBufs == 1) team_sync<NT>();
     };
     if constexpr (!G::kSplit) {
       x.template turn<0, R>(c);
-      put_tile<T, R, kTop>(x, b0, tid);
+      put_tile<T, R, kTop, G::kCarry>(x, b0, tid);
       middle();
       if (G::kWords && late) {
-        bar_arrive<2, NT + 32>();  // the fence warp may be waiting for this step's
+        if (G::kFenceWarp) bar_arrive<2, NT + 32>();  // the fence warp may be waiting for this step's
         break;
       }
       if (pending && tid < 32) publish(j & 1, 0);
       fetch(j + kTeamRing - 1);
-      get_tile<T, R, kBot>(x, b0, tid);
+      get_tile<T, R, kBot, G::kCarry>(x, b0, tid);
       reuse();
-      x.template turn<0, R>(c);
-      put_tile<T, R, kBot>(x, b1, tid);
+      x.template turn<0, R>(c, !G::kCarry);
+      put_tile<T, R, kBot, G::kCarry>(x, b1, tid);
       team_sync<NT>();
-      get_tile<T, R, kMid>(x, b1, tid);
+      get_tile<T, R, kMid, G::kCarry>(x, b1, tid);
       reuse();
       x.template turn<0, T - 2 * R>(c);
     } else {
       x.template turn<0, T - 2 * R>(c);
-      put_tile<T, R, kMid>(x, b0, tid);
+      put_tile<T, R, kMid, G::kCarry>(x, b0, tid);
       middle();
       if (G::kWords && late) {
-        bar_arrive<2, NT + 32>();  // the fence warp may be waiting for this step's
+        if (G::kFenceWarp) bar_arrive<2, NT + 32>();  // the fence warp may be waiting for this step's
         break;
       }
       if (pending && tid < 32) publish(j & 1, 0);
       fetch(j + kTeamRing - 1);
-      get_tile<T, R, kBot>(x, b0, tid);
+      get_tile<T, R, kBot, G::kCarry>(x, b0, tid);
       reuse();
-      x.template turn<0, R>(c);
-      put_tile<T, R, kBot>(x, b1, tid);
+      x.template turn<0, R>(c, !G::kCarry);
+      put_tile<T, R, kBot, G::kCarry>(x, b1, tid);
       team_sync<NT>();
-      get_tile<T, R, kTop>(x, b1, tid);
+      get_tile<T, R, kTop, G::kCarry>(x, b1, tid);
       reuse();
-      x.template turn<0, R>(c);
+      x.template turn<0, R>(c, !G::kCarry);
     }
     // only the values leave: the one rounding of an amplitude per step
     if constexpr (!G::kLeft)
@@ -419,7 +423,7 @@ __global__ void __launch_bounds__(TeamGeom<T, R, C, CLUSTER>::kThreads, (TeamGeo
         float2* dst = xb + (static_cast<size_t>(l0 >> D) << T) + ((l0 & dm) | static_cast<int>(cta) << D);
         float2* src = xb + (static_cast<size_t>(cta) << T) + win_base<T, R, kTop>(tid);
         if constexpr (G::kWords) {
-          if (j >= kWordFenceLag) {  // the fence warp is done with step j - kWordFenceLag
+          if (G::kFenceWarp && j >= kWordFenceLag) {  // the fence warp is done with step j - kWordFenceLag
             static_assert(kWordFenceLag == 2, "one barrier per parity");
             if (j & 1) bar_sync<4, NT + 32>(); else bar_sync<3, NT + 32>();
           }
@@ -429,7 +433,7 @@ __global__ void __launch_bounds__(TeamGeom<T, R, C, CLUSTER>::kThreads, (TeamGeo
               word_store(dst + ((static_cast<size_t>((r * ls) >> D) << T) + ((r * ls) & dm)), f2_bits(v[r]));
           }
           if (!take_words<N>(v, src, win_step<T, R, kTop>(), A.polls)) s_late = 1;
-          bar_arrive<2, NT + 32>();
+          if (G::kFenceWarp) bar_arrive<2, NT + 32>();
         } else {
 #pragma unroll
           for (int r = 0; r < N; ++r) __stcg(dst + ((static_cast<size_t>((r * ls) >> D) << T) + ((r * ls) & dm)), v[r]);
@@ -457,11 +461,11 @@ __global__ void __launch_bounds__(TeamGeom<T, R, C, CLUSTER>::kThreads, (TeamGeo
     } else {
       x.template turn<0, R>(c, true);
       float2* b2 = buffer(b);
-      put_tile<T, R, kTop>(x, b2, tid);
+      put_tile<T, R, kTop, G::kCarry>(x, b2, tid);
       team_sync<NT>();
-      get_tile<T, R, kMid>(x, b2, tid);
+      get_tile<T, R, kMid, G::kCarry>(x, b2, tid);
       reuse();
-      x.template turn<D - R, T - 2 * R>(c);
+      x.template turn<D - R, T - 2 * R>(c, !G::kCarry);
       if (G::kBufs == 2) b ^= 1;
     }
     if (j & 1)
@@ -577,14 +581,19 @@ bool fits(int num_sms, int m) {
 //   n = 20 grid (12,4) with two CTAs per SM 6.36, (13,5) 6.65    n = 21 grid (14,5) 11.5
 // The kernels as they are, 400 steps, against the streaming passes (n = 12..14: the
 // earlier one-CTA kernel): n = 12 1.40 / 3.16, 13 1.88 / 4.85, 14 2.41 / 8.60, 15 2.30 /
-// 12.4, 16 3.04 / 12.4, 17 3.49 / 13.2, 18 3.71 / 14.6, 19 5.16 / 14.7, 20 6.58 / 18.8,
+// 12.4, 16 3.04 / 12.4, 17 3.49 / 13.2, 18 3.71 / 14.6, 19 5.16 / 14.7, 20 7.18 / 18.8,
 // 21 12.3 / 24.9; the state's error against 64 bits 2e-7 / 3.2e-6 (n = 16).
 // Without the increments in the transposes (an amplitude rounded at every window) n = 16
 // took 2.94, n = 19 4.44, with four times the error of <H_P> and of the ground
 // probability; with what a rounding leaves out packed into 4 bytes instead n = 16 3.51,
-// n = 19 5.08.  n = 20 and 21 have no registers for them (n = 20 so 9.1): every pair of
-// turns rounds, and the errors are about half of the streaming passes' (n = 20, 200
-// steps, rms of 8 instances: state 1.2e-6, <H_P> 9e-8, ground probability 3.9e-7).
+// n = 19 5.08.  n = 20 rounds at every window (9.1 with the increments in the transposes;
+// 8.5 with a fence warp, whose share leaves 96 registers; 6.6 without increments: a
+// rounding per pair of turns), 200 steps, rms of 24 instances: state 7.3e-7 (1.2e-6 without
+// increments, 2.5e-6 from the earlier passes), <H_P> 5.5e-8 (1.1e-7, 1.9e-7), ground
+// probability 2.3e-7 (4.3e-7, 6.1e-7).  n = 21 has no registers for increments: a
+// rounding per pair of turns, state 1.3e-6 (2.6e-6 from the earlier passes), <H_P> 1.1e-7
+// (1e-7), ground probability 3.1e-7 (2.9e-7), 400 steps 1.8e-6 (3.7e-6), 3.7e-7 (6.3e-7),
+// 2.1e-7 (2.1e-7).
 // n <= 11 stays with one CTA (0.94 at n = 11 against 1.07 in a cluster); 2^22
 // amplitudes do not fit in the registers.
 #define QAA_TEAMS(X)                                                                                       \

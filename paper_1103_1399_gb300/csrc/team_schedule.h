@@ -24,7 +24,9 @@ QAA_HD constexpr int cluster_receive(int j) { return 2 + (j & 1); }
 // kWordBuffers.  Behind the takes and emptyings of step j a warp of each CTA runs a
 // fence, and the CTA's stores of step j + kWordFenceLag wait for it.  The emptying is
 // before the next store if a fence of the receiver, words sent behind it and a fence of
-// the sender behind those words' arrival lie in between: twice the lag.
+// the sender behind those words' arrival lie in between: twice the lag.  (Two CTAs on an
+// SM have no room for a fence warp: thread 0 runs the fence between the transposes of step
+// j + 1, whose barriers put it before that step's stores: a lag of one.)
 constexpr int kWordBuffers = 4;
 constexpr int kWordFenceLag = 2;
 QAA_HD constexpr int word_buffer(int j) { return j % kWordBuffers; }

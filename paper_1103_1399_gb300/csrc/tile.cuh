@@ -151,15 +151,17 @@ template <int T, int R, bool INC>
 __host__ __device__ constexpr size_t tile_bytes() {
   return (INC ? 16u : 8u) * static_cast<size_t>(CtaGeom<T, R>::SLOTS);
 }
-template <int T, int R, int W, bool INC>
-__device__ __forceinline__ void put_tile(const Tile<1 << R, INC>& x, float2* buf, int tid) {
+template <int T, int R, int W, bool CARRY = true, bool INC>
+__device__ __forceinline__ void put_tile(Tile<1 << R, INC>& x, float2* buf, int tid) {
+  if (!CARRY) x.settle();
   put<T, R, W>(x.v, buf, tid);
-  if constexpr (INC) put<T, R, W>(x.d, buf + CtaGeom<T, R>::SLOTS, tid);
+  if constexpr (INC && CARRY) put<T, R, W>(x.d, buf + CtaGeom<T, R>::SLOTS, tid);
 }
-template <int T, int R, int W, bool INC>
+template <int T, int R, int W, bool CARRY = true, bool INC>
 __device__ __forceinline__ void get_tile(Tile<1 << R, INC>& x, const float2* buf, int tid) {
   get<T, R, W>(x.v, buf, tid);
-  if constexpr (INC) get<T, R, W>(x.d, buf + CtaGeom<T, R>::SLOTS, tid);
+  if (!CARRY) x.zero();
+  if constexpr (INC && CARRY) get<T, R, W>(x.d, buf + CtaGeom<T, R>::SLOTS, tid);
 }
 
 }  // namespace qaa

@@ -8,7 +8,8 @@
 // arrival of sent words (a wait orders the waiting CTA behind the threads that sent to
 // it, no others).
 //
-// Word form: the same two CTAs, each with a third thread that runs the fences.  Between
+// Word form: the same two CTAs, the fences run by a third thread of each or by the first
+// one.  Between
 // CTAs only a fence before the sent words and a fence behind their arrival order
 // anything: the arrival itself is a relaxed load.
 // Prints "ok" and exits 0, else prints the first violation and exits 1.
@@ -114,15 +115,22 @@ int cluster() {
   return g.check("cluster");
 }
 
-int words() {
+// A fence warp of its own (the stores of step j + kWordFenceLag wait for the fence behind
+// step j), or thread 0 between the transposes of step j + 1.
+int words(bool warp) {
   Graph g;
+  const int lag = warp ? qaa::kWordFenceLag : 1;
   int fence[2][kSteps], leave[2][kSteps];  // the fence warp's fence and its release of step j
   int sent[2][2];                          // [receiver][sender], this step's
   for (int j = 0; j < kSteps; ++j) {
     g.barrier(j, 2);  // of the transposes
-    if (j >= qaa::kWordFenceLag)
+    if (!warp && j > 0) {
+      for (int c = 0; c < 2; ++c) fence[c][j - 1] = g.add({c, 0, j, "fence", c, -1, false});
+      g.barrier(j, 2);
+    }
+    if (warp && j >= lag)
       for (int c = 0; c < 2; ++c)
-        for (int t = 0; t < 2; ++t) g.next[leave[c][j - qaa::kWordFenceLag]].push_back(g.add({c, t, j, "await fence", c, -1, false}));
+        for (int t = 0; t < 2; ++t) g.next[leave[c][j - lag]].push_back(g.add({c, t, j, "await fence", c, -1, false}));
     // slot of a buffer: by sender; thread s of the receiver takes the words of CTA s
     auto slot = [&](int sender) { return 2 * qaa::word_buffer(j) + sender; };
     for (int c = 0; c < 2; ++c)
@@ -130,24 +138,24 @@ int words() {
     for (int c = 0; c < 2; ++c)
       for (int t = 0; t < 2; ++t) g.own.push_back({sent[c][t], g.add({c, t, j, "take and empty", c, slot(t), true})});
     // the threads arrive, the fence warp waits for them
-    for (int c = 0; c < 2; ++c) {
+    for (int c = 0; warp && c < 2; ++c) {
       const int a0 = g.add({c, 0, j, "arrive", c, -1, false}), a1 = g.add({c, 1, j, "arrive", c, -1, false});
       fence[c][j] = g.add({c, 2, j, "fence", c, -1, false});
       g.next[a0].push_back(fence[c][j]);
       g.next[a1].push_back(fence[c][j]);
     }
-    for (int c = 0; c < 2; ++c) leave[c][j] = g.add({c, 2, j, "release", c, -1, false});
+    for (int c = 0; warp && c < 2; ++c) leave[c][j] = g.add({c, 2, j, "release", c, -1, false});
   }
   // a fence of the sender before a word it sends, and a fence of the receiver behind it
   for (int r = 0; r < 2; ++r)
-    for (int j = qaa::kWordFenceLag; j < kSteps; ++j) g.next[fence[1 - r][j - qaa::kWordFenceLag]].push_back(fence[r][j]);
-  return g.check("words");
+    for (int j = lag; j < kSteps - 1; ++j) g.next[fence[1 - r][j - lag]].push_back(fence[r][j]);
+  return g.check(warp ? "words, fence warp" : "words, thread 0's fence");
 }
 
 }  // namespace
 
 int main() {
-  if (cluster() || words()) return 1;
+  if (cluster() || words(true) || words(false)) return 1;
   std::puts("ok");
   return 0;
 }
