@@ -97,8 +97,9 @@ qaa_status qaa_set_stream(qaa_handle h, void* cuda_stream);
 
 /*
  * qaa_set_variant -- choose the Walsh-Hadamard implementation of the
- * streaming passes (n >= 15; the on-chip path for n <= 14 is always FP32).  A call with an explicit
- * variant runs the passes also where the default is a team of CTAs (15 <= n <= 21).
+ * streaming passes (n >= 15; the on-chip path for n <= 14 is always FP32).
+ * After it the handle runs the passes, also where the default is a team of
+ * CTAs (15 <= n <= 21), until qaa_autotune chooses for it again.
  *   wht_kind 0: FP32 CUDA-core butterflies, the whole-register W.B.W form.
  *            1: the W.B.W form with every transform on the tensor cores
  *               (tcgen05): each group of <= 10 qubits in two 5-qubit stages,
@@ -173,7 +174,12 @@ int qaa_tune_candidates(int n, char* buf, size_t len);
  *   evals    host array of k doubles: the lowest levels found, ascending;
  *            *found = how many (<= k).
  * FP64 real vectors (three arrays of 2^n doubles, allocated by the handle on
- * first use; QAA_E_NOMEM if they do not fit), FP64 recurrence scalars and host
+ * first use; QAA_E_NOMEM if they do not fit); from n = 18 on the neighbour sums of
+ * H_B are exact sums of 64-bit fixed-point numbers, 59 bits below the largest
+ * exponent of each tile of 2^11 or 2^12 amplitudes, so H v carries the same error
+ * relative to |v| (about 1e-15) as FP64 sums do, but an amplitude 2^-k below its
+ * tile's largest enters with 59 - k bits and one below 2^-59 not at all.  FP64
+ * recurrence scalars and host
  * tridiagonal eigenvalues (Sturm bisection); repeated and spurious Ritz values
  * of finite-precision Lanczos are removed by the Cullum-Willoughby test
  * (levels closer than 1e-9 ||T|| count as one).
@@ -442,7 +448,8 @@ typedef enum {
   QAA_K_OBSERVE = 7,       /* observable reductions (all kernels of a call) */
   QAA_K_DIAG = 8,          /* E(x) export                                   */
   QAA_K_INIT = 9,          /* uniform-state initialisation                  */
-  QAA_K_GRAPH = 10,        /* one launch-graph evolve (all its passes)      */
+  QAA_K_GRAPH = 10,        /* one evolve in launch-graph mode, n >= 15: its
+                              graph, or the team's launches where no graph is built */
   QAA_K_COUNT = 11
 } qaa_kernel_kind;
 

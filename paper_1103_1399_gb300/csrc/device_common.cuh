@@ -607,8 +607,9 @@ __device__ __forceinline__ float fold_factor_block(const NormFold& f) {
 // The scale the turns of the steps so far still owe, as R = prod (1 + r) - 1, and
 // the norm fold.  Both are applied together, every fold_period steps and after the
 // last of a launch (so that the result carries no drift of the steps since the
-// last fold: up to 8e-7 with most of the weight in one amplitude): multiplying by 1 + r in every step (r ~ -1e-7 towards the end of a
-// sweep) would round an amplitude that hardly changes the same way every time.
+// last fold: up to 8e-7 with most of the weight in one amplitude): multiplying by
+// 1 + r in every step (r ~ -1e-7 towards the end of a sweep) would round an amplitude
+// that hardly changes the same way every time.
 struct TurnScale {
   float R = 0.f;
   __device__ __forceinline__ void step(float r) { R = fmaf(R, r, R + r); }

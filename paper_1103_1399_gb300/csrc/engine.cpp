@@ -657,8 +657,10 @@ qaa_status qaa_autotune(qaa_handle h, void* psi, int steps, double budget_ms, ch
     qaa::make_plan(h->n, h->plan);
     return finish(fail(QAA_E_CUDA, "autotune: no candidate plan ran"));
   }
+  // the later stages vary the passes of the best plan: not where it is a team
+  auto passes_on_tma = [&] { return best.use_tma && (tc_kind || !best.team); };
   // stage 2: run length of each group that has a choice (Q >= 7 on TMA passes)
-  if (best.use_tma && !(best.team && !tc_kind))
+  if (passes_on_tma())
     for (size_t i = 0; i < best.strided.size() && spent() <= budget_ms; ++i) {
       if (best.strided[i].q < 7) continue;
       qaa::PassPlan c = best;
@@ -666,7 +668,7 @@ qaa_status qaa_autotune(qaa_handle h, void* psi, int steps, double budget_ms, ch
       consider(c);
     }
   // stage 3: two equal q-bit groups (q >= 10) recombined as {10..14, 15+q..} and {15..14+q}, or back
-  if (best.use_tma && !(best.team && !tc_kind) && best.strided.size() == 2 && best.strided[0].q == best.strided[1].q && best.strided[0].q >= 10 &&
+  if (passes_on_tma() && best.strided.size() == 2 && best.strided[0].q == best.strided[1].q && best.strided[0].q >= 10 &&
       spent() <= budget_ms) {
     qaa::PassPlan c = best;
     const int q = c.strided[0].q, L = c.low_bits;
@@ -683,7 +685,7 @@ qaa_status qaa_autotune(qaa_handle h, void* psi, int steps, double budget_ms, ch
   // stage 4: plain loads instead of TMA (groups of at most 10 bits, contiguous)
   bool narrow = true;
   for (const auto& g : best.strided) narrow = narrow && g.q <= 10;
-  if (best.use_tma && !(best.team && !tc_kind) && narrow && best.low_bits == qaa::kLowBits && spent() <= budget_ms) {
+  if (passes_on_tma() && narrow && best.low_bits == qaa::kLowBits && spent() <= budget_ms) {
     qaa::PassPlan c = best;
     c.use_tma = false;
     c.wht_kind = 0;  // plain loads: the W.B.W form only
@@ -696,7 +698,7 @@ qaa_status qaa_autotune(qaa_handle h, void* psi, int steps, double budget_ms, ch
   }
   // stage 5: the rotation form of the H_B factor on the best plan (same step,
   // g instead of 2g - 2 round trips; FP32 CUDA-core passes only)
-  if (!tc_kind && best.use_tma && !(best.team && !tc_kind) && spent() <= budget_ms) {
+  if (!tc_kind && passes_on_tma() && spent() <= budget_ms) {
     qaa::PassPlan c = best;
     c.wht_kind = qaa::kRotationForm;
     consider(c);

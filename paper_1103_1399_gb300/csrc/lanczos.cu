@@ -18,7 +18,10 @@
 // kTileMinBits on the sum is taken in 64-bit integers instead, tile by tile: the
 // tile's values as fixed-point numbers with 59 bits below the tile's largest
 // exponent (rounding 2^-60 of the tile's largest value; an FP64 sum rounds each
-// amplitude to 2^-53 of itself), added exactly, converted back once.  A tile of
+// amplitude to 2^-53 of itself), added exactly, converted back once.  |error of H u| /
+// |u| against extended precision, FP64 sums / this: ground state at s = 0.2 1.0e-15 /
+// 0.9e-15, at s = 0.5 4.8e-16 / 3.0e-16, a Krylov residual at s = 0.2 1.0e-15 / 1.1e-15, random
+// 8.2e-16 / 8.1e-16 (n = 18..20; amplitudes over up to 2^80).  A tile of
 // 2^TB values in shared memory serves the TB bits it spans: a low pass for bits
 // [0, TB) and strided passes of up to TB - 3 bits (64-byte runs) above, whose sums go
 // through y.

@@ -417,7 +417,7 @@ std::string describe_plan(const PassPlan& plan) {
       d += " R " + std::to_string(tma_run_bytes(g.q, plan.run_c[i])) + "B runs";
     }
     d += "; " + std::to_string(ng + 1) + " HBM round trips per step";
-    return team_plan(plan) ? d + "; none by default: the state in the registers of a team of CTAs" : d;
+    return team_plan(plan) ? d + "; run instead, where it fits, by a team of CTAs: the state in their registers, one exchange per step" : d;
   }
   const char* wk = plan.wht_kind == 1 ? "tensor-core BF16x3" : (plan.wht_kind == 2 ? "tensor-core BF16x2" : "FP32");
   std::string d = "streaming, " + std::string(plan.wht_kind ? "plain" : (plan.use_tma ? "TMA" : "classic")) +

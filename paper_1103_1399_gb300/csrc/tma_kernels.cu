@@ -309,10 +309,11 @@ __global__ void __launch_bounds__(TmaGeom<Q, C>::NT, (TmaGeom<Q, C>::NT >= 512 ?
 }
 
 // ----------------------------------------------------------- low pass -------
-// One 1024-amplitude tile per warp at a time, one buffer per warp: the TMA
-// engine writes the tile dense, the warp reads it into registers (layout X),
-// reuses the buffer for its two padded transposes, then asks for its next tile
-// and folds and counts that tile's clauses while the copy is in flight.
+// One 1024-amplitude tile per warp at a time: the bulk copy writes the tile dense, the
+// warp reads it into registers (layout X), transposes twice through a padded buffer
+// and asks for its next tile.  One buffer serves both, or the tiles land in a buffer of
+// their own (SPLIT == 1).  Where the counts are not stored, the next tile's clauses are
+// folded and counted while its copy is in flight.
 constexpr int kLpRowT = 33;
 constexpr int kLpSlotsT = 32 * kLpRowT;
 constexpr int kLpTmaWarps = 8;
