@@ -44,10 +44,10 @@ FALLBACK_HBM_GBS = 6800.0
 # the capture; a mismatch (kernel changed since) reports traffic = null.
 TRAFFIC = {
     # ncu full-set capture of sp_tma_kernel<10,4,2> (the default rotation form's
-    # strided pass, 128-byte runs) on the 28-qubit instance with
-    # QAA_GROUP_BITS=10,8: DRAM bytes read + written per launch for 2^28
-    # amplitudes, scaled by the amplitude count (x4) to one 30-qubit launch.
-    "strided": {"bytes_per_launch": 4 * (2.147551e9 + 2.086624e9), "src_sha": "5f1e3ea4bd430d04"},
+    # strided pass, 128-byte runs) on the 28-qubit instance: DRAM bytes read +
+    # written per launch for 2^28 amplitudes, scaled by the amplitude count (x4)
+    # to one 30-qubit launch.
+    "strided": {"bytes_per_launch": 4 * (2.150295e9 + 2.086470e9), "src_sha": "48365e88807ed2c4"},
 }
 
 

@@ -270,7 +270,7 @@ void make_default_plan(int n, PassPlan& plan, int max_q, int low, bool rotation)
   // Rotation form, n = 26..29: a 10-bit group {L..L+4} + the top 5 bits (128-byte runs,
   // 128 rows' pages per tile) and the 6 to 9 bits between, instead of two groups of 8 or
   // 9: a 10-bit pass with its early copy moves 6.4 TB/s, a 9-bit one 5.5 (per step, n = 27
-  // 1137 -> 1081 us, n = 28 2321 -> 2170, n = 29 4626 -> 4539, n = 26 556 -> 549).
+  // 1136 -> 1072 us, n = 28 2331 -> 2160, n = 29 4565 -> 4461, n = 26 547 -> 539).
   if (split && rotation && sizes_default && L == kLowBits && n >= 26 && n <= 29 && plan.strided.size() == 2) {
     plan.strided[0] = {L, 10, n - 5};
     plan.strided[1] = {L + 5, n - 5 - (L + 5), L + 10};
