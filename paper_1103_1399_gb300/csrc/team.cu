@@ -39,9 +39,11 @@ namespace qaa {
 namespace {
 
 constexpr int kTeamRing = 3;  // phase rows in flight: this step's and two ahead
-// Polls of a wait before it gives up, by default and with an injected fault.  The cluster
-// form must not give up while words sent to it are in flight (its CTAs return after
-// giving up): even the smaller limit takes hundreds of times a word's flight.
+// Polls of a wait before it gives up, by default (half a second in the grid forms, eight
+// in the cluster form, whose polls sleep) and with an injected fault (1 ms, 15 ms).  The
+// cluster form must not give up while words sent to it are in flight, because its
+// CTAs return after giving up: the smaller limit, too, is thousands of times a word's
+// flight.
 constexpr int kTeamPolls = 1 << 21, kTeamPollsInjected = 1 << 12;
 
 struct TeamArgs {
